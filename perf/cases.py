@@ -212,3 +212,107 @@ def tolerance(case):
     if case["kind"] == "wire":
         return "exact"
     return {"rel": 5e-7, "max": 1.5e-6}
+
+
+def _softmax(logits, T):
+    """Rows [R, V] at their temperatures [R], in 64 bits."""
+    return torch.softmax(logits.double() / T.double()[:, None], dim=1)
+
+
+def _row_blocks(R, V):
+    n = max(1, (1 << 26) // V)
+    return [(i, min(R, i + n)) for i in range(0, R, n)]
+
+
+def _pick(weight, u):
+    """First entry at which the running sum of each row's weights exceeds u times its total."""
+    run = weight.cumsum(1)
+    return (run <= u.double()[:, None] * run[:, -1:]).sum(1).clamp_(max=weight.shape[1] - 1)
+
+
+def _exact_compress(logits, T, K, top_p, u):
+    """[R, V] rows: the K largest logits (ties: lower index first), the nucleus cut, the draw."""
+    R, V = logits.shape
+    n = min(K, V)
+    idx = torch.full((R, K), -1, dtype=torch.int64, device=logits.device)
+    prob = torch.zeros((R, K), dtype=torch.float64, device=logits.device)
+    count = torch.empty((R,), dtype=torch.int64, device=logits.device)
+    tok = torch.empty_like(count)
+    for a, b in _row_blocks(R, V):
+        p = _softmax(logits[a:b], T[a:b])
+        order = logits[a:b].sort(dim=1, descending=True, stable=True).indices[:, :n]
+        w = p.gather(1, order)
+        m = (w.cumsum(1) < top_p).sum(1).add_(1).clamp_(max=n) if top_p < 1.0 else torch.full_like(count[a:b], n)
+        live = torch.arange(n, device=w.device) < m[:, None]
+        q = torch.where(live, w, torch.zeros_like(w))
+        q /= q.sum(1, keepdim=True)
+        idx[a:b, :n] = torch.where(live, order, torch.full_like(order, -1))
+        prob[a:b, :n], count[a:b] = q, m
+        if u is not None:
+            tok[a:b] = order.gather(1, _pick(q, u[a:b])[:, None])[:, 0]
+    return idx, prob, count, tok
+
+
+def _exact_verify(st, idx, prob, tok):
+    """p(x), the residual mass and the accept test of every draft position."""
+    B, G, K = idx.shape
+    V = st["target"].shape[2]
+    logits = st["target"][:, :G].reshape(B * G, V)
+    T = st["temperature"].repeat_interleave(G)
+    idx, q, tok = idx.reshape(B * G, K), prob.reshape(B * G, K).double(), tok.reshape(B * G, 1)
+    px, mass = (torch.empty((B * G,), dtype=torch.float64, device=q.device) for _ in range(2))
+    for a, b in _row_blocks(B * G, V):
+        p = _softmax(logits[a:b], T[a:b])
+        px[a:b] = p.gather(1, tok[a:b].long())[:, 0]
+        at = idx[a:b].clamp(min=0).long()
+        mass[a:b] = p.scatter_add_(1, at, -q[a:b]).clamp_(min=0.0).sum(1)       # (an empty slot has q = 0)
+    qx = torch.where(idx == tok, q, torch.zeros_like(q)).sum(1)
+    accept = (qx <= 0) | (st["u_accept"].reshape(-1).double() < (px / qx).clamp(max=1.0))
+    return px.reshape(B, G), mass.reshape(B, G), accept.reshape(B, G)
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits from torch.  The drawn tokens of the two-level sampler and the
+    count of borderline tests are left out; the codec's bytes are no computed numbers."""
+    if case["kind"] == "wire":
+        return None
+    B, G, K = case["B"], case["G"], case["k"]
+    st = prepare(case, seed)
+    T = st["temperature"]
+    seq = torch.arange(B, device=T.device)
+    if case["kind"] == "step":
+        R = B * G
+        idx, prob, count, tok = _exact_compress(st["draft"].reshape(R, -1), T.repeat_interleave(G), K, case["top_p"],
+                                                st["u_draft"].reshape(-1))
+        # the rows are stored in 32 bits and verified as they are stored
+        px, mass, accept = _exact_verify(st, idx.reshape(B, G, K), prob.float().reshape(B, G, K), tok)
+        length = accept.long().cumprod(1).sum(1)
+        return {"sparse": [idx.reshape(B, G, K), prob.reshape(B, G, K), count.reshape(B, G), tok.reshape(B, G)],
+                "verdict": {"accept_len": length, "p_draft": px, "resid_mass": mass, "borderline_count": None, "token": None}}
+    if case["kind"] == "range":
+        idx, prob, count, tok = st["sparse"]
+        px, mass, accept = _exact_verify(st, idx, prob, tok)
+        gamma = st["gamma"].long()
+        at = torch.arange(G, device=T.device)
+        drafted = at < gamma[:, None]
+        length = (accept & drafted).long().cumprod(1).sum(1)
+        last = torch.zeros_like(length)         # first row after the window that decides the sequence
+        for r0, r1 in _windows(G):
+            last = torch.where((length >= r0) & (length < r1), torch.full_like(last, r1), last)
+        seen = drafted & (at < last[:, None])
+        return {"accept_len": length, "p_draft": px * seen, "resid_mass": mass * seen, "borderline_count": None,
+                "token": None, "state": torch.zeros_like(length)}
+    pos = st["pos"].long()
+    p = _softmax(st["target"][seq, pos], T)
+    if case["kind"] == "residual":
+        idx, prob = st["sparse"][0], st["sparse"][1]
+        row = pos.clamp(max=G - 1)
+        q = prob[seq, row].double() * (pos < G)[:, None]
+        return [None, p.scatter_add_(1, idx[seq, row].clamp(min=0).long(), -q).clamp_(min=0.0).sum(1)]
+    idx, _, count, _ = _exact_compress(st["target"][seq, pos], T, K, 1.0, None)
+    live = idx >= 0
+    top = torch.where(live, p.gather(1, idx.clamp(min=0)), torch.zeros(1, dtype=p.dtype, device=p.device))
+    sent = top.float().double()                 # the message carries 32 bits
+    own = _softmax(st["draft"][seq, pos], T).gather(1, idx.clamp(min=0))
+    left = torch.where(live, (sent - own).clamp(min=0.0), torch.zeros_like(own))
+    return {"top": [idx, top, count], "token": None, "mass": left.sum(1)}
