@@ -76,6 +76,14 @@ __device__ __forceinline__ u64 make_key(float l, int v) {
 __device__ __forceinline__ int key_index(u64 k) { return (int)(0xFFFFFFFFu - (uint32_t)k); }
 __device__ __forceinline__ float key_logit(u64 k) { return from_orderable((uint32_t)(k >> 32)); }
 
+// Exchange area of a group of 256 threads that finishes one row (a group of 32 exchanges by shuffles).
+struct RowShared {
+    int first[WARPS], draw_first[WARPS], draw_last[WARPS];   // one slot per warp and use
+    int flag;
+    double Wn;
+    double warp_tot[2][WARPS];
+};
+
 struct CompressShared {
     int hist[256];
     int count;
@@ -83,9 +91,7 @@ struct CompressShared {
     int nan;
     u64 prefix;
     int krem;
-    int n, first, last, flag;
-    double Wn;
-    double warp_tot[WARPS];
+    RowShared row;
     float wM[WARPS];
     double wS[WARPS];
 };
@@ -201,35 +207,61 @@ __device__ void bitonic_sort_desc(u64* keys, int n2) {
     workers_sync();
 }
 
-__device__ __forceinline__ void emit_invalid_row(const CompressArgs& a, int row) {
-    for (int j = threadIdx.x; j < a.k_max; j += THREADS) {
+// ---- one row, finished by a group of TPR threads: a warp (TPR = 32) or the 256 worker threads ----
+template <int TPR> __device__ __forceinline__ int group_tid() { return TPR == 32 ? (threadIdx.x & 31) : threadIdx.x; }
+template <int TPR> __device__ __forceinline__ void group_sync() {
+    if (TPR == 32) __syncwarp();
+    else workers_sync();
+}
+// Inclusive scan of one double per thread over the group; `slot` (0 / 1): which exchange row is used.
+template <int TPR> __device__ __forceinline__ double group_scan_incl(double x, RowShared* sh, int slot, double& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, x, d);
+        x += lane >= d ? y : 0.0;
+    }
+    if (TPR == 32) {
+        total = __shfl_sync(0xffffffffu, x, 31);
+        return x;
+    }
+    if (lane == 31) sh->warp_tot[slot][warp] = x;
+    workers_sync();
+    double base = 0.0, tot = 0.0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) {
+        const double t = sh->warp_tot[slot][w];
+        if (w < warp) base += t;
+        tot += t;
+    }
+    total = tot;
+    return x + base;
+}
+
+template <int TPR> __device__ __forceinline__ void emit_invalid_row(const CompressArgs& a, int row) {
+    const int tid = group_tid<TPR>();
+    for (int j = tid; j < a.k_max; j += TPR) {
         a.q_idx[(long long)row * a.k_max + j] = -1;
         a.q_prob[(long long)row * a.k_max + j] = 0.f;
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         a.q_count[row] = -1;
         if (a.draft_tok) a.draft_tok[row] = -1;
     }
 }
 
 // Top-p cut, renormalisation, emission and draft draw for one row whose k_eff best candidates
-// sit sorted in keys[0..k_eff).  Z is the row normaliser on the scale of Weight<PRECISE>
-// (ignored when top_p >= 1).  Returns (to thread 0, via sh.flag) whether the cut was too close
-// to call in the fast path.
-template <bool PRECISE, int E>
-__device__ void finish_row_ranks(const CompressArgs& a, int row, const u64* keys, int k_eff, float Tb, double Z,
-                           CompressShared& sh) {
-    const int tid = threadIdx.x;
+// sit sorted in keys[0..k_eff), by a group of TPR threads with E consecutive ranks each.  Z is the row
+// normaliser on the scale of Weight<PRECISE> (ignored when top_p >= 1).  A cut that the fast path
+// cannot call puts the row on the queue of the double-precision pass.  `sh`: not used by a warp.
+template <bool PRECISE, int E, int TPR>
+__device__ __forceinline__ void finish_row_ranks(const CompressArgs& a, int row, const u64* keys, int k_eff, float Tb,
+                                                 double Z, RowShared* sh) {
+    const int tid = group_tid<TPR>(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float mx = key_logit(keys[0]);
+    const float u = a.draft_tok ? a.u_draft[row] : 0.f;      // requested long before it is needed
     Weight<PRECISE> wt;
     wt.init(Tb, mx);
-    if (tid == 0) {
-        sh.first = 0x7fffffff;
-        sh.last = -1;
-        sh.flag = 0;
-        sh.n = k_eff;
-    }
-    // E consecutive ranks per thread
     double w[E], cum[E], loc = 0.0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -239,38 +271,54 @@ __device__ void finish_row_ranks(const CompressArgs& a, int row, const u64* keys
         cum[e] = loc;
     }
     double Wtot;
-    const double base = block_scan_incl(loc, sh.warp_tot, Wtot) - loc;   // syncs: sh.first is set
+    const double base = group_scan_incl<TPR>(loc, sh, 0, Wtot) - loc;
+    int n = k_eff;
     if (a.top_p < 1.0f) {
         const double thrZ = (double)a.top_p * Z;
         int mine = 0x7fffffff;
 #pragma unroll
         for (int e = E - 1; e >= 0; --e)
             if (tid * E + e < k_eff && base + cum[e] >= thrZ) mine = tid * E + e;
-        if (mine != 0x7fffffff) atomicMin(&sh.first, mine);
-        workers_sync();
-        const int jn = sh.first;   // rank of the entry that reaches top_p, if any
-        if (jn != 0x7fffffff && jn == mine) {
-            sh.n = jn + 1;
-            if (!PRECISE) {
-                const int e = jn - tid * E;
-                const double E = GUARD_Z * thrZ;
-                const double hi = base + cum[e] - thrZ;
-                const double lo = thrZ - (base + cum[e] - w[e]);
-                // reaching top_p one entry earlier or later changes n unless the cap hides it
-                if ((hi < E && jn + 1 < k_eff) || (lo <= E && jn > 0)) sh.flag = 1;
-            }
+        int jn = __reduce_min_sync(0xffffffffu, mine);      // rank of the entry that reaches top_p, if any
+        if (TPR != 32) {
+            if (lane == 0) sh->first[warp] = jn;
+            workers_sync();
+#pragma unroll
+            for (int x = 0; x < WARPS; ++x) jn = min(jn, sh->first[x]);
         }
-        if (!PRECISE && jn == 0x7fffffff && tid == 0) {
-            // never reached: n = k_eff either way, nothing to decide
-        }
-        workers_sync();
+        if (jn != 0x7fffffff) n = jn + 1;
     }
-    const int n = sh.n;
+    // the owner of the last rank kept knows the mass of the kept entries and whether the cut was close
+    double Wn = 0.0;
+    int flag = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e)
-        if (tid * E + e == n - 1) sh.Wn = base + cum[e];
-    workers_sync();
-    const double Wn = sh.Wn;
+        if (tid * E + e == n - 1) {
+            Wn = base + cum[e];
+            if (!PRECISE && a.top_p < 1.0f) {
+                const double thrZ = (double)a.top_p * Z;
+                const double G = GUARD_Z * thrZ;
+                const double hi = Wn - thrZ;
+                const double lo = thrZ - (Wn - w[e]);
+                // reaching top_p one entry earlier or later changes n unless the cap hides it; never
+                // reached (hi < 0): n = k_eff either way, nothing to decide
+                if (hi >= 0.0 && ((hi < G && n < k_eff) || (lo <= G && n > 1))) flag = 1;
+            }
+            if (TPR != 32) {
+                sh->Wn = Wn;
+                sh->flag = flag;
+            }
+        }
+    if (TPR == 32) {
+        const int owner = (n - 1) / E;
+        Wn = __shfl_sync(0xffffffffu, Wn, owner);
+        flag = __shfl_sync(0xffffffffu, flag, owner);
+    } else {
+        workers_sync();
+        Wn = sh->Wn;
+        flag = sh->flag;
+    }
+    const bool flagged = !PRECISE && flag;
     // stored probabilities, and their running sum for the draft draw
     float pf[E];
     double ploc = 0.0, pcum[E];
@@ -282,8 +330,7 @@ __device__ void finish_row_ranks(const CompressArgs& a, int row, const u64* keys
         ploc += (double)pf[e];
         pcum[e] = ploc;
     }
-    const bool flagged = !PRECISE && sh.flag;
-    long long o = (long long)row * a.k_max;
+    const long long o = (long long)row * a.k_max;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int j = tid * E + e;
@@ -295,29 +342,36 @@ __device__ void finish_row_ranks(const CompressArgs& a, int row, const u64* keys
             a.q_prob[o + j] = pf[e];
         }
     }
-    for (int j = THREADS * E + tid; j < a.k_max; j += THREADS) {   // slots beyond the ranks the threads hold
+    for (int j = TPR * E + tid; j < a.k_max; j += TPR) {   // slots beyond the ranks the threads hold
         a.q_idx[o + j] = -1;
         a.q_prob[o + j] = 0.f;
     }
     if (a.draft_tok) {
-        if (tid == 0) {
-            sh.first = 0x7fffffff;
-            sh.last = -1;
-        }
         double Ptot;
-        const double pbase = block_scan_incl(ploc, sh.warp_tot, Ptot) - ploc;
-        const double thr = (double)a.u_draft[row] * Ptot;
+        const double pbase = group_scan_incl<TPR>(ploc, sh, 1, Ptot) - ploc;
+        const double thr = (double)u * Ptot;
         int mine = 0x7fffffff, mylast = -1;
 #pragma unroll
         for (int e = E - 1; e >= 0; --e) {
             if (tid * E + e < n && pbase + pcum[e] > thr) mine = tid * E + e;
             if (pf[e] > 0.f && mylast < 0) mylast = tid * E + e;
         }
-        if (mine != 0x7fffffff) atomicMin(&sh.first, mine);
-        if (mylast >= 0) atomicMax(&sh.last, mylast);
-        workers_sync();
+        mine = __reduce_min_sync(0xffffffffu, mine);
+        mylast = __reduce_max_sync(0xffffffffu, mylast);
+        if (TPR != 32) {
+            if (lane == 0) {
+                sh->draw_first[warp] = mine;
+                sh->draw_last[warp] = mylast;
+            }
+            workers_sync();
+#pragma unroll
+            for (int x = 0; x < WARPS; ++x) {
+                mine = min(mine, sh->draw_first[x]);
+                mylast = max(mylast, sh->draw_last[x]);
+            }
+        }
         if (tid == 0) {
-            const int j = sh.first != 0x7fffffff ? sh.first : sh.last;
+            const int j = mine != 0x7fffffff ? mine : mylast;
             a.draft_tok[row] = j >= 0 ? key_index(keys[j]) : -1;
         }
     }
@@ -331,17 +385,17 @@ __device__ void finish_row_ranks(const CompressArgs& a, int row, const u64* keys
             atomicAdd(a.slow_rows, 1ull);
         }
     }
-    workers_sync();
+    group_sync<TPR>();
 }
 
 // (the ranks are spread over as many threads as there are: one per thread up to 256 candidates,
 // which shortens the serial part -- the exponentials and the running sums -- fourfold)
-template <bool PRECISE>
+template <bool PRECISE, int TPR>
 __device__ __forceinline__ void finish_row(const CompressArgs& a, int row, const u64* keys, int k_eff, float Tb, double Z,
-                                           CompressShared& sh) {
-    if (k_eff <= THREADS) finish_row_ranks<PRECISE, 1>(a, row, keys, k_eff, Tb, Z, sh);
-    else if (k_eff <= 2 * THREADS) finish_row_ranks<PRECISE, 2>(a, row, keys, k_eff, Tb, Z, sh);
-    else finish_row_ranks<PRECISE, 4>(a, row, keys, k_eff, Tb, Z, sh);
+                                           RowShared* sh) {
+    if (k_eff <= TPR) finish_row_ranks<PRECISE, 1, TPR>(a, row, keys, k_eff, Tb, Z, sh);
+    else if (k_eff <= 2 * TPR) finish_row_ranks<PRECISE, 2, TPR>(a, row, keys, k_eff, Tb, Z, sh);
+    else finish_row_ranks<PRECISE, 4, TPR>(a, row, keys, k_eff, Tb, Z, sh);
 }
 
 template <typename T, bool ALIGNED, bool STATS>
@@ -373,14 +427,14 @@ __global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
         const float Tb = a.temperature[b];
         workers_sync();
         if (!temp_ok(Tb)) {
-            emit_invalid_row(a, row);
+            emit_invalid_row<THREADS>(a, row);
             if (tid == 0) atomicOr(a.status, ST_TEMPERATURE);
             continue;
         }
         const float c32 = temp_scale(Tb);
         const long long srow = source_row(a, row);
         if (srow < 0) {
-            emit_invalid_row(a, row);
+            emit_invalid_row<THREADS>(a, row);
             if (tid == 0) atomicOr(a.status, ST_RANGE);
             continue;
         }
@@ -494,11 +548,11 @@ __global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
         const float top = key_logit(keep[0]);
         const bool bad = sh.nan || !(top > -CUDART_INF_F) || !(top < CUDART_INF_F) || (STATS && !(Z > 0.0));
         if (bad) {
-            emit_invalid_row(a, row);
+            emit_invalid_row<THREADS>(a, row);
             if (tid == 0) atomicOr(a.status, ST_LOGIT);
             continue;
         }
-        finish_row<false>(a, row, keep, k_eff, Tb, Z, sh);
+        finish_row<false, THREADS>(a, row, keep, k_eff, Tb, Z, &sh.row);
     }
 }
 
@@ -561,7 +615,7 @@ __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs 
             double Z = 0.0;
             for (int w = 0; w < WARPS; ++w) Z += sh.wS[w];
             workers_sync();
-            finish_row<true>(a, row, keep, k_eff, a.temperature[b], Z, sh);
+            finish_row<true, THREADS>(a, row, keep, k_eff, a.temperature[b], Z, &sh.row);
         }
         __syncthreads();
     }

@@ -32,9 +32,9 @@
 // the ties of the k-th, for 32-bit logits plus what shares its 16-bit code) go to a per-row scratch
 // area in global memory, with the bound itself.
 //
-// compress_finish_kernel (one CTA per row) trims them to k where that is cheap, sorts them with a
-// bitonic network held in registers and calls finish_row (top-p cut, renormalisation, emission,
-// draft draw).
+// compress_finish_kernel (a warp or a CTA per row) selects the k best of them and puts them in order
+// with a counting sort over the 16-bit logit codes, then calls finish_row (top-p cut,
+// renormalisation, emission, draft draw).
 #pragma once
 #include "compress_kernels.cuh"
 
@@ -225,10 +225,11 @@ __device__ __forceinline__ unsigned coord_code(int G) {
     }
     return (unsigned)(0x7FFF - ((0x7FFF - G) + CS_DEAD));
 }
-// bin of an orderable key at or above the first tile's bound (coordinate g0)
-__device__ __forceinline__ int hist_bin(unsigned okey, int g0) {
-    return min(bin_coord(okey >> 16) - g0, CS_BINS - 1);
+// bin of an orderable key at or above the bound whose coordinate is g0, the last of N bins open-ended
+template <int N> __device__ __forceinline__ int hist_bin_in(unsigned okey, int g0) {
+    return min(bin_coord(okey >> 16) - g0, N - 1);
 }
+__device__ __forceinline__ int hist_bin(unsigned okey, int g0) { return hist_bin_in<CS_BINS>(okey, g0); }
 __device__ __forceinline__ void hist_add(unsigned* hist, int bin) {
     atomicAdd(&hist[bin >> 1], (bin & 1) ? 0x10000u : 1u);
     atomicAdd(&hist[CS_BINS / 2 + (bin >> 5)], 1u);
@@ -671,135 +672,57 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
     }
 }
 
-// ---- block-wide sort in registers ----------------------------------------------------------------
-// Bitonic network (descending) over N = 256 * R keys, R per thread: element e = warp * 32R + r * 32
-// + lane sits in register r of that lane.  Strides below 32 are warp shuffles, strides 32 .. 16R
-// are compare-exchanges between two registers of one thread, and only the three largest strides
-// of a merge cross warps: those go through shared memory (two buffers in turn, one barrier per
-// stage).  Keys are unsigned and larger = earlier; equal keys are interchangeable.
-__device__ __forceinline__ uint32_t shfl_xor_key(uint32_t k, int d) { return __shfl_xor_sync(0xffffffffu, k, d); }
-__device__ __forceinline__ u64 shfl_xor_key(u64 k, int d) {
-    const uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)k, d);
-    const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(k >> 32), d);
-    return ((u64)hi << 32) | lo;
-}
-template <typename K> __device__ __forceinline__ K key_pick(K mine, K other, bool keep_max) {
-    const K hi = mine > other ? mine : other, lo = mine > other ? other : mine;
-    return keep_max ? hi : lo;
-}
-
-template <typename K, int R>
-__device__ __forceinline__ void block_sort_desc(K (&key)[R], K* buf) {
-    constexpr int N = THREADS * R;
-    const int lane = threadIdx.x & 31;
-    const int ebase = (threadIdx.x >> 5) * (32 * R) + lane;
-    int phase = 0;
-#pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride >= 32 * R) {
-                K* bp = buf + (phase & 1) * N;
-                ++phase;
-#pragma unroll
-                for (int r = 0; r < R; ++r) bp[ebase + 32 * r] = key[r];
-                __syncthreads();
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int e = ebase + 32 * r;
-                    key[r] = key_pick(key[r], bp[e ^ stride], ((e & size) == 0) == ((e & stride) == 0));
-                }
-            } else if (stride >= 32) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int dr = stride >> 5;
-                    if ((r & dr) == 0) {
-                        const bool desc = ((ebase + 32 * r) & size) == 0;
-                        const K x = key[r], y = key[r + dr];
-                        const K hi = x > y ? x : y, lo = x > y ? y : x;
-                        key[r] = desc ? hi : lo;
-                        key[r + dr] = desc ? lo : hi;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int e = ebase + 32 * r;
-                    key[r] = key_pick(key[r], shfl_xor_key(key[r], stride), ((e & size) == 0) == ((lane & stride) == 0));
-                }
-            }
-        }
-    }
-}
-
-// Sort `count` keys held in shared memory at in[0 .. count) (the rest of the 256R-element network
-// is padding) into out[0 .. 256R), as 64-bit keys, largest first.  `in` may be either exchange
-// buffer; out is the first.  NARROW: 16-bit logits whose codes lie in [lo16, lo16 + 2^14) and
-// V <= 2^18 run the network on 32-bit keys, (code - lo16) << 18 | index complement.
-template <int R, bool NARROW>
-__device__ __noinline__ void sort_keys(const u64* in, int count, u64* out, unsigned lo16) {
-    const int lane = threadIdx.x & 31;
-    const int ebase = (threadIdx.x >> 5) * (32 * R) + lane;
-    u64 k[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int e = ebase + 32 * r;
-        k[r] = e < count ? in[e] : 0ull;
-    }
-    __syncthreads();                // every key is in registers: the buffers are free
-    if (NARROW) {
-        uint32_t n[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            n[r] = ebase + 32 * r < count ? ((((uint32_t)(k[r] >> 48) - lo16) << 18) | ((uint32_t)k[r] & 0x3FFFFu)) : 0u;
-        block_sort_desc<uint32_t, R>(n, reinterpret_cast<uint32_t*>(out));
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const uint32_t o16 = (n[r] >> 18) + lo16;
-            // a 16-bit logit's orderable form ends in sixteen ones when the logit is negative
-            const uint32_t o32 = (o16 << 16) | ((o16 & 0x8000u) ? 0u : 0xFFFFu);
-            out[ebase + 32 * r] = ((u64)o32 << 32) | (u64)(0xFFFC0000u | (n[r] & 0x3FFFFu));
-        }
-    } else {
-        block_sort_desc<u64, R>(k, out);
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < R; ++r) out[ebase + 32 * r] = k[r];
-    }
-    __syncthreads();
-}
-
-constexpr int CS_TIE_CAP = 256;     // boundary-group size up to which the survivors are trimmed to k
+// ---- finish: select, order, cut, emit ---------------------------------------------------------
 constexpr int CS_MAX_PIECES = 8;    // most pieces a row is dealt in
+// A group of TPR threads finishes a row: the CTA's 256 threads, or a warp (four rows per CTA).
+//   CAP     keys at or above the boundary bin the group can hold (more: the direct kernel)
+//   KCAP    largest k_eff
+//   BINS    bins of the counting sort: one per 16-bit logit code (bin_coord), counted up from the row's
+//           bound, i.e. BINS / 128 binades for values away from zero; the last one is open-ended
+template <int TPR> struct FinishGeom;
+template <> struct FinishGeom<32> {
+    static constexpr int ROWS = 4, CAP = 512, KCAP = 128, BINS = 512, AHEAD = 4, CTAS = 7;
+};
+template <> struct FinishGeom<THREADS> {
+    static constexpr int ROWS = 1, CAP = 2 * MAX_K, KCAP = MAX_K, BINS = 2048, AHEAD = 2, CTAS = 6;
+};
+template <int TPR> constexpr int finish_smem_bytes() {
+    return FinishGeom<TPR>::ROWS * (FinishGeom<TPR>::CAP * 8 + FinishGeom<TPR>::KCAP * 8 + FinishGeom<TPR>::BINS * 4);
+}
 
 struct CsFinishShared {
-    unsigned hi16;      // largest 16-bit logit code among the survivors
-    int kept, ties;     // slot counters: survivors above the bound's code / with it
-    int overflow;       // more survivors than the exchange buffers hold
-    int found;          // multi-piece rows: bin of the k-th largest code among all pieces' survivors
-    int piece_id[CS_MAX_PIECES];
-    int piece_count[CS_MAX_PIECES];
+    RowShared row;
+    int scan[WARPS];    // bin counts per warp
+    int kth;            // bin that holds the row's k-th largest key
+    int overflow;       // more keys at or above that bin than the buffer holds
 };
 
-// One CTA per row: put the row's pieces together, trim the survivors to the k best where that is
-// cheap, sort, cut / renormalise / emit.  The survivors of a piece are all its elements at or above
-// its final bound, i.e. its k best plus whatever shares the bound's 16-bit code with the k-th (ties
-// of a 16-bit logit; values within 2^-7 relative of it for 32-bit logits).  The largest of the
-// pieces' bounds is a bound for the row.  A row in several pieces holds about k survivors per piece
-// above it: their 16-bit codes are counted in the filter kernel's two-level histogram first, which
-// gives the code of the row's k-th largest logit, and only survivors at or above that code go on.
-// When the survivors would need a larger sort network than k keys do, the members of the boundary
-// group (the lowest code) are ranked among themselves (all pairs) and only the best
-// k - (number above the group) are kept.
-template <typename T, bool STATS>
-__global__ void __launch_bounds__(THREADS, 6) compress_finish_kernel(CompressArgs a, FilterPlan plan, int n2cap) {
-    extern __shared__ u64 keys[];          // two exchange buffers of n2cap keys; the sorted keys end up in the first
-    __shared__ CompressShared sh;
-    __shared__ CsFinishShared fs;
-    __shared__ __align__(16) unsigned fhist[CS_HIST_WORDS];    // (kth_bin reads four super-bins at a time)
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int row = blockIdx.x;
+// A row's survivors lie in one scratch area, or in those of its pieces if it was dealt in pieces.  A
+// survivor set holds all of a piece's elements at or above its final bound, i.e. its k best plus
+// whatever shares the bound's 16-bit code with the k-th; the largest of the pieces' bounds is a bound
+// for the row.  The k best are found and put in order by a counting sort over the 16-bit codes: count
+// the keys per bin, sum from the top, move every key that is not below the bin of the k-th into its
+// bin's stretch, then place each by its rank among the keys of its own stretch (all pairs: a
+// stretch holds the ties of one code, a few keys).  Bound by latency for few rows (meta, survivors, six
+// short phases: about 9 K cycles) and by issue for many.  It replaces a trim and a bitonic network over
+// the survivors, which was 32 of 51 K cycles of a row with k = 1024: 172 -> 72 us for 4096 rows with
+// k = 1024, 22 -> 15.5 us for 1536 rows with k = 256, 41 -> 9.1 us for 4096 rows with k = 8 (a warp
+// each), 16.4 -> 7.0 us for 40 rows in eight pieces with k = 64 (the pieces' records are read by one
+// lane each instead of one after the other).
+template <typename T, bool STATS, int TPR>
+__global__ void __launch_bounds__(TPR * FinishGeom<TPR>::ROWS, FinishGeom<TPR>::CTAS)
+compress_finish_kernel(CompressArgs a, FilterPlan plan) {
+    typedef FinishGeom<TPR> Geom;
+    constexpr int AHEAD = Geom::AHEAD, PER = Geom::BINS / TPR;
+    extern __shared__ __align__(16) unsigned char fin_mem[];
+    __shared__ CsFinishShared shared[Geom::ROWS];
+    const int tid = group_tid<TPR>(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int group = TPR == 32 ? warp : 0;
+    const int row = blockIdx.x * Geom::ROWS + group;
+    CsFinishShared& fs = shared[group];
+    u64* stretch = reinterpret_cast<u64*>(fin_mem) + group * (Geom::CAP + Geom::KCAP);
+    u64* keys = stretch + Geom::CAP;
+    int* bins = reinterpret_cast<int*>(reinterpret_cast<u64*>(fin_mem) + Geom::ROWS * (Geom::CAP + Geom::KCAP)) + group * Geom::BINS;
     int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
     if (k_eff > a.k_max) k_eff = a.k_max;
     if (k_eff > a.V) k_eff = a.V;
@@ -809,173 +732,163 @@ __global__ void __launch_bounds__(THREADS, 6) compress_finish_kernel(CompressArg
     const bool split_row = row >= whole_rows;
     const int area0 = split_row ? plan.rows + (row - whole_rows) * plan.split : row;
     const int nareas = split_row ? plan.split : 1;
+    for (int x = tid; x < Geom::BINS / 4; x += TPR) reinterpret_cast<int4*>(bins)[x] = make_int4(0, 0, 0, 0);
+    if (tid == 0) fs.overflow = 0;
     grid_dependency_sync();
-    // the first piece's first 512 scratch slots exist for every k_max: requested before its count is known
-    const u64* src0 = a.surv_keys + (long long)area0 * surv_cap;
-    const u64 first0 = src0[tid], first1 = src0[tid + THREADS];
-    // ---- the pieces: flags, the row's bound ----------------------------------------------------------
-    int np = 0, flags = 0;
-    unsigned thr_key = 0u;
-    for (int j = 0; j < nareas; ++j) {
-        if (split_row && j > 0 && plan_piece_tile(plan, j + 1) <= plan_piece_tile(plan, j)) continue;   // an empty piece
-        const CsRowMeta meta = a.surv_meta[area0 + j];
-        flags |= meta.flags;
-        thr_key = max(thr_key, meta.thr_key);
-        if (np < CS_MAX_PIECES && tid == 0) {
-            fs.piece_id[np] = area0 + j;
-            fs.piece_count[np] = meta.count;
-        }
-        ++np;
-    }
-    if (np > CS_MAX_PIECES) flags |= CSF_REDO;
+    if (row >= plan.rows) return;       // (a warp beyond the last row)
+    const u64* src = a.surv_keys + (long long)area0 * surv_cap;
+    // the first area's first slots exist for every k_max: requested before their number is known
+    u64 ahead[AHEAD];
+#pragma unroll
+    for (int x = 0; x < AHEAD; ++x) ahead[x] = src[x * TPR + tid];
+    const float Tb = a.temperature[row / a.G];
+    // ---- the pieces, one per lane: flags, the row's bound, where each piece's survivors begin -------
+    CsRowMeta meta;
+    meta.count = 0; meta.flags = 0; meta.thr_key = 0u; meta.ref_off = 0.f; meta.z_stream = 0.0;
+    if (lane < nareas && (!split_row || lane == 0 || plan_piece_tile(plan, lane + 1) > plan_piece_tile(plan, lane)))
+        meta = a.surv_meta[area0 + lane];
+    __syncwarp();
+    const unsigned flags = __reduce_or_sync(0xffffffffu, (unsigned)meta.flags);
+    const unsigned thr_key = __reduce_max_sync(0xffffffffu, meta.thr_key);
     if (flags & (CSF_ABORT | CSF_TEMPERATURE | CSF_LOGIT | CSF_RANGE)) {
-        emit_invalid_row(a, row);
+        emit_invalid_row<TPR>(a, row);
         if (tid == 0 && !(flags & CSF_ABORT))
             atomicOr(a.status, (flags & CSF_TEMPERATURE) ? ST_TEMPERATURE : (flags & CSF_RANGE) ? ST_RANGE : ST_LOGIT);
         return;
     }
-    if (flags & CSF_REDO) {
-        // a piece's candidates did not fit: the direct kernel writes this row
-        if (tid == 0) {
-            a.redo_rows[atomicAdd(a.redo_count, 1)] = row;
-            atomicAdd(a.redo_total, 1ull);
-        }
-        return;
+    int begin[CS_MAX_PIECES], m = 0;        // begin[p]: flat number of piece p's first survivor
+#pragma unroll
+    for (int p = 0; p < CS_MAX_PIECES; ++p) {
+        begin[p] = m;
+        m += __shfl_sync(0xffffffffu, meta.count, p);
     }
-    const float Tb = a.temperature[row / a.G];
-    u64* bufA = keys;
-    u64* bufB = keys + n2cap;
-    if (tid == 0) {
-        fs.hi16 = 0u;
-        fs.kept = 0;
-        fs.ties = 0;
-        fs.overflow = 0;
-        fs.found = -1;
-    }
-    if (np > 1)
-        for (int x = tid; x < CS_HIST_WORDS; x += THREADS) fhist[x] = 0u;
-    __syncthreads();
-    if (np > 1) {
-        // ---- several pieces: the code of the row's k-th largest logit among all their survivors ------
+    bool redo = (flags & CSF_REDO) != 0;
+    if (!redo) {
         const int g0 = bin_coord(thr_key >> 16);
-        for (int p = 0; p < np; ++p) {
-            const u64* src = a.surv_keys + (long long)fs.piece_id[p] * surv_cap;
-            const int m = fs.piece_count[p];
-            for (int e = tid; e < m; e += THREADS) {
-                const unsigned okey = (unsigned)(src[e] >> 32);
-                if (okey >= thr_key) hist_add(fhist, hist_bin(okey, g0));
+        auto key_at = [&](int i) -> u64 {       // survivor i of the row (i < m)
+            if (nareas == 1) return src[i];
+            int p = 0, b = 0;
+#pragma unroll
+            for (int x = 1; x < CS_MAX_PIECES; ++x)
+                if (i >= begin[x]) {
+                    p = x;
+                    b = begin[x];
+                }
+            return src[(long long)p * surv_cap + (i - b)];
+        };
+        const int held = nareas == 1 ? AHEAD * TPR : 0;      // survivors the group holds in registers
+        group_sync<TPR>();      // the bins are zero
+        // ---- count ------------------------------------------------------------------------------
+        auto bin_of = [&](u64 key) { return hist_bin_in<Geom::BINS>((unsigned)(key >> 32), g0); };
+#pragma unroll
+        for (int x = 0; x < AHEAD; ++x)
+            if (nareas == 1 && x * TPR + tid < m && (unsigned)(ahead[x] >> 32) >= thr_key) atomicAdd(&bins[bin_of(ahead[x])], 1);
+#pragma unroll 4
+        for (int i = held + tid; i < m; i += TPR) {
+            const u64 key = key_at(i);
+            if ((unsigned)(key >> 32) >= thr_key) atomicAdd(&bins[bin_of(key)], 1);
+        }
+        group_sync<TPR>();
+        // ---- bins -> number of keys in higher bins (thread t owns PER bins, the highest first) ------
+        int cnt[PER], own = 0;
+        int4* mine = reinterpret_cast<int4*>(bins + Geom::BINS - (tid + 1) * PER);
+#pragma unroll
+        for (int x = 0; x < PER / 4; ++x) {
+            const int4 v = mine[x];
+            cnt[4 * x] = v.x; cnt[4 * x + 1] = v.y; cnt[4 * x + 2] = v.z; cnt[4 * x + 3] = v.w;
+            own += v.x + v.y + v.z + v.w;
+        }
+        int run = own;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, run, d);
+            run += lane >= d ? y : 0;
+        }
+        if (TPR != 32) {
+            if (lane == 31) fs.scan[warp] = run;
+            group_sync<TPR>();
+#pragma unroll
+            for (int w = 0; w < WARPS; ++w)
+                if (w < warp) run += fs.scan[w];
+        }
+        const int live = run;                                         // (the last thread has counted all of them)
+        const bool holds_kth = run - own < k_eff && run >= k_eff;     // one thread
+        run -= own;
+#pragma unroll
+        for (int x = PER - 1; x >= 0; --x) {
+            const int c = cnt[x];
+            cnt[x] = run;
+            run += c;
+        }
+        if (holds_kth) {
+            int x = PER - 1;        // the k-th lies in the lowest of the thread's bins with fewer than k_eff keys above it
+#pragma unroll
+            for (int y = PER - 2; y >= 0; --y)
+                if (cnt[y] < k_eff) x = y;
+            int end = run;          // keys down to and including bin x
+#pragma unroll
+            for (int y = 1; y < PER; ++y)
+                if (y == x) end = cnt[y - 1];
+            fs.kth = Geom::BINS - (tid + 1) * PER + x;
+            if (end > Geom::CAP) fs.overflow = 1;         // too many ties with the k-th
+        }
+        if (tid == TPR - 1 && live < k_eff) fs.overflow = 1;          // cannot happen with valid bounds; be safe
+#pragma unroll
+        for (int x = 0; x < PER / 4; ++x) mine[x] = make_int4(cnt[4 * x], cnt[4 * x + 1], cnt[4 * x + 2], cnt[4 * x + 3]);
+        group_sync<TPR>();
+        redo = fs.overflow != 0;
+        if (!redo) {
+            // ---- move: afterwards bins[b] is the end of bin b's stretch, which begins where bin b + 1's ends
+            const int kth = fs.kth;
+            auto move = [&](u64 key) {
+                if ((unsigned)(key >> 32) >= thr_key) {
+                    const int b = bin_of(key);
+                    if (b >= kth) stretch[atomicAdd(&bins[b], 1)] = key;
+                }
+            };
+#pragma unroll
+            for (int x = 0; x < AHEAD; ++x)
+                if (nareas == 1 && x * TPR + tid < m) move(ahead[x]);
+#pragma unroll 4
+            for (int i = held + tid; i < m; i += TPR) move(key_at(i));
+            group_sync<TPR>();
+            // ---- rank inside the stretch
+            const int total = bins[kth];
+            for (int i = tid; i < total; i += TPR) {
+                const u64 key = stretch[i];
+                const int b = bin_of(key);
+                const int s0 = b + 1 < Geom::BINS ? bins[b + 1] : 0, s1 = bins[b];
+                int rank = s0;
+                for (int x = s0; x < s1; ++x) rank += stretch[x] > key ? 1 : 0;
+                if (rank < k_eff) keys[rank] = key;         // keys are distinct: every rank is taken once
             }
+            group_sync<TPR>();
         }
-        __syncthreads();
-        if (warp == 0) {
-            const int found = kth_bin(fhist, k_eff, lane);
-            if (lane == 0) fs.found = found;
-        }
-        __syncthreads();
-        if (fs.found >= 0) thr_key = max(thr_key, coord_code(g0 + fs.found) << 16);
     }
-    const unsigned thr16 = thr_key >> 16;
-    // ---- survivors to shared memory: those above the bound's code to buffer A, the boundary group
-    // ---- to buffer B, both in arrival order (warp-aggregated slots)
-    {
-        const unsigned lt = (1u << lane) - 1u;
-        unsigned hi = 0u;
-        for (int p = 0; p < np; ++p) {
-            const u64* src = a.surv_keys + (long long)fs.piece_id[p] * surv_cap;
-            const int m = fs.piece_count[p];
-            for (int e0 = 0; e0 < m; e0 += THREADS) {
-                const int e = e0 + tid;
-                const u64 key = (p == 0 && e0 == 0) ? first0 : (p == 0 && e0 == THREADS) ? first1 : (e < m ? src[e] : 0ull);
-                const unsigned code = (unsigned)(key >> 48);
-                const bool live = e < m && (unsigned)(key >> 32) >= thr_key;
-                const bool is_above = live && code > thr16;
-                const bool is_tie = live && !is_above;
-                if (live) hi = max(hi, code);
-                const unsigned ma = __ballot_sync(0xffffffffu, is_above), mt = __ballot_sync(0xffffffffu, is_tie);
-                int ba = 0, bt = 0;
-                if (lane == 0) {
-                    if (ma) ba = atomicAdd(&fs.kept, __popc(ma));
-                    if (mt) bt = atomicAdd(&fs.ties, __popc(mt));
-                }
-                ba = __shfl_sync(0xffffffffu, ba, 0);
-                bt = __shfl_sync(0xffffffffu, bt, 0);
-                const int sa = ba + __popc(ma & lt), st = bt + __popc(mt & lt);
-                if (is_above) {
-                    if (sa < n2cap) bufA[sa] = key;
-                    else fs.overflow = 1;
-                }
-                if (is_tie) {
-                    if (st < n2cap) bufB[st] = key;
-                    else fs.overflow = 1;
-                }
-            }
-        }
-        hi = __reduce_max_sync(0xffffffffu, hi);
-        if (lane == 0) atomicMax(&fs.hi16, hi);
-    }
-    __syncthreads();
-    const int above = fs.kept, t = fs.ties, m = above + t;
-    if (fs.overflow || m > n2cap || m < k_eff) {
-        // more survivors than the buffers hold (a histogram window too coarse for this row): direct kernel
+    if (redo) {
+        // a piece's candidates did not fit, or too many ties: the direct kernel writes this row
         if (tid == 0) {
             a.redo_rows[atomicAdd(a.redo_count, 1)] = row;
             atomicAdd(a.redo_total, 1ull);
         }
         return;
-    }
-    const bool narrow = sizeof(T) == 2 && a.V <= (1 << 18) && fs.hi16 - thr16 < (1u << 14);
-    int nk = 256;                       // network size for k keys
-    while (nk < k_eff) nk <<= 1;
-    int nm = 256;                       // network size for all m survivors
-    while (nm < m) nm <<= 1;
-    int count = m, n2 = nm;
-    if (nm > nk && above < k_eff && t <= CS_TIE_CAP) {
-        // trim: of the boundary group only the best k - above, each placed by its rank in the group
-        const int need = k_eff - above;
-        for (int j = tid; j < t; j += THREADS) {
-            const u64 key = bufB[j];
-            int rank = 0;
-            for (int x = 0; x < t; ++x) rank += bufB[x] > key ? 1 : 0;
-            if (rank < need) bufA[above + rank] = key;      // keys are distinct: every rank is taken once
-        }
-        count = k_eff;
-        n2 = nk;
-    } else {
-        for (int j = tid; j < t; j += THREADS) bufA[above + j] = bufB[j];
-    }
-    __syncthreads();
-    const u64* in = bufA;
-    // the boundary group's ranks are written (or nothing was): sort `count` keys from `in`
-    // (sort_keys moves them to registers before either buffer is reused)
-    const int R = n2 >> 8;
-    if (narrow) {
-        if (R == 1) sort_keys<1, true>(in, count, bufA, thr16);
-        else if (R == 2) sort_keys<2, true>(in, count, bufA, thr16);
-        else if (R == 4) sort_keys<4, true>(in, count, bufA, thr16);
-        else sort_keys<8, true>(in, count, bufA, thr16);
-    } else {
-        if (R == 1) sort_keys<1, false>(in, count, bufA, 0u);
-        else if (R == 2) sort_keys<2, false>(in, count, bufA, 0u);
-        else if (R == 4) sort_keys<4, false>(in, count, bufA, 0u);
-        else sort_keys<8, false>(in, count, bufA, 0u);
     }
     const float top = key_logit(keys[0]);
     double Z = 0.0;
     if (STATS) {
         // move every piece's streamed sum from its reference onto the scale of the weights exp(l/T - top/T)
         const float c32 = temp_scale(Tb);
-        for (int p = 0; p < np; ++p) {
-            const CsRowMeta meta = a.surv_meta[fs.piece_id[p]];
-            Z += meta.z_stream * exp2((double)meta.ref_off - (double)top * (double)c32);
-        }
+        if (meta.count > 0) Z = meta.z_stream * exp2((double)meta.ref_off - (double)top * (double)c32);
+        __syncwarp();
+        Z = warp_sum(Z);
     }
     const bool bad = !(top > -CUDART_INF_F) || !(top < CUDART_INF_F) || (STATS && !(Z > 0.0));
     if (bad) {
-        emit_invalid_row(a, row);
+        emit_invalid_row<TPR>(a, row);
         if (tid == 0) atomicOr(a.status, ST_LOGIT);
         return;
     }
-    finish_row<false>(a, row, keys, k_eff, Tb, Z, sh);
+    finish_row<false, TPR>(a, row, keys, k_eff, Tb, Z, &fs.row);
 }
 
 }  // namespace picospec

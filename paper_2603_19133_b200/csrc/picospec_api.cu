@@ -162,6 +162,14 @@ void launch_compress_direct(const CompressArgs& a, int grid, bool stats, cudaStr
     else launch_chained(compress_kernel<T, ALIGNED, false>, grid, THREADS, COMPRESS_SMEM, s, a);
 }
 
+template <typename T, int TPR>
+void launch_compress_finish(const CompressArgs& a, const FilterPlan& plan, bool stats, cudaStream_t s) {
+    constexpr int ROWS = FinishGeom<TPR>::ROWS;
+    const int grid = (plan.rows + ROWS - 1) / ROWS;
+    if (stats) launch_chained(compress_finish_kernel<T, true, TPR>, grid, TPR * ROWS, finish_smem_bytes<TPR>(), s, a, plan);
+    else launch_chained(compress_finish_kernel<T, false, TPR>, grid, TPR * ROWS, finish_smem_bytes<TPR>(), s, a, plan);
+}
+
 template <typename T>
 cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool aligned, cudaStream_t s) {
     const int rows = a.B * a.G;
@@ -194,12 +202,13 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         cudaError_t e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;
         {
-            int n2 = 1;
-            while (n2 < cs_survivor_cap(a.k_max)) n2 <<= 1;
             ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_FINISH, 2, s);
-            // two exchange buffers of the sort network (the sorted keys end up in the first)
-            if (stats) launch_chained(compress_finish_kernel<T, true>, rows, THREADS, (size_t)n2 * 16, s, a, plan, n2);
-            else launch_chained(compress_finish_kernel<T, false>, rows, THREADS, (size_t)n2 * 16, s, a, plan, n2);
+            // A warp per row while the row that has most survivors has few of them: a row dealt in 8 pieces
+            // at k = 64 (560 survivors) took 15.9 us of a call by warps, 7.0 by CTAs; 4096 whole rows at
+            // k = 8 take 9.1 us by warps and took 41 with a CTA and a sort network each.
+            const int survivors = plan.rem > 0 ? k_eff * plan.split : k_eff;
+            if (survivors <= FinishGeom<32>::KCAP) launch_compress_finish<T, 32>(a, plan, stats, s);
+            else launch_compress_finish<T, THREADS>(a, plan, stats, s);
         }
         e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;
