@@ -1,5 +1,4 @@
-// Draft-side compression, staged variant: rows whose base, pitch and length are multiples of 16
-// bytes and that hold at least one full tile.  Two kernels.
+// Draft-side compression, staged variant: rows that hold at least one full tile.  Two kernels.
 //
 // compress_filter_kernel streams the rows (one CTA per row at a time, tiles of 8 chunks staged in
 // shared memory by bulk async copies; the producer lane runs ahead into the next row) and keeps
@@ -328,7 +327,7 @@ __device__ __noinline__ int maintain_region(int wcount, int region_off, int hist
 // reach, which is a valid bound for the row, and leaves its survivors in its own scratch area (whole
 // row r: area r; tail piece n: area rows + n).  The finish kernel puts the pieces of a row together.
 // No piece starts at a row's last tile when that tile is ragged (the first tile of a piece must be a
-// full one).
+// full one, up to the few entries that a row's offset from a 16-byte boundary takes from it).
 struct FilterPlan {
     int tiles_per_row;
     int ragged_last;        // the last tile of a row holds fewer than TILE_CHUNKS full chunks
@@ -460,8 +459,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         FilterPiece pc;
         for (int k = 0; plan_piece(plan, blockIdx.x, k, pc); ++k) {
             const long long srow = source_row(a, pc.row);
-            const bool valid = temp_ok(a.temperature[pc.row / a.G]) && srow >= 0;
-            const T* rowp = reinterpret_cast<const T*>(a.logits) + (srow < 0 ? 0 : srow) * a.row_stride;
+            // (a row with a bad temperature is copied for nothing: its workers look the temperature up)
+            const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (srow < 0 ? 0 : srow) * a.row_stride, a.V);
             for (int ti = pc.tile0; ti < pc.tile1; ++ti, ++i) {
                 const int s = (int)(i % STAGES);
                 const uint32_t round = i / STAGES;
@@ -470,15 +469,9 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     if (wr != WAIT_OK) atomicOr(a.status, ST_INTERNAL);
                     if (wr == WAIT_LOST) return;      // nothing more is issued
                 }
-                if (valid) {
-                    const int v0 = ti * TILE_CHUNKS * CHUNK;
-                    const int v1 = min(a.V, v0 + TILE_CHUNKS * CHUNK);
-                    const uint32_t bytes = (uint32_t)(v1 - v0) * (uint32_t)sizeof(T);
-                    mbar_arrive_expect_tx(&full[s], bytes);
-                    bulk_load(stage_mem + s * TILE_BYTES, rowp + v0, bytes, &full[s], pol);
-                } else {
-                    mbar_arrive(&full[s]);
-                }
+                constexpr int GRANULES = TILE_BYTES / 16;
+                if (srow >= 0) stage_tile<T>(stage_mem + s * TILE_BYTES, sr, ti * GRANULES, GRANULES, &full[s], pol);
+                mbar_arrive(&full[s]);
             }
         }
         return;
@@ -509,7 +502,11 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         parity ^= 1;
         const int row = pc.row;
         const float Tb = a.temperature[row / a.G];
-        const bool in_range = source_row(a, row) >= 0;
+        const long long srow = source_row(a, row);
+        const bool in_range = srow >= 0;
+        // chunks are counted from the row's first granule here: which 1024 entries make one is no matter
+        const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (in_range ? srow : 0) * a.row_stride, a.V);
+        const int mis = sr.mis, end = sr.end;
         const bool valid = temp_ok(Tb) && in_range;
         const float c32 = temp_scale(Tb);
         float ref_off = 0.f, acc = 0.f;
@@ -532,10 +529,10 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 }
             }
             const int c = ti * TILE_CHUNKS + warp;
-            const bool work = !dead && valid && !full_region && c < a.nch;
+            const bool work = !dead && valid && !full_region && c * CHUNK < end;
             const unsigned char* chunk = stage_mem + s * TILE_BYTES + warp * (CHUNK * (int)sizeof(T));
             ChunkRegs<T> regs;
-            if (work) load_staged(regs, chunk, c * CHUNK, a.V, lane);
+            if (work) load_staged(regs, chunk, c * CHUNK, end, lane);
             if (ti == pc.tile0 && valid) {
                 // first tile of a piece (every warp holds a full chunk): each warp's own bound, then the minimum
                 if (work) {
@@ -582,7 +579,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                             added = 0;
                         }
                     }
-                    const int vchunk = c * CHUNK;
+                    const int vchunk = c * CHUNK - mis;
                     // every lane appends its own passing values: its slots come from the warp's counter
                     if (mask) {
                         int pos = atomicAdd(&cta.wcnt[warp], n);

@@ -175,8 +175,9 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
     const int rows = a.B * a.G;
     const int grid = rows < ctx->num_sms * 2 ? rows : ctx->num_sms * 2;
     const bool stats = a.top_p < 1.0f || a.raw_probs;     // raw probabilities need the normaliser too
-    // staged kernel: 16-byte aligned rows of at least one full tile
-    const bool staged = aligned && ((size_t)a.V * sizeof(T)) % 16 == 0 && a.V >= TILE_CHUNKS * CHUNK;
+    // staged kernel: rows of at least one full tile, at any offset (96 rows of 50381 entries at odd offsets
+    // took 45.8 us in the direct kernel, which reads such rows element by element)
+    const bool staged = a.V >= TILE_CHUNKS * CHUNK;
     if (staged) {
         cudaError_t ea = ensure_kernel_attrs(ctx->device);
         if (ea != cudaSuccess) return ea;
@@ -193,8 +194,11 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         if (per_sm < 1) per_sm = 1;
         if (per_sm > FILTER_MAX_CTAS_PER_SM) per_sm = FILTER_MAX_CTAS_PER_SM;
         // whole rows first, the remainder in pieces so that every CTA streams about the same number of tiles
-        const FilterPlan plan = make_filter_plan(rows, (a.nch + TILE_CHUNKS - 1) / TILE_CHUNKS,
-                                                 a.V % (TILE_CHUNKS * CHUNK) != 0, (long long)ctx->num_sms * per_sm);
+        // (a row that does not start on a 16-byte boundary is staged with up to one granule more)
+        constexpr int TILE = TILE_CHUNKS * CHUNK;
+        const int longest = a.V + (aligned ? 0 : 16 / (int)sizeof(T) - 1);
+        const FilterPlan plan = make_filter_plan(rows, (longest + TILE - 1) / TILE, longest % TILE != 0 || !aligned,
+                                                 (long long)ctx->num_sms * per_sm);
         {
             ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_STREAM, 1, s);
             launch_chained(kern, plan.grid, STREAM_THREADS, smem, s, a, plan, ctx->wait_limit_ns);
@@ -216,7 +220,8 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         CompressArgs r = a;
         r.use_redo_list = 1;
         ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_REDO, 2, s);
-        launch_compress_direct<T, true>(r, grid, stats, s);
+        if (aligned) launch_compress_direct<T, true>(r, grid, stats, s);
+        else launch_compress_direct<T, false>(r, grid, stats, s);
     } else {
         ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_STREAM, 1, s);
         if (aligned) launch_compress_direct<T, true>(a, grid, stats, s);
@@ -237,35 +242,24 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
 
 // the streaming statistics pass over the rows a call reads
 template <typename T>
-cudaError_t launch_verify_stream(picospec_ctx* ctx, const VerifyArgs& a, bool aligned, cudaStream_t s) {
+cudaError_t launch_verify_stream(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s) {
     const int stream_rows = a.sample_only ? a.B : a.B * (a.r1 - a.r0);
-    const long long items = (long long)stream_rows * a.nch;
-    long long want = (items + WARPS - 1) / WARPS;
-    const int cap = ctx->num_sms * 4;
-    const int grid = (int)(want < cap ? want : cap);
-    const bool staged = aligned && ((size_t)a.V * sizeof(T)) % 16 == 0;
-    if (staged) {
-        cudaError_t ea = ensure_kernel_attrs(ctx->device);
-        if (ea != cudaSuccess) return ea;
-        const int tiles_per_row = (a.nch + TileGeom<T>::CHUNKS - 1) / TileGeom<T>::CHUNKS;
-        const long long tiles = (long long)stream_rows * tiles_per_row;
-        const int gcap = ctx->num_sms * StreamCfg<T>::CTAS_PER_SM;
-        const int g = (int)(tiles < gcap ? tiles : gcap);
-        ProfScope ps(ctx, PICOSPEC_PROF_VERIFY_STREAM, 1, s);
-        launch_chained(chunk_stats_bulk_kernel<T>, g, STREAM_THREADS, TileGeom<T>::SMEM_BYTES, s, a, tiles_per_row, tiles,
-                       ctx->wait_limit_ns);
-    } else {
-        ProfScope ps(ctx, PICOSPEC_PROF_VERIFY_STREAM, 1, s);
-        if (aligned) launch_chained(chunk_stats_kernel<T, true>, grid, THREADS, 0, s, a);
-        else launch_chained(chunk_stats_kernel<T, false>, grid, THREADS, 0, s, a);
-    }
+    cudaError_t ea = ensure_kernel_attrs(ctx->device);
+    if (ea != cudaSuccess) return ea;
+    const int tiles_per_row = (a.nch + TileGeom<T>::CHUNKS - 1) / TileGeom<T>::CHUNKS;
+    const long long tiles = (long long)stream_rows * tiles_per_row;
+    const int gcap = ctx->num_sms * StreamCfg<T>::CTAS_PER_SM;
+    const int g = (int)(tiles < gcap ? tiles : gcap);
+    ProfScope ps(ctx, PICOSPEC_PROF_VERIFY_STREAM, 1, s);
+    launch_chained(chunk_stats_bulk_kernel<T>, g, STREAM_THREADS, TileGeom<T>::SMEM_BYTES, s, a, tiles_per_row, tiles,
+                   ctx->wait_limit_ns);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_verify(picospec_ctx* ctx, const VerifyArgs& a, bool aligned, cudaStream_t s, bool edge = false) {
+cudaError_t launch_verify(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s, bool edge = false) {
     {
-        cudaError_t e0 = launch_verify_stream<T>(ctx, a, aligned, s);
+        cudaError_t e0 = launch_verify_stream<T>(ctx, a, s);
         if (e0 != cudaSuccess) return e0;
     }
     cudaError_t e = cudaGetLastError();
@@ -611,9 +605,9 @@ static int verify_common(picospec_ctx* ctx, VerifyArgs& a, picospec_dtype dtype,
     cudaStream_t s = (cudaStream_t)cuda_stream;
     cudaError_t e;
     if (dtype == PICOSPEC_BF16)
-        e = launch_verify<__nv_bfloat16>(ctx, a, rows_aligned(a.logits, a.row_stride, 2), s, edge);
+        e = launch_verify<__nv_bfloat16>(ctx, a, s, edge);
     else
-        e = launch_verify<float>(ctx, a, rows_aligned(a.logits, a.row_stride, 4), s, edge);
+        e = launch_verify<float>(ctx, a, s, edge);
     return e == cudaSuccess ? PICOSPEC_OK : fail_cuda(ctx, e);
 }
 
@@ -779,11 +773,11 @@ int picospec_vp_local(picospec_ctx* ctx, const void* slice_logits, picospec_dtyp
     cudaStream_t s = (cudaStream_t)cuda_stream;
     cudaError_t e;
     if (dtype == PICOSPEC_BF16) {
-        e = launch_verify_stream<__nv_bfloat16>(ctx, a, rows_aligned(slice_logits, row_stride_elems, 2), s);
+        e = launch_verify_stream<__nv_bfloat16>(ctx, a, s);
         if (e == cudaSuccess && G > 0)
             launch_chained(vp_gather_kernel<__nv_bfloat16>, ctx->num_sms * 4, THREADS, 0, s, a, v0, Vs, entries_local);
     } else {
-        e = launch_verify_stream<float>(ctx, a, rows_aligned(slice_logits, row_stride_elems, 4), s);
+        e = launch_verify_stream<float>(ctx, a, s);
         if (e == cudaSuccess && G > 0)
             launch_chained(vp_gather_kernel<float>, ctx->num_sms * 4, THREADS, 0, s, a, v0, Vs, entries_local);
     }
@@ -1007,9 +1001,9 @@ extern "C" int picospec_verify_static(const void* target_logits, picospec_dtype 
     a.queue_count = ws->counters; a.status = &ws->status; a.slow_rows = &ws->slow_rows;
     cudaError_t e;
     if (dtype == PICOSPEC_BF16)
-        e = launch_verify<__nv_bfloat16>(&local, a, rows_aligned(a.logits, a.row_stride, 2), s);
+        e = launch_verify<__nv_bfloat16>(&local, a, s);
     else
-        e = launch_verify<float>(&local, a, rows_aligned(a.logits, a.row_stride, 4), s);
+        e = launch_verify<float>(&local, a, s);
     if (e == cudaSuccess && device_status_out)
         e = cudaMemcpyAsync(device_status_out, &ws->status, sizeof(int), cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess && slow_rows_out)

@@ -29,6 +29,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -107,6 +110,65 @@ __device__ __forceinline__ void bulk_load(void* dst_smem, const void* src_gmem, 
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
         ::"r"(smem_addr(dst_smem)), "l"(src_gmem), "r"(bytes), "r"(smem_addr(bar)), "l"(policy)
         : "memory");
+}
+
+// ---- rows at any element offset -----------------------------------------------------------------
+// Bulk copies move whole 16-byte granules, so a row is staged from the granule that holds its first
+// element: "virtual" element v of a row is element v - mis of the vocabulary, mis < GRAIN of them lie
+// before the row and read as -inf, as do those behind its end in its last granule.
+template <typename T> struct StagedRow {
+    static constexpr int GRAIN = 16 / (int)sizeof(T);    // elements per granule
+    const unsigned char* base;    // the row's first granule
+    int mis;                      // elements of it that belong to the row before
+    int end;                      // virtual elements: mis + V
+    __device__ __forceinline__ StagedRow(const T* row, int V) {
+        const uintptr_t p = reinterpret_cast<uintptr_t>(row);
+        base = reinterpret_cast<const unsigned char*>(p & ~(uintptr_t)15);
+        mis = (int)(p & 15u) / (int)sizeof(T);
+        end = mis + V;
+    }
+};
+__device__ __forceinline__ uint32_t logit_bits(const unsigned char* p, const __nv_bfloat16*) {
+    return __ldg(reinterpret_cast<const unsigned short*>(p));
+}
+__device__ __forceinline__ uint32_t logit_bits(const unsigned char* p, const float*) {
+    return __ldg(reinterpret_cast<const uint32_t*>(p));
+}
+// Granule g of a row that is not the row's own to the full: its elements, -inf around them.  The bytes
+// of the neighbouring rows are not read.
+template <typename T> __device__ __forceinline__ void stage_partial_granule(void* dst, const StagedRow<T>& r, int g) {
+    constexpr int GRAIN = StagedRow<T>::GRAIN;
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int e = 0; e < GRAIN; ++e) {
+        const int v = g * GRAIN + e;
+        uint32_t bits = sizeof(T) == 2 ? 0xFF80u : 0xFF800000u;
+        if (v >= r.mis && v < r.end) bits = logit_bits(r.base + (long long)v * (int)sizeof(T), (const T*)nullptr);
+        w[e * (int)sizeof(T) / 4] |= bits << ((e * (int)sizeof(T) % 4) * 8);
+    }
+    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+    // a later bulk copy into this stage must not pass the store
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+// The producer lane's work for one tile, up to its arrival on `bar` (so that what it still has to look up
+// is looked up while the copy is in flight): granules [g0, g0 + n) of the row, as far as the row
+// reaches, to `dst`.  Whole granules come as one bulk copy, the partial ones at the row's two ends are
+// stored by this thread.
+template <typename T>
+__device__ __forceinline__ void stage_tile(unsigned char* dst, const StagedRow<T>& r, int g0, int n, uint64_t* bar,
+                                           uint64_t policy) {
+    constexpr int GRAIN = StagedRow<T>::GRAIN;
+    const int glast = r.end / GRAIN;                            // first granule that is not full at its end
+    const int f0 = max(g0, r.mis ? 1 : 0), f1 = min(g0 + n, glast);
+    if (f1 > f0) {
+        const uint32_t bytes = (uint32_t)(f1 - f0) * 16u;
+        mbar_expect_tx(bar, bytes);
+        bulk_load(dst + (f0 - g0) * 16, r.base + (long long)f0 * 16, bytes, bar, policy);
+    }
+    const bool head = r.mis != 0 && g0 == 0;
+    if (head) stage_partial_granule(dst, r, 0);
+    if (r.end % GRAIN != 0 && glast >= g0 && glast < g0 + n && !(head && glast == 0))
+        stage_partial_granule(dst + (glast - g0) * 16, r, glast);
 }
 
 // ---- packed fp32 pairs (fma.rn.f32x2 / add.rn.f32x2) ------------------------------------------
@@ -196,12 +258,13 @@ template <> struct StreamCfg<float> {
 template <typename T> struct TileGeom {
     static constexpr int CHUNKS = TILE_CHUNKS * StreamCfg<T>::CPW;
     static constexpr int TILE_BYTES = CHUNKS * CHUNK * (int)sizeof(T);
-    static constexpr int SMEM_BYTES = StreamCfg<T>::STAGES * TILE_BYTES;
+    static constexpr int STAGE_BYTES = TILE_BYTES + 16;      // a shifted tile reaches into one more granule
+    static constexpr int SMEM_BYTES = StreamCfg<T>::STAGES * STAGE_BYTES;
 };
 
 // One chunk of a staged tile -> registers, in the lane layout of ChunkRegs (vector j of a lane is
-// the 16 bytes at j*512 + lane*16 of the chunk).  v0: vocabulary index of the chunk's first entry;
-// vectors at or beyond V read as -inf (V is a multiple of the vector length on this path).
+// the 16 bytes at j*512 + lane*16 of the chunk).  v0: (virtual) index of the chunk's first entry;
+// vectors at or beyond V read as -inf (the vector that V cuts is padded with -inf where it is staged).
 __device__ __forceinline__ void load_staged(ChunkRegs<__nv_bfloat16>& r, const unsigned char* chunk, int v0, int V,
                                             int lane) {
     const uint4* p = reinterpret_cast<const uint4*>(chunk) + lane;
@@ -229,6 +292,36 @@ __device__ __forceinline__ void load_staged(ChunkRegs<float>& r, const unsigned 
         for (int j = 0; j < 8; ++j)
             if (v0 + j * 128 + lane * 4 >= V) r.f[4 * j + 0] = r.f[4 * j + 1] = r.f[4 * j + 2] = r.f[4 * j + 3] = -CUDART_INF_F;
     }
+}
+
+// The chunk that begins `mis` elements behind `chunk`: every vector but one is the aligned one; lane 0's
+// first vector takes its first `mis` elements, which belong to the chunk before, from the granule behind
+// the chunk instead, so that the warp holds exactly the chunk's 1024 entries (in an order of its own).
+__device__ __forceinline__ void splice_granule(ChunkRegs<__nv_bfloat16>& r, uint4 next, int mis) {
+    const uint32_t n[4] = {next.x, next.y, next.z, next.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t m = (2 * i < mis ? 0xFFFFu : 0u) | (2 * i + 1 < mis ? 0xFFFF0000u : 0u);
+        r.w[i] = (r.w[i] & ~m) | (n[i] & m);
+    }
+}
+__device__ __forceinline__ void splice_granule(ChunkRegs<float>& r, uint4 next, int mis) {
+    const uint32_t n[4] = {next.x, next.y, next.z, next.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (i < mis) r.f[i] = __uint_as_float(n[i]);
+}
+template <typename T>
+__device__ __forceinline__ void load_staged_shifted(ChunkRegs<T>& r, const unsigned char* chunk, int v0, int end, int mis,
+                                                    int lane) {
+    load_staged(r, chunk, v0, end, lane);
+    if (mis && lane == 0) {
+        uint4 next = *reinterpret_cast<const uint4*>(chunk + CHUNK * (int)sizeof(T));
+        const uint32_t none = sizeof(T) == 2 ? 0xFF80FF80u : 0xFF800000u;
+        if (v0 + CHUNK >= end) next = make_uint4(none, none, none, none);
+        splice_granule(r, next, mis);
+    }
+    if (mis) __syncwarp();
 }
 
 }  // namespace picospec

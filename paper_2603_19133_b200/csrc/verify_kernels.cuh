@@ -57,20 +57,6 @@ struct VerifyArgs {
     unsigned long long* slow_rows;  // cumulative rows re-evaluated in double precision
 };
 
-// ---------------------------------------------------------------------------------------------
-// Streaming pass, direct variant (rows that are not 16-byte aligned): one warp per 1024-entry
-// chunk, read straight from global memory and software-pipelined over two register buffers.
-// Per chunk: exact maximum logit and the fp32 sum of 2^((l - max) * log2e / T).
-// ---------------------------------------------------------------------------------------------
-// one (row, chunk) item of the direct variant
-template <typename T> struct ItemMeta {
-    const T* row;
-    int v0;
-    float c32;
-    long long slot;  // index into stats
-    bool valid;
-};
-
 // Row r of the rows a verify call streams -> (sequence, row of the logits tensor); false: the row
 // is not read (sequence decided earlier, or the row lies beyond the sequence's bonus row).
 __device__ __forceinline__ bool streamed_row(const VerifyArgs& a, int r, int& b, int& src_row) {
@@ -93,82 +79,8 @@ __device__ __forceinline__ long long record_index(const VerifyArgs& a, int row, 
 // flags of VerifyArgs::pick
 constexpr int PICK_RESIDUAL = 1, PICK_FLAGGED = 2, PICK_DRAW_ONLY = 4, PICK_MASS_ONLY = 8;
 
-template <typename T> __device__ __forceinline__ ItemMeta<T> decode_item(const VerifyArgs& a, long long item) {
-    ItemMeta<T> m;
-    const int r = (int)(item / a.nch);
-    const int c = (int)(item - (long long)r * a.nch);
-    int b, src_row;
-    m.valid = true;
-    if (a.sample_only) {
-        b = r;
-        const int j = a.pos[b];
-        if (j < 0 || j > a.G) m.valid = false;
-        src_row = b * (a.G + 1) + (m.valid ? j : 0);
-    } else {
-        if (!streamed_row(a, r, b, src_row)) m.valid = false;
-    }
-    const float Tb = a.temperature[b];
-    if (!temp_ok(Tb)) m.valid = false;
-    m.c32 = temp_scale(Tb);
-    m.row = reinterpret_cast<const T*>(a.logits) + (long long)src_row * a.row_stride;
-    m.v0 = c * CHUNK;
-    m.slot = (long long)src_row * (a.stats_pitch > 0 ? a.stats_pitch : a.nch) + c;
-    return m;
-}
-
-template <typename T> __device__ __forceinline__ void chunk_stats_compute(const ChunkRegs<T>& regs, const ItemMeta<T>& m,
-                                                                          float2* stats, int lane) {
-    const float lm = regs.lane_max();
-    // NaN anywhere in the chunk: the exp-sum below turns NaN and the finish kernel reports it
-    const float cm = warp_max(lm);
-    const float off = __fmul_rn(cm, m.c32);
-    float s = 0.f;
-    if (cm > -CUDART_INF_F) s = lane_exp_sum(regs, m.c32, off);
-    if (lm != lm) s = CUDART_NAN_F;
-    s = warp_sum(s);
-    if (lane == 0) stats[m.slot] = make_float2(cm, s);
-}
-
-template <typename T, bool ALIGNED>
-__global__ void __launch_bounds__(THREADS, 4) chunk_stats_kernel(VerifyArgs a) {
-    grid_dependency_sync();
-    const int lane = threadIdx.x & 31;
-    const long long gw = (long long)blockIdx.x * WARPS + (threadIdx.x >> 5);
-    const long long nw = (long long)gridDim.x * WARPS;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *a.queue_count = 0;
-        *a.rowq_count = 0;
-        if (a.borderline) *a.borderline = 0;
-    }
-    const long long total = (long long)(a.sample_only ? a.B : a.B * (a.r1 - a.r0)) * a.nch;
-    long long itA = gw;
-    if (itA >= total) return;
-    ChunkRegs<T> A, Bf;
-    ItemMeta<T> mA = decode_item<T>(a, itA), mB;
-    if (mA.valid) A.template load<ALIGNED>(mA.row, mA.v0, a.V, lane);
-    for (;;) {
-        const long long itB = itA + nw;
-        const bool hasB = itB < total;
-        if (hasB) {
-            mB = decode_item<T>(a, itB);
-            if (mB.valid) Bf.template load<ALIGNED>(mB.row, mB.v0, a.V, lane);
-        }
-        if (mA.valid) chunk_stats_compute<T>(A, mA, a.stats, lane);
-        if (!hasB) break;
-        itA = itB + nw;
-        const bool hasA = itA < total;
-        if (hasA) {
-            mA = decode_item<T>(a, itA);
-            if (mA.valid) A.template load<ALIGNED>(mA.row, mA.v0, a.V, lane);
-        }
-        if (mB.valid) chunk_stats_compute<T>(Bf, mB, a.stats, lane);
-        if (!hasA) break;
-    }
-}
-
 // ---------------------------------------------------------------------------------------------
-// Streaming pass through shared memory (rows whose base, pitch and length are multiples of 16
-// bytes).  A tile is TILE_CHUNKS consecutive chunks of one row; CTA c takes tiles c, c + grid,
+// Streaming pass through shared memory.  A tile is TILE_CHUNKS consecutive chunks of one row; CTA c takes tiles c, c + grid,
 // c + 2 grid, ...  Warp 8 lane 0 is the producer: it keeps STAGES bulk copies in flight.  Each of
 // the 8 consumer warps moves its chunk of a landed tile to registers, hands the stage back and
 // then reduces the chunk to (maximum logit, fp32 sum of 2^((l - max) * log2e / T)).
@@ -177,7 +89,8 @@ struct TileDesc {
     int src_row;   // row of the logits tensor
     int c0;        // first chunk of the tile
     float c32;     // log2(e) / T of the row's sequence
-    int valid;     // 0: bad temperature or position, or a row that is not read: nothing was copied
+    int mis;       // elements between the row's first granule's start and the row (StagedRow)
+    int valid;     // 0: bad temperature or position, or a row that is not read
 };
 
 template <typename T>
@@ -188,7 +101,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
     constexpr int STAGES = StreamCfg<T>::STAGES;
     constexpr int CPW = StreamCfg<T>::CPW;
     constexpr int TCH = TileGeom<T>::CHUNKS;
-    constexpr int TILE_BYTES = TileGeom<T>::TILE_BYTES;
+    constexpr int TILE_BYTES = TileGeom<T>::TILE_BYTES, STAGE_BYTES = TileGeom<T>::STAGE_BYTES;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES];
     __shared__ TileDesc desc[STAGES];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -211,42 +124,47 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
         // ---- producer ---------------------------------------------------------------------
         if (lane != 0) return;
         const uint64_t pol = l2_evict_first_policy();
-        long long t = blockIdx.x;
-        for (uint32_t i = 0; t < total_tiles; ++i, t += gridDim.x) {
+        // tile t = (streamed row r, tile tc of it); the next tile of this CTA is gridDim.x further on
+        const int step_r = (int)gridDim.x / tiles_per_row, step_tc = (int)gridDim.x - step_r * tiles_per_row;
+        int r = (int)blockIdx.x / tiles_per_row, tc = (int)blockIdx.x - r * tiles_per_row;
+        uint32_t i = 0;
+        for (long long t = blockIdx.x; t < total_tiles; ++i, t += gridDim.x) {
             const int s = (int)(i % STAGES);
             const uint32_t round = i / STAGES;
+            TileDesc d;
+            bool wanted = true;
+            int b;
+            if (a.sample_only) {
+                b = r;
+                const int j = a.pos[b];
+                if (j < 0 || j > a.G) wanted = false;
+                d.src_row = b * (a.G + 1) + (wanted ? j : 0);
+            } else {
+                wanted = streamed_row(a, r, b, d.src_row);
+            }
+            const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (long long)d.src_row * a.row_stride, a.V);
             if (round > 0) {
                 const int wr = mbar_wait_twice(&empty[s], (round - 1) & 1, wait_limit_ns);
                 if (wr != WAIT_OK) atomicOr(a.status, ST_INTERNAL);
                 if (wr == WAIT_LOST) break;       // nothing more is issued
             }
-            const int r = (int)(t / tiles_per_row);
-            const int tc = (int)(t - (long long)r * tiles_per_row);
-            TileDesc d;
-            d.valid = 1;
-            int b;
-            if (a.sample_only) {
-                b = r;
-                const int j = a.pos[b];
-                if (j < 0 || j > a.G) d.valid = 0;
-                d.src_row = b * (a.G + 1) + (d.valid ? j : 0);
-            } else {
-                if (!streamed_row(a, r, b, d.src_row)) d.valid = 0;
+            if (wanted) {
+                constexpr int GRANULES = TILE_BYTES / 16;
+                stage_tile<T>(stage_mem + s * STAGE_BYTES, sr, tc * GRANULES, GRANULES + (sr.mis ? 1 : 0), &full[s], pol);
             }
+            // (looked up with the copy in flight; the copy of a row with a bad temperature is not used)
             const float Tb = a.temperature[b];
-            if (!temp_ok(Tb)) d.valid = 0;
+            d.valid = wanted && temp_ok(Tb);
             d.c32 = temp_scale(Tb);
             d.c0 = tc * TCH;
+            d.mis = sr.mis;
             desc[s] = d;
-            if (d.valid) {
-                const int v0 = d.c0 * CHUNK;
-                const int v1 = min(a.V, v0 + TCH * CHUNK);
-                const uint32_t bytes = (uint32_t)(v1 - v0) * (uint32_t)sizeof(T);
-                const T* src = reinterpret_cast<const T*>(a.logits) + (long long)d.src_row * a.row_stride + v0;
-                mbar_arrive_expect_tx(&full[s], bytes);
-                bulk_load(stage_mem + s * TILE_BYTES, src, bytes, &full[s], pol);
-            } else {
-                mbar_arrive(&full[s]);
+            mbar_arrive(&full[s]);
+            r += step_r;
+            tc += step_tc;
+            if (tc >= tiles_per_row) {
+                tc -= tiles_per_row;
+                ++r;
             }
         }
         return;
@@ -270,7 +188,9 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
             const int c = d.c0 + warp * CPW + q;
             const bool work = d.valid && c < a.nch && !late;
             ChunkRegs<T> regs;
-            if (work) load_staged(regs, stage_mem + s * TILE_BYTES + (warp * CPW + q) * (CHUNK * (int)sizeof(T)), c * CHUNK, a.V, lane);
+            if (work)
+                load_staged_shifted(regs, stage_mem + s * STAGE_BYTES + (warp * CPW + q) * (CHUNK * (int)sizeof(T)), c * CHUNK,
+                                    a.V + d.mis, d.mis, lane);
             if (q == CPW - 1) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);     // the warp's chunks are in registers or done
