@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the picospec C-ABI (include/picospec.h).
+"""Thin binding of the picospec C-ABI (include/picospec.h): ctypes, and native marshalling
+(csrc/marshal.cpp) for the calls of the hot path.
 
 Argument marshalling only: every step of the path runs in the CUDA kernels of
 libpicospec.so.  torch supplies device memory and the current stream.  There is no CPU
@@ -19,15 +20,19 @@ OK, EINVAL, ECUDA, ECAPACITY, EDATA = 0, -1, -2, -3, -4
 CHUNK = 1024
 
 _lib = None
+_marshal = None
 
 
 def lib() -> ctypes.CDLL:
     """Load libpicospec.so (built in-tree by build.build()); fail loudly if it is absent."""
-    global _lib
+    global _lib, _marshal
     if _lib is None:
         path = _build.LIB
-        if not os.path.exists(path):
+        if not os.path.exists(path) or not os.path.exists(_build.MARSHAL):
             path = _build.build()
+        from . import _marshal as native
+        native.open(path)
+        _marshal = native
         L = ctypes.CDLL(path)
         c_int, c_ll, c_f, vp = ctypes.c_int, ctypes.c_longlong, ctypes.c_float, ctypes.c_void_p
         L.picospec_create.argtypes = [ctypes.POINTER(vp), c_int, c_int, c_int, c_int, c_int]
@@ -240,20 +245,17 @@ class Context:
                  k_max: int, u_draft: Optional[torch.Tensor] = None, out=None):
         """picospec_compress.  Returns (q_idx [B,G,k_max] i32, q_prob f32, q_count [B,G] i32,
         draft_tok [B,G] i32 or None)."""
-        p, dt, B, G, V, pitch = _logits(draft_logits)
-        dev = draft_logits.device
         if out is None:
+            B, G, _ = draft_logits.shape
+            dev = draft_logits.device
             q_idx = torch.empty((B, G, k_max), dtype=torch.int32, device=dev)
             q_prob = torch.empty((B, G, k_max), dtype=torch.float32, device=dev)
             q_count = torch.empty((B, G), dtype=torch.int32, device=dev)
             tok = torch.empty((B, G), dtype=torch.int32, device=dev) if u_draft is not None else None
         else:
             q_idx, q_prob, q_count, tok = out
-        _check(lib().picospec_compress(
-            self._h, p, dt, B, G, V, pitch, _ptr(temperature, torch.float32, (B,)), int(top_k), float(top_p),
-            int(k_max), _ptr(q_idx, torch.int32, (B, G, k_max)), _ptr(q_prob, torch.float32, (B, G, k_max)),
-            _ptr(q_count, torch.int32, (B, G)), _ptr(u_draft, torch.float32, (B, G)),
-            _ptr(tok, torch.int32, (B, G)), _stream()), "picospec_compress")
+        _check(_marshal.compress(self._h.value or 0, draft_logits, temperature, int(top_k), float(top_p), int(k_max),
+                                 u_draft, q_idx, q_prob, q_count, tok), "picospec_compress")
         return q_idx, q_prob, q_count, tok
 
     # -- half 2a (+2b fused) ------------------------------------------------------------
@@ -262,11 +264,9 @@ class Context:
                u_resample: Optional[torch.Tensor] = None, out=None):
         """picospec_verify.  Returns dict(accept_len [B], p_draft [B,G], resid_mass [B,G],
         borderline_count [1], token [B] or None)."""
-        p, dt, B, G1, V, pitch = _logits(target_logits)
-        G = G1 - 1
-        k_max = q_idx.shape[-1]
-        dev = target_logits.device
         if out is None:
+            B, G = target_logits.shape[0], target_logits.shape[1] - 1
+            dev = target_logits.device
             out = {
                 "accept_len": torch.empty((B,), dtype=torch.int32, device=dev),
                 "p_draft": torch.empty((B, G), dtype=torch.float32, device=dev),
@@ -274,14 +274,9 @@ class Context:
                 "borderline_count": torch.empty((1,), dtype=torch.int32, device=dev),
                 "token": torch.empty((B,), dtype=torch.int32, device=dev) if u_resample is not None else None,
             }
-        _check(lib().picospec_verify(
-            self._h, p, dt, B, G, V, pitch, _ptr(temperature, torch.float32, (B,)),
-            _ptr(draft_tok, torch.int32, (B, G)), _ptr(q_idx, torch.int32, (B, G, k_max)),
-            _ptr(q_prob, torch.float32, (B, G, k_max)), _ptr(q_count, torch.int32, (B, G)), int(k_max),
-            _ptr(u_accept, torch.float32, (B, G)), _ptr(out["accept_len"], torch.int32, (B,)),
-            _ptr(out["p_draft"], torch.float32, (B, G)), _ptr(out["resid_mass"], torch.float32, (B, G)),
-            _ptr(out["borderline_count"], torch.int32, (1,)), _ptr(u_resample, torch.float32, (B, 2)),
-            _ptr(out["token"], torch.int32, (B,)), _stream()), "picospec_verify")
+        _check(_marshal.verify(self._h.value or 0, target_logits, temperature, draft_tok, q_idx, q_prob, q_count, u_accept,
+                               u_resample, out["accept_len"], out["p_draft"], out["resid_mass"],
+                               out["borderline_count"], out["token"]), "picospec_verify")
         return out
 
     def verify_range(self, target_logits: torch.Tensor, temperature: torch.Tensor, gamma: Optional[torch.Tensor],
@@ -291,11 +286,9 @@ class Context:
         """picospec_verify_range on the target rows [r0, r1).  `out` is the dict of an earlier call
         (its arrays are updated in place; state may alias state_in) or None.  Returns dict(accept_len,
         p_draft, resid_mass, borderline_count, token or None, state [B] i32)."""
-        p, dt, B, G1, V, pitch = _logits(target_logits)
-        G = G1 - 1
-        k_max = q_idx.shape[-1]
-        dev = target_logits.device
         if out is None:
+            B, G = target_logits.shape[0], target_logits.shape[1] - 1
+            dev = target_logits.device
             out = {
                 "accept_len": torch.full((B,), -2, dtype=torch.int32, device=dev),
                 "p_draft": torch.full((B, G), float("nan"), dtype=torch.float32, device=dev),
@@ -304,16 +297,10 @@ class Context:
                 "token": torch.full((B,), -2, dtype=torch.int32, device=dev) if u_resample is not None else None,
                 "state": torch.empty((B,), dtype=torch.int32, device=dev),
             }
-        _check(lib().picospec_verify_range(
-            self._h, p, dt, B, G, V, pitch, _ptr(temperature, torch.float32, (B,)), _ptr(gamma, torch.int32, (B,)),
-            int(r0), int(r1), _ptr(state_in, torch.int32, (B,)),
-            _ptr(draft_tok, torch.int32, (B, G)), _ptr(q_idx, torch.int32, (B, G, k_max)),
-            _ptr(q_prob, torch.float32, (B, G, k_max)), _ptr(q_count, torch.int32, (B, G)), int(k_max),
-            _ptr(u_accept, torch.float32, (B, G)), _ptr(out["accept_len"], torch.int32, (B,)),
-            _ptr(out["p_draft"], torch.float32, (B, G)), _ptr(out["resid_mass"], torch.float32, (B, G)),
-            _ptr(out["borderline_count"], torch.int32, (1,)), _ptr(u_resample, torch.float32, (B, 2)),
-            _ptr(out["token"], torch.int32, (B,)), _ptr(out["state"], torch.int32, (B,)), _stream()),
-            "picospec_verify_range")
+        _check(_marshal.verify_range(self._h.value or 0, target_logits, temperature, gamma, int(r0), int(r1), state_in,
+                                     draft_tok, q_idx, q_prob, q_count, u_accept, u_resample, out["accept_len"],
+                                     out["p_draft"], out["resid_mass"], out["borderline_count"], out["token"],
+                                     out["state"]), "picospec_verify_range")
         return out
 
     # -- the paper's own data flow (Sec. 3.3) ---------------------------------------------------
@@ -321,18 +308,15 @@ class Context:
                     out=None):
         """picospec_target_topk.  Returns (p_idx [B,k] i32, p_prob [B,k] f32 unnormalised, p_count [B] i32);
         `out` = such a triple to write into."""
-        p, dt, B, R, V, pitch = _logits(target_logits)
-        dev = target_logits.device
         if out is not None:
             p_idx, p_prob, p_count = out
-            _ptr(p_idx, torch.int32, (B, k)), _ptr(p_prob, torch.float32, (B, k)), _ptr(p_count, torch.int32, (B,))
         else:
+            B, dev = target_logits.shape[0], target_logits.device
             p_idx = torch.empty((B, k), dtype=torch.int32, device=dev)
             p_prob = torch.empty((B, k), dtype=torch.float32, device=dev)
             p_count = torch.empty((B,), dtype=torch.int32, device=dev)
-        _check(lib().picospec_target_topk(
-            self._h, p, dt, B, R, V, pitch, _ptr(temperature, torch.float32, (B,)), _ptr(pos, torch.int32, (B,)),
-            int(k), _ptr(p_idx), _ptr(p_prob), _ptr(p_count), _stream()), "picospec_target_topk")
+        _check(_marshal.target_topk(self._h.value or 0, target_logits, temperature, pos, int(k), p_idx, p_prob, p_count),
+               "picospec_target_topk")
         return p_idx, p_prob, p_count
 
     def edge_resample(self, draft_logits: torch.Tensor, temperature: torch.Tensor, pos: torch.Tensor,
@@ -340,19 +324,14 @@ class Context:
                       want_mass: bool = True, out=None):
         """picospec_edge_resample.  Returns (token [B] i32, mass [B] f32 or None); `out` = such a pair
         to write into."""
-        p, dt, B, R, V, pitch = _logits(draft_logits)
-        k = p_idx.shape[-1]
-        dev = draft_logits.device
         if out is not None:
             token, mass = out
-            _ptr(token, torch.int32, (B,)), _ptr(mass, torch.float32, (B,))
         else:
+            B, dev = draft_logits.shape[0], draft_logits.device
             token = torch.empty((B,), dtype=torch.int32, device=dev)
             mass = torch.empty((B,), dtype=torch.float32, device=dev) if want_mass else None
-        _check(lib().picospec_edge_resample(
-            self._h, p, dt, B, R, V, pitch, _ptr(temperature, torch.float32, (B,)), _ptr(pos, torch.int32, (B,)),
-            _ptr(p_idx, torch.int32, (B, k)), _ptr(p_prob, torch.float32, (B, k)), _ptr(p_count, torch.int32, (B,)),
-            int(k), _ptr(u, torch.float32, (B,)), _ptr(token), _ptr(mass), _stream()), "picospec_edge_resample")
+        _check(_marshal.edge_resample(self._h.value or 0, draft_logits, temperature, pos, p_idx, p_prob, p_count, u, token,
+                                      mass), "picospec_edge_resample")
         return token, mass
 
     # -- wire format of the sparse rows (Sec. 3.3) ---------------------------------------------
@@ -368,9 +347,8 @@ class Context:
             buf = torch.empty((wire_bytes(R, R * K, ptype),), dtype=torch.uint8, device=q_idx.device)
         if bytes_out is None:
             bytes_out = torch.empty((1,), dtype=torch.int64, device=q_idx.device)
-        _check(lib().picospec_wire_pack(
-            self._h, _ptr(q_idx, torch.int32), _ptr(q_prob, torch.float32), _ptr(q_count, torch.int32), R, int(K), ptype,
-            _ptr(buf, torch.uint8), int(buf.numel()), _ptr(bytes_out, torch.int64, (1,)), _stream()), "picospec_wire_pack")
+        _check(_marshal.wire_pack(self._h.value or 0, q_idx, q_prob, q_count, R, K, ptype, buf, bytes_out),
+               "picospec_wire_pack")
         return buf, bytes_out
 
     def wire_unpack(self, buf: torch.Tensor, nbytes: int, rows: int, k: int, out=None):
@@ -380,9 +358,7 @@ class Context:
             out = (torch.empty((rows, k), dtype=torch.int32, device=dev),
                    torch.empty((rows, k), dtype=torch.float32, device=dev),
                    torch.empty((rows,), dtype=torch.int32, device=dev))
-        _check(lib().picospec_wire_unpack(
-            self._h, _ptr(buf, torch.uint8), int(nbytes), int(rows), int(k), _ptr(out[0], torch.int32, (rows, k)),
-            _ptr(out[1], torch.float32, (rows, k)), _ptr(out[2], torch.int32, (rows,)), _stream()), "picospec_wire_unpack")
+        _check(_marshal.wire_unpack(self._h.value or 0, buf, int(nbytes), int(rows), int(k), *out), "picospec_wire_unpack")
         return out
 
     # -- half 2b ---------------------------------------------------------------------
@@ -390,15 +366,9 @@ class Context:
                         q_idx: torch.Tensor, q_prob: torch.Tensor, q_count: torch.Tensor,
                         u_resample: torch.Tensor, want_mass: bool = True):
         """picospec_residual_sample.  Returns (token [B] i32, mass [B] f32 or None)."""
-        p, dt, B, G1, V, pitch = _logits(target_logits)
-        G = G1 - 1
-        k_max = q_idx.shape[-1] if G > 0 else 1
-        dev = target_logits.device
+        B, dev = target_logits.shape[0], target_logits.device
         token = torch.empty((B,), dtype=torch.int32, device=dev)
         mass = torch.empty((B,), dtype=torch.float32, device=dev) if want_mass else None
-        _check(lib().picospec_residual_sample(
-            self._h, p, dt, B, G, V, pitch, _ptr(temperature, torch.float32, (B,)), _ptr(pos, torch.int32, (B,)),
-            _ptr(q_idx, torch.int32), _ptr(q_prob, torch.float32), _ptr(q_count, torch.int32), int(k_max),
-            _ptr(u_resample, torch.float32, (B, 2)), _ptr(token, torch.int32, (B,)),
-            _ptr(mass, torch.float32, (B,)), _stream()), "picospec_residual_sample")
+        _check(_marshal.residual_sample(self._h.value or 0, target_logits, temperature, pos, q_idx, q_prob, q_count, u_resample,
+                                        token, mass), "picospec_residual_sample")
         return token, mass

@@ -1,13 +1,17 @@
-"""Build the C-ABI CUDA library for sm_100a with nvcc (no GPU needed to compile)."""
+"""Build the C-ABI CUDA library for sm_100a with nvcc and the torch argument marshaller with g++ (no GPU
+needed to compile)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpicospec.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
+MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 SOURCES = [os.path.join(CSRC, "picospec_api.cu")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
@@ -37,7 +41,30 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(res.stdout + res.stderr)
         if res.returncode != 0:
             raise RuntimeError("nvcc failed building libpicospec.so")
+    build_marshal(force)
     return LIB
+
+
+def build_marshal(force: bool = False) -> str:
+    """Compile _marshal.so (csrc/marshal.cpp) against the installed torch."""
+    header = os.path.join(os.path.dirname(HERE), "include", "picospec.h")
+    if not force and os.path.exists(MARSHAL) and all(
+            os.path.getmtime(p) <= os.path.getmtime(MARSHAL) for p in (MARSHAL_SOURCE, header)):
+        return MARSHAL
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    lib = os.path.join(root, "lib")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], MARSHAL_SOURCE, "-o", MARSHAL,
+           "-L" + lib, "-Wl,-rpath," + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("g++ failed building _marshal.so")
+    return MARSHAL
 
 
 if __name__ == "__main__":

@@ -28,6 +28,7 @@ struct picospec_ctx {
     unsigned long long wait_limit_ns;   // first limit of the staged kernels' waits
     int last_cuda_error;
     unsigned long long compress_calls;
+    int filter_ctas[2][2][2];           // resident CTAs per SM of the filter kernel's variants (0: not asked yet)
     // optional per-kernel timing (picospec_profile_*): rings of event pairs per kernel kind
     int prof_level;
     cudaEvent_t prof_ev[PICOSPEC_PROF_KINDS][PROF_RING][2];
@@ -188,11 +189,14 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
             small ? (stats ? compress_filter_kernel<T, true, true> : compress_filter_kernel<T, false, true>)
                   : (stats ? compress_filter_kernel<T, true, false> : compress_filter_kernel<T, false, false>);
         const int smem = small ? CsGeom<T, true>::SMEM_BYTES : CsGeom<T, false>::SMEM_BYTES;
-        int per_sm = 1;     // resident CTAs per SM for this kernel's registers and shared memory
-        cudaError_t eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, STREAM_THREADS, smem);
-        if (eo != cudaSuccess) return eo;
-        if (per_sm < 1) per_sm = 1;
-        if (per_sm > FILTER_MAX_CTAS_PER_SM) per_sm = FILTER_MAX_CTAS_PER_SM;
+        // resident CTAs per SM for this kernel's registers and shared memory (asking costs a microsecond: once)
+        int& per_sm = ctx->filter_ctas[sizeof(T) == 2][small][stats];
+        if (per_sm == 0) {
+            cudaError_t eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, STREAM_THREADS, smem);
+            if (eo != cudaSuccess) return eo;
+            if (per_sm < 1) per_sm = 1;
+            if (per_sm > FILTER_MAX_CTAS_PER_SM) per_sm = FILTER_MAX_CTAS_PER_SM;
+        }
         // whole rows first, the remainder in pieces so that every CTA streams about the same number of tiles
         // (a row that does not start on a 16-byte boundary is staged with up to one granule more)
         constexpr int TILE = TILE_CHUNKS * CHUNK;
