@@ -45,7 +45,6 @@ struct picospec_ctx {
     int* redo_rows; // rows the staged compress kernel hands to the direct kernel
     unsigned long long* surv_keys;  // staged compress: survivors per row
     CsRowMeta* surv_meta;
-    int* wire_off;                  // wire codec: first entry of each row, [rows + 1]
     int* vp_listed;                 // vocabulary-parallel verify: per sequence, its kind in the double-precision pass
     int* tickets;                   // compress: per queue slot, chunk sums completed in the double-precision cut
     int* rowq;                      // verify: rows whose exact chunk sums are wanted (count: counters[5])
@@ -350,7 +349,6 @@ int picospec_create(picospec_ctx** out, int device, int max_batch, int max_gamma
     const size_t pieces = rows + 2 * (size_t)ctx->num_sms * FILTER_MAX_CTAS_PER_SM;
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->surv_keys, pieces * (size_t)cs_survivor_cap(max_k) * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->surv_meta, pieces * sizeof(CsRowMeta));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->wire_off, (rows + 1) * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->vp_listed, (size_t)max_batch * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->tickets, rows * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->rowq, rows * sizeof(int));
@@ -386,7 +384,6 @@ int picospec_destroy(picospec_ctx* ctx) {
     cudaFree(ctx->redo_rows);
     cudaFree(ctx->surv_keys);
     cudaFree(ctx->surv_meta);
-    cudaFree(ctx->wire_off);
     cudaFree(ctx->vp_listed);
     cudaFree(ctx->tickets);
     cudaFree(ctx->rowq);
@@ -536,18 +533,15 @@ static int wire_common(picospec_ctx* ctx, WireArgs& a, bool pack, void* cuda_str
     if (a.R == 0 && !pack) return PICOSPEC_OK;
     DeviceGuard g(ctx->device);
     if (!g.ok) return fail_cuda(ctx, cudaErrorInvalidDevice);
-    a.offsets = ctx->wire_off;
     a.status = ctx->status;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int rows_grid = a.R > 0 ? (a.R + WARPS - 1) / WARPS : 1;
-    const int grid = rows_grid < ctx->num_sms * 8 ? rows_grid : ctx->num_sms * 8;
-    if (pack) {
-        launch_chained(wire_scan_kernel<true>, 1, THREADS, 0, s, a);
-        launch_chained(wire_move_kernel<true>, grid, THREADS, 0, s, a);
-    } else {
-        launch_chained(wire_scan_kernel<false>, 1, THREADS, 0, s, a);
-        launch_chained(wire_move_kernel<false>, grid, THREADS, 0, s, a);
-    }
+    const int together = THREADS / wire_row_threads(a.K);        // rows a CTA moves at a time
+    const int most = ctx->num_sms * 8;
+    int per_cta = (a.R + most - 1) / most;
+    per_cta = per_cta < 1 ? together : (per_cta + together - 1) / together * together;
+    const int grid = a.R > 0 ? (a.R + per_cta - 1) / per_cta : 1;
+    if (pack) launch_chained(wire_kernel<true>, grid, THREADS, 0, s, a, per_cta);
+    else launch_chained(wire_kernel<false>, grid, THREADS, 0, s, a, per_cta);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PICOSPEC_OK : fail_cuda(ctx, e);
 }
