@@ -191,14 +191,18 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
             if (work)
                 load_staged_shifted(regs, stage_mem + s * STAGE_BYTES + (warp * CPW + q) * (CHUNK * (int)sizeof(T)), c * CHUNK,
                                     a.V + d.mis, d.mis, lane);
+            // chunk maximum with NaN ignored; a NaN (or +inf) logit turns the exp-sum into NaN by
+            // itself, which the finish kernel reports; a chunk of -inf only sums to zero
+            const float cm = work ? warp_max_redux(regs.lane_max_plain()) : 0.f;
             if (q == CPW - 1) {
+                // The stage is handed back only behind an instruction that needs every lane's entries: an
+                // arrive may overtake shared-memory loads that are issued but still queued, and with
+                // another kernel's gathers in the queue they were queued long enough for the next copy
+                // to land first.
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);     // the warp's chunks are in registers or done
+                if (lane == 0) mbar_arrive(&empty[s]);
             }
             if (work) {
-                // chunk maximum with NaN ignored; a NaN (or +inf) logit turns the exp-sum into NaN by
-                // itself, which the finish kernel reports; a chunk of -inf only sums to zero
-                const float cm = warp_max_redux(regs.lane_max_plain());
                 const float off = cm > -CUDART_INF_F ? __fmul_rn(cm, d.c32) : 0.f;
                 const float sum = warp_sum(lane_exp_sum2(regs, d.c32, off));
                 if (lane == 0) a.stats[(long long)d.src_row * (a.stats_pitch > 0 ? a.stats_pitch : a.nch) + c] = make_float2(cm, sum);
