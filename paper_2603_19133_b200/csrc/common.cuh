@@ -249,10 +249,17 @@ template <typename T> __device__ __forceinline__ float lane_exp_sum(const ChunkR
 // access to global memory, until that kernel has completed and its writes are visible; then the
 // CTA allows the kernel after it to be scheduled in the same way.  (Without the launch attribute
 // both instructions do nothing.)
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_sync() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    grid_dependency_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+
+// exp / exp2 as real calls.  The finish kernels are long chains that each CTA runs once, so the time to
+// fetch instructions counts: two dozen inlined copies of the double-precision exponential are most
+// of their code.
+__device__ __noinline__ double exp_call(double x) { return exp(x); }
+__device__ __noinline__ double exp2_call(double x) { return exp2(x); }
 
 // Double-precision weight of one logit: exp(l * (1/T) - row_max * (1/T)) (the definition's
 // exp(l/T - max/T) with the division replaced by one multiplication: 2^-53 relative per term).
@@ -267,10 +274,11 @@ template <bool PRECISE> struct Weight {
         t = 1.0 / (double)T;
         m = (double)row_max * t;
     }
-    __device__ __forceinline__ double operator()(float l) const { return exp((double)l * t - m); }
+    __device__ __forceinline__ double operator()(float l) const { return exp_call((double)l * t - m); }
+    __device__ __forceinline__ double inlined(float l) const { return exp((double)l * t - m); }   // several in flight
 };
 __device__ __forceinline__ double stream_sum_scale(float row_max, float c32) {
-    return exp2((double)__fmul_rn(row_max, c32) - (double)row_max * (double)c32);
+    return exp2_call((double)__fmul_rn(row_max, c32) - (double)row_max * (double)c32);
 }
 
 }  // namespace picospec

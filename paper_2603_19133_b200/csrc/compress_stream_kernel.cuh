@@ -875,7 +875,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
     if (STATS) {
         // move every piece's streamed sum from its reference onto the scale of the weights exp(l/T - top/T)
         const float c32 = temp_scale(Tb);
-        if (meta.count > 0) Z = meta.z_stream * exp2((double)meta.ref_off - (double)top * (double)c32);
+        if (meta.count > 0) Z = meta.z_stream * exp2_call((double)meta.ref_off - (double)top * (double)c32);
         __syncwarp();
         Z = warp_sum(Z);
     }

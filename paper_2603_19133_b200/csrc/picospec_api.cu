@@ -243,6 +243,17 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
     return cudaGetLastError();
 }
 
+// Shared memory of the verify finish kernel: the chunk masses of every row that it reads where they fit
+// the 48 KB that need no opt-in beside the kernel's static 6 KB (up to 11 rows of 262144 entries) and the
+// warp that reads a row has few entries to take out of them (about 200 cycles per 32); else those of the
+// sampled row, formed by the whole CTA once the row is known (about 3300 cycles).
+size_t finish_masses_bytes(VerifyArgs& a) {
+    const size_t row = (size_t)a.nch * sizeof(double);
+    const size_t all = row * (size_t)(a.sample_only ? 1 : a.r1 - a.r0);
+    a.cm_rows = all <= 40960 && a.k_max <= (a.sample_only ? 128 : 256);
+    return a.cm_rows ? all : row;
+}
+
 // the streaming statistics pass over the rows a call reads
 template <typename T>
 cudaError_t launch_verify_stream(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s) {
@@ -267,11 +278,12 @@ cudaError_t launch_verify(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const size_t dyn = (size_t)a.nch * sizeof(double);
+    VerifyArgs f = a;
+    const size_t dyn = finish_masses_bytes(f);
     {
         ProfScope ps(ctx, PICOSPEC_PROF_VERIFY_FINISH, 2, s);
         if (edge) launch_chained(edge_finish_kernel<T, false>, a.B, THREADS, 0, s, a);
-        else launch_chained(verify_finish_kernel<T, false>, a.B, THREADS, dyn, s, a);
+        else launch_chained(verify_finish_kernel<T, false>, a.B, THREADS, dyn, s, f);
     }
     ProfScope ps3(ctx, PICOSPEC_PROF_VERIFY_PRECISE, 2, s);
     PreciseArgs p;
@@ -282,7 +294,7 @@ cudaError_t launch_verify(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s
     launch_chained(precise_chunk_sums_kernel<T>, ctx->num_sms * 6, THREADS, 0, s, p);
     const int g2 = a.B < ctx->num_sms ? a.B : ctx->num_sms;
     if (edge) launch_chained(edge_finish_kernel<T, true>, g2, THREADS, 0, s, a);
-    else launch_chained(verify_finish_kernel<T, true>, g2, THREADS, dyn, s, a);
+    else launch_chained(verify_finish_kernel<T, true>, g2, THREADS, dyn, s, f);
     return cudaGetLastError();
 }
 
@@ -805,7 +817,7 @@ int picospec_vp_decide(picospec_ctx* ctx, int B, int G, int V, int ranks, int ch
     a.dsum = const_cast<double*>(sums_all);
     a.entry_logits = entries_all; a.pick = pick;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const size_t dyn = (size_t)a.nch * sizeof(double);
+    const size_t dyn = finish_masses_bytes(a);
     cudaError_t e = cudaSuccess;
     if (!sums_all) {
         e = cudaMemsetAsync(borderline_count, 0, sizeof(int), s);

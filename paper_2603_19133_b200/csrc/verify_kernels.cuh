@@ -43,6 +43,7 @@ struct VerifyArgs {
     long long rank_stride = 0;      // records between two ranks' blocks
     int stats_pitch = 0;            // records per row written by the streaming pass (0: nch)
     const float* entry_logits = nullptr;   // [B*G, k_max + 1]
+    bool cm_rows = false;           // the finish kernel keeps the chunk masses of every row it reads
     int* pick = nullptr;            // [B, 4]: sampled row, picked chunk (-1: none), flags, unused
     // workspace
     float2* stats;             // [B*(G+1), nch]: (chunk max logit, sum of 2^(l*c32 - max*c32))
@@ -219,101 +220,153 @@ struct FinishShared {
     double Zraw[MAX_G1];  // the same sum on the streaming pass's own scale (fast path)
     float mx[MAX_G1];
     int bad;
-    int acc[MAX_G1], amb[MAX_G1], bord[MAX_G1], small[MAX_G1];
-    double warp_tot[WARPS];
-    double red[WARPS];
-    int tok, last, flag;
-    int cstar;
-    double Rtot;
-    float qloc[CHUNK];
+    int flag;
+    unsigned char test[MAX_G1];   // per draft position: TEST_* bits
+    double warp_tot[WARPS], warp_q[WARPS];
+    int warp_first[WARPS], warp_last[WARPS];
+    __align__(16) float qloc[CHUNK];
 };
 
 // queue entries of the verify path: the sequence, plus a flag
 constexpr int QUEUE_SEQ_MASK = 0x1FFFFFFF, QUEUE_DRAW_ONLY = 0x40000000, QUEUE_MASS_ONLY = 0x20000000;
 
+// outcome of a position's test: accepted, too close to call, borderline, small residual mass
+constexpr int TEST_ACC = 1, TEST_AMB = 2, TEST_BORD = 4, TEST_SMALL = 8;
+
 // bit i of a sequence's row mask (rows beyond 63 always count as set)
 __device__ __forceinline__ bool row_needed(unsigned long long need, int i) { return i >= 64 || ((need >> i) & 1ull); }
 
+// Combine the chunk statistics of one row (called by a full warp): the exact double-precision chunk sums
+// if they were recomputed for this row, else the fp32 streaming statistics.  masses (or null): [nch]
+// doubles of shared memory that receive the chunk masses, in units where the row sums to one.
 template <typename T>
 __device__ __forceinline__ void row_stats(const VerifyArgs& a, int src_row, float c32, int lane, bool exact, double& Z,
-                                          double& Zraw, float& mx, bool& bad) {
-    // combine the chunk statistics of one row (called by a full warp): the exact double-precision
-    // chunk sums if they were recomputed for this row, else the fp32 streaming statistics
+                                          double& Zraw, float& mx, bool& bad, double* masses = nullptr) {
     bad = false;
     Zraw = 0.0;
+    double scale;
     if (exact) {
         mx = a.row_max[src_row];
         double s = 0.0;
-        for (int c = lane; c < a.nch; c += 32) s += a.dsum[record_index(a, src_row, c)];
+        for (int c = lane; c < a.nch; c += 32) {
+            const double e = a.dsum[record_index(a, src_row, c)];
+            s += e;
+            if (masses) masses[c] = e;
+        }
+        __syncwarp();
         Z = warp_sum(s);
+        scale = 1.0 / Z;
     } else {
-        const float2* st = a.stats;
+        constexpr int HELD = 8;         // records per lane that stay in registers: the first 256 chunks
+        float2 held[HELD];
         float m = -CUDART_INF_F;
         bool nan = false;
-        for (int c = lane; c < a.nch; c += 32) {
-            float2 v = st[record_index(a, src_row, c)];
-            m = fmaxf(m, v.x);
-            nan |= (v.y != v.y);
+#pragma unroll
+        for (int u = 0; u < HELD; ++u) {
+            const int c = u * 32 + lane;
+            held[u] = c < a.nch ? a.stats[record_index(a, src_row, c)] : make_float2(-CUDART_INF_F, 0.f);
         }
-        m = warp_max(m);
+#pragma unroll
+        for (int u = 0; u < HELD; ++u) {
+            m = fmaxf(m, held[u].x);
+            nan |= held[u].y != held[u].y;
+        }
+        for (int c = HELD * 32 + lane; c < a.nch; c += 32) {
+            const float2 v = a.stats[record_index(a, src_row, c)];
+            m = fmaxf(m, v.x);
+            nan |= v.y != v.y;
+        }
+        __syncwarp();
+        m = warp_max_redux(m);
         nan = __any_sync(0xffffffffu, nan);
         mx = m;
         bad = nan || !(m > -CUDART_INF_F) || !(m < CUDART_INF_F);
         double s = 0.0;
+        const double off = (double)__fmul_rn(m, c32);
         if (!bad) {
-            const double off = (double)__fmul_rn(m, c32);
-            for (int c = lane; c < a.nch; c += 32) {
-                float2 v = st[record_index(a, src_row, c)];
-                if (v.x > -CUDART_INF_F) s += (double)v.y * exp2((double)__fmul_rn(v.x, c32) - off);
+            // (one copy of the body, the records shifted through: see exp_call)
+#pragma unroll 1
+            for (int c0 = 0; c0 < a.nch; c0 += 32) {
+                const int c = c0 + lane;
+                float2 v = held[0];
+#pragma unroll
+                for (int u = 0; u + 1 < HELD; ++u) held[u] = held[u + 1];
+                if (c0 >= HELD * 32) v = c < a.nch ? a.stats[record_index(a, src_row, c)] : make_float2(-CUDART_INF_F, 0.f);
+                const double e = v.x > -CUDART_INF_F ? (double)v.y * exp2_call((double)__fmul_rn(v.x, c32) - off) : 0.0;
+                s += e;
+                if (masses && c < a.nch) masses[c] = e;
             }
         }
+        __syncwarp();
         Zraw = warp_sum(s);
         if (!(Zraw > 0.0)) bad = true;
         Z = bad ? 0.0 : Zraw * stream_sum_scale(m, c32);
+        scale = 1.0 / Zraw;
     }
+    if (masses)
+        for (int c = lane; c < a.nch; c += 32) masses[c] *= scale;      // (each lane its own)
+    __syncwarp();
 }
 
 // Level 2 of the sampler, by the 256 threads of a CTA: the token inside chunk `cs` of a row whose
 // logits start at `row` with vocabulary index `vbase` (0 for a whole row; the first index of the
 // slice when the vocabulary is sharded).  Weights are max(0, p - q~) with the stored entries
-// (idx, prob)[0 .. n) if use_resid, else p.  Sets sh.flag when the fast pass cannot call the draw.
+// (idx, prob)[0 .. n) if use_resid, else p.  sh.qloc is zero on entry (and a barrier lies behind that).
+// Sets sh.flag when the fast pass cannot call the draw.
 template <typename T, bool PRECISE>
 __device__ __forceinline__ int level2_draw(const VerifyArgs& a, const T* row, int vbase, int cs, const int* idx,
                                            const float* prob, int n, bool use_resid, const Weight<PRECISE>& wt,
                                            double invZ, float u2, FinishShared& sh) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // the 1024 entries of chunk cs, four consecutive entries per thread
     const int v0 = cs * CHUNK;
-    for (int k = tid; k < CHUNK; k += THREADS) sh.qloc[k] = 0.f;
-    if (tid == 0) {
-        sh.tok = 0x7fffffff;
-        sh.last = -1;
+    float l[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int v = v0 + tid * 4 + e;
+        l[e] = v < a.V ? load_logit(row, v - vbase) : -CUDART_INF_F;
     }
-    __syncthreads();
-    if (use_resid)
+    if (use_resid) {
         for (int k = tid; k < n; k += THREADS) {
             const int v = idx[k];
             if (v >= v0 && v < v0 + CHUNK) sh.qloc[v - v0] = prob[k];
         }
-    __syncthreads();
+        __syncthreads();
+    }
+    const float4 ql = *reinterpret_cast<const float4*>(&sh.qloc[tid * 4]);
+    const float qv[4] = {ql.x, ql.y, ql.z, ql.w};
     double r[4], cum[4], qsum = 0.0, loc = 0.0;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const int v = v0 + tid * 4 + e;
-        double w = 0.0;
-        if (v < a.V) w = wt(load_logit(row, v - vbase)) * invZ;
-        const double q = (double)sh.qloc[tid * 4 + e];
+        const double w = v0 + tid * 4 + e < a.V ? wt(l[e]) * invZ : 0.0;
+        const double q = (double)qv[e];
         qsum += q;
-        double d = w - q;
+        const double d = w - q;
         r[e] = d > 0.0 ? d : 0.0;
         loc += r[e];
         cum[e] = loc;
     }
-    double M;
-    const double incl = block_scan_incl(loc, sh.warp_tot, M);
-    const double base = incl - loc;
-    double Q;
-    block_scan_incl(qsum, sh.warp_tot, Q);
+    // running sum of the weights and total of the stored probabilities
+    double incl = loc;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, incl, d);
+        incl += lane >= d ? y : 0.0;
+    }
+    qsum = use_resid ? warp_sum(qsum) : 0.0;
+    if (lane == 31) {
+        sh.warp_tot[warp] = incl;
+        sh.warp_q[warp] = qsum;
+    }
+    __syncthreads();
+    double M = 0.0, Q = 0.0, base = incl - loc;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) {
+        const double t = sh.warp_tot[w];
+        if (w < warp) base += t;
+        M += t;
+        Q += sh.warp_q[w];
+    }
     const double thr2 = (double)u2 * M;
     int mine = 0x7fffffff, mylast = -1;
 #pragma unroll
@@ -321,19 +374,35 @@ __device__ __forceinline__ int level2_draw(const VerifyArgs& a, const T* row, in
         if (base + cum[e] > thr2) mine = v0 + tid * 4 + e;
         if (r[e] > 0.0 && mylast < 0) mylast = v0 + tid * 4 + e;
     }
-    if (mine != 0x7fffffff) atomicMin(&sh.tok, mine);
-    if (mylast >= 0) atomicMax(&sh.last, mylast);
+    const int wfirst = __reduce_min_sync(0xffffffffu, mine), wlast = __reduce_max_sync(0xffffffffu, mylast);
+    if (lane == 0) {
+        sh.warp_first[warp] = wfirst;
+        sh.warp_last[warp] = wlast;
+    }
     __syncthreads();
-    const int token = sh.tok != 0x7fffffff ? sh.tok : sh.last;
+    int first = 0x7fffffff, last = -1;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) {
+        first = min(first, sh.warp_first[w]);
+        last = max(last, sh.warp_last[w]);
+    }
+    const int token = first != 0x7fffffff ? first : last;
     if (!PRECISE && use_resid && Q > 0.0) {
         // with q~ present the thresholds depend on the normaliser: error <= GUARD_Z * Q
         const double E2 = 2.0 * GUARD_Z * Q;
-        if (sh.tok == 0x7fffffff) {
+        if (first == 0x7fffffff) {
             if (tid == 0) sh.flag = 1;
-        } else if (mine == sh.tok) {
+        } else if (mine == first) {
             const int e = mine - (v0 + tid * 4);
-            const double hi = base + cum[e] - thr2;
-            const double lo = thr2 - (base + cum[e] - r[e]);
+            double at = 0.0, re = 0.0;
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (x == e) {
+                    at = base + cum[x];
+                    re = r[x];
+                }
+            const double hi = at - thr2;
+            const double lo = thr2 - (at - re);
             if (hi < E2 || lo < E2) sh.flag = 1;
         }
     }
@@ -341,9 +410,77 @@ __device__ __forceinline__ int level2_draw(const VerifyArgs& a, const T* row, in
     return token;
 }
 
+__device__ __forceinline__ void zero_qloc(FinishShared& sh) {
+    *reinterpret_cast<float4*>(&sh.qloc[threadIdx.x * 4]) = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+// bits lo .. hi - 1
+__device__ __forceinline__ unsigned long long bit_range(int lo, int hi) {
+    const unsigned long long below_hi = hi >= 64 ? ~0ull : (1ull << hi) - 1ull;
+    return lo >= 64 ? 0ull : below_hi & (~0ull << lo);
+}
+
+// Chunk masses of row j by the 256 threads of a CTA, into cm (a barrier follows); `entries`: with the stored
+// entries' shares taken out.  For the calls whose rows' masses do not all fit shared memory, and for
+// a residual that vanished.
+template <typename T, bool PRECISE, bool SHARDED>
+__device__ __noinline__ void chunk_masses(const VerifyArgs& a, FinishShared& sh, double* cm, int b, int j, bool exact,
+                                          bool entries, int n) {
+    const int G1 = a.G + 1, tid = threadIdx.x, rj = b * a.G + j;
+    const float Tb = a.temperature[b];
+    const float c32 = temp_scale(Tb);
+    const double invZ = 1.0 / sh.Z[j];
+    // at most 1024 entries, four per thread: their logits are under way while the masses form
+    constexpr int PER = MAX_K / THREADS;
+    const T* row = reinterpret_cast<const T*>(a.logits) + (long long)(b * G1 + j) * a.row_stride;
+    int vv[PER];
+    float qq[PER], ll[PER];
+    if (!entries) n = 0;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int k = tid + u * THREADS;
+        vv[u] = k < n ? a.q_idx[(long long)rj * a.k_max + k] : -2;
+        qq[u] = k < n ? a.q_prob[(long long)rj * a.k_max + k] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const bool ok = vv[u] >= 0 && vv[u] < a.V;
+        if (vv[u] != -2 && !ok) atomicOr(&sh.bad, (int)ST_RANGE);
+        ll[u] = ok ? (SHARDED ? a.entry_logits[(long long)rj * (a.k_max + 1) + tid + u * THREADS] : load_logit(row, vv[u]))
+                   : -CUDART_INF_F;
+    }
+    if (exact) {
+        for (int c = tid; c < a.nch; c += THREADS) cm[c] = a.dsum[record_index(a, b * G1 + j, c)] * invZ;
+    } else {
+        const double off = (double)__fmul_rn(sh.mx[j], c32);
+        const double scale = 1.0 / sh.Zraw[j];
+        for (int c = tid; c < a.nch; c += THREADS) {
+            const float2 v = a.stats[record_index(a, b * G1 + j, c)];
+            cm[c] = v.x > -CUDART_INF_F ? (double)v.y * exp2_call((double)__fmul_rn(v.x, c32) - off) * scale : 0.0;
+        }
+    }
+    __syncthreads();
+    if (!entries) return;
+    Weight<PRECISE> wt;
+    wt.init(Tb, sh.mx[j]);
+    double w[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) w[u] = wt.inlined(ll[u]);
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (vv[u] >= 0 && vv[u] < a.V) atomicAdd(&cm[vv[u] / CHUNK], -fmin(w[u] * invZ, (double)qq[u]));
+    __syncthreads();
+}
+
 // One sequence (fast pass: sequence `slot`; double-precision pass: entry `slot` of the queue), by the
-// 256 threads of a CTA.  cm: [nch] doubles of shared memory (chunk masses of the sampled row).
+// 256 threads of a CTA.  cm: shared memory for the chunk masses: of every row that is read ([rows, nch]
+// doubles) if a.cm_rows, else of the sampled row alone.
 // SHARDED: vocabulary-parallel verification (a.entry_logits and a.pick are set).
+//
+// Bound by latency: a chain of loads, double-precision arithmetic and (since a CTA runs through the code
+// once) instruction fetches.  Hence the order: all that does not depend on the streaming pass -- the
+// stored entries and the logits at them -- is read before the kernel waits for that pass; a warp takes
+// a row from its statistics through its test and leaves the row's chunk masses, with the entries'
+// shares taken out, in shared memory, so that the draw starts from them whichever row it falls on.
 template <typename T, bool PRECISE, bool SHARDED>
 __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot, FinishShared& sh, double* cm) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -360,6 +497,7 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
         const unsigned long long need = PRECISE ? a.need_rows[b] : 0ull;   // rows with exact chunk sums
         if (!a.sample_only && a.state_in && a.state_in[b] == 0) {
             // decided by an earlier call: nothing of this sequence is read or written
+            grid_dependency_sync();
             if (tid == 0 && a.state_out) a.state_out[b] = 0;
             return;
         }
@@ -368,8 +506,6 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
         const T* seq = reinterpret_cast<const T*>(a.logits) + (long long)b * G1 * a.row_stride;
         unsigned st_bits = 0;
         if (!temp_ok(Tb)) st_bits |= ST_TEMPERATURE;
-        // (requested now, looked at when the outputs are written)
-        const unsigned status_word = *(volatile unsigned*)a.status;
         // the two uniforms of the draw, requested long before the chunk masses are ready
         const float u_chunk = a.u_resample ? a.u_resample[2 * b] : 0.f;
         const float u_entry = a.u_resample ? a.u_resample[2 * b + 1] : 0.f;
@@ -379,28 +515,67 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
         if (g < 0 || g > G || g < lo) st_bits |= ST_RANGE;
         const int hi = a.sample_only ? G : min(g, a.r1);
         const int row_hi = a.sample_only ? G1 : min(g + 1, a.r1);
-        __syncthreads();
-        if (tid == 0) {
-            sh.bad = 0;
-            sh.flag = 0;
-        }
-        __syncthreads();
-
-        // ---- 1. normaliser of every row that is needed ------------------------------------
         int jpos = -1;
         if (a.sample_only) {
             jpos = a.pos[b];
             if (jpos < 0 || jpos > G) st_bits |= ST_RANGE;
         }
+        const int i_lo = a.sample_only ? jpos : lo, i_hi = a.sample_only ? jpos + 1 : row_hi;
+        __syncthreads();        // (the sequence before is done with the shared state)
+        if (tid == 0) {
+            sh.bad = 0;
+            sh.flag = 0;
+        }
+        if (!SHARDED) zero_qloc(sh);
+        __syncthreads();
+
+        // ---- 1. a warp per row: the normaliser; for a draft position p(x), q~(x), accept test,
+        // ----    residual mass
         if (!st_bits) {
-            const int i_lo = a.sample_only ? jpos : lo, i_hi = a.sample_only ? jpos + 1 : row_hi;
             for (int i = i_lo + warp; i < i_hi; i += WARPS) {
                 if (draw_only && i != alen_fast) continue;
                 if (mass_only && !row_needed(need, i)) continue;
+                const bool tested = !a.sample_only && !draw_only && i < hi;
+                const bool entries = tested || (a.cm_rows && (a.sample_only ? i < G : i < hi));
+                const int ri = b * G + (entries ? i : 0);
+                const int* idx = a.q_idx + (long long)ri * a.k_max;
+                const float* prob = a.q_prob + (long long)ri * a.k_max;
+                const T* row = seq + (long long)i * a.row_stride;
+                const float* ent = SHARDED ? a.entry_logits + (long long)ri * (a.k_max + 1) : nullptr;
+                // the first batch of stored entries is requested before the row's count is known
+                // (every slot below k_max exists; slots at or beyond the count are dropped below)
+                int vv[8], x = -1, n = 0;
+                float qq[8], ll[8], ux = 0.f, lx = -CUDART_INF_F;
+                bool range_bad = false;
+                if (entries) {
+                    n = a.q_count[ri];
+                    if (tested) {
+                        x = a.draft_tok[ri];
+                        ux = a.u_accept[ri];
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int k = u * 32 + lane;
+                        vv[u] = k < a.k_max ? idx[k] : -2;
+                        qq[u] = k < a.k_max ? prob[k] : 0.f;
+                    }
+                    range_bad = n < 0 || n > a.k_max || (tested && (x < 0 || x >= a.V));
+                    // p(x) on every lane (the same instructions as on one lane, and no divergent tail)
+                    if (tested && !range_bad) lx = SHARDED ? ent[a.k_max] : load_logit(row, x);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int k = u * 32 + lane;
+                        if (k >= n || range_bad) vv[u] = -2;
+                        const bool ok = vv[u] >= 0 && vv[u] < a.V;
+                        ll[u] = ok ? (SHARDED ? ent[k] : load_logit(row, vv[u])) : -CUDART_INF_F;
+                    }
+                }
+                grid_dependency_sync();
                 double Z, Zraw;
                 float mx;
                 bool bad;
-                row_stats<T>(a, b * G1 + i, c32, lane, PRECISE && row_needed(need, i), Z, Zraw, mx, bad);
+                double* masses = a.cm_rows ? cm + (long long)(i - i_lo) * a.nch : nullptr;
+                row_stats<T>(a, b * G1 + i, c32, lane, PRECISE && row_needed(need, i), Z, Zraw, mx, bad, masses);
                 if (lane == 0) {
                     sh.Z[i] = Z;
                     sh.Zraw[i] = Zraw;
@@ -408,87 +583,87 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                     if (!PRECISE) a.row_max[b * G1 + i] = mx;
                     if (bad) atomicOr(&sh.bad, (int)ST_LOGIT);
                 }
-            }
-        }
-        __syncthreads();
-
-        // ---- 2. per draft position: p(x), q~(x), accept test, residual mass ----------------
-        if (!st_bits && !sh.bad && !a.sample_only && !draw_only) {
-            for (int i = lo + warp; i < hi; i += WARPS) {
-                if (mass_only && !row_needed(need, i)) continue;
-                const int ri = b * G + i;
-                const int* idx = a.q_idx + (long long)ri * a.k_max;
-                const float* prob = a.q_prob + (long long)ri * a.k_max;
-                const T* row = seq + (long long)i * a.row_stride;
-                // the first batch of stored entries is requested before the row's count is known
-                // (every slot below k_max exists; slots at or beyond the count are dropped below)
-                int vv[8];
-                float qq[8], ll[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int k = u * 32 + lane;
-                    vv[u] = k < a.k_max ? idx[k] : -2;
-                    qq[u] = k < a.k_max ? prob[k] : 0.f;
-                }
-                const int x = a.draft_tok[ri];
-                const int n = a.q_count[ri];
-                const float ux = a.u_accept[ri];
-                bool range_bad = (x < 0 || x >= a.V || n < 0 || n > a.k_max);
+                if (!entries || bad) continue;
                 Weight<PRECISE> wt;
-                wt.init(Tb, sh.mx[i]);
-                const double Z = sh.Z[i];
+                wt.init(Tb, mx);
                 const double invZ = 1.0 / Z;     // the sums below take p = w * (1/Z): 2^-53 relative per term
                 double smin = 0.0;
-                float qx = 0.f, qx_mine = 0.f;
+                float qx_mine = 0.f;
                 int kx = 0x7fffffff;
-                // p(x) on every lane (the same instructions as on one lane, and no divergent tail)
-                const float* ent = SHARDED ? a.entry_logits + (long long)ri * (a.k_max + 1) : nullptr;
-                const float lx = range_bad ? -CUDART_INF_F : (SHARDED ? ent[a.k_max] : load_logit(row, x));
-                if (!range_bad) {
-                    for (int k0 = 0; k0 < n; k0 += 256) {
-                        if (k0 > 0) {
+                const int n_read = range_bad ? 0 : n;
+                // entry k (v, q) with the logit l: its share of the residual; the weight w = exp(l/T - mx/T)
+                auto take = [&](int k, int v, float q, double w) {
+                    const bool ok = v >= 0 && v < a.V;
+                    if (v != -2 && !ok) range_bad = true;
+                    if (ok) {
+                        const double d = fmin(w * invZ, (double)q);
+                        smin += d;
+                        if (masses) atomicAdd(&masses[v / CHUNK], -d);
+                        if (v == x && k < kx) {
+                            kx = k;
+                            qx_mine = q;
+                        }
+                    }
+                };
+                if (n_read <= 64) {
+                    // few entries: one copy of the body (see exp_call)
+#pragma unroll 1
+                    for (int k0 = 0; k0 < n_read; k0 += 32) {
+                        take(k0 + lane, vv[0], qq[0], wt(ll[0]));
+                        vv[0] = vv[1];
+                        qq[0] = qq[1];
+                        ll[0] = ll[1];
+                        __syncwarp();
+                    }
+                } else {
+                    // many: four exponentials in flight
+#pragma unroll 1
+                    for (int k0 = 0; k0 < n_read; k0 += 128) {
+                        if ((k0 & 255) == 0 && k0 > 0) {
+                            // the next 256 entries, loads first
 #pragma unroll
                             for (int u = 0; u < 8; ++u) {
                                 const int k = k0 + u * 32 + lane;
                                 vv[u] = k < n ? idx[k] : -2;
                                 qq[u] = k < n ? prob[k] : 0.f;
                             }
-                        }
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            if (k0 + u * 32 + lane >= n) vv[u] = -2;
-                            const bool ok = vv[u] >= 0 && vv[u] < a.V;
-                            if (vv[u] != -2 && !ok) range_bad = true;
-                            ll[u] = ok ? (SHARDED ? ent[k0 + u * 32 + lane] : load_logit(row, vv[u])) : -CUDART_INF_F;
-                        }
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int k = k0 + u * 32 + lane;
-                            if (vv[u] >= 0 && vv[u] < a.V) {
-                                const double pk = wt(ll[u]) * invZ;
-                                smin += fmin(pk, (double)qq[u]);
-                                if (vv[u] == x && k < kx) {
-                                    kx = k;
-                                    qx_mine = qq[u];
-                                }
+                            for (int u = 0; u < 8; ++u) {
+                                const bool ok = vv[u] >= 0 && vv[u] < a.V;
+                                ll[u] = ok ? (SHARDED ? ent[k0 + u * 32 + lane] : load_logit(row, vv[u])) : -CUDART_INF_F;
                             }
                         }
+                        double w[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) w[u] = wt.inlined(ll[u]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) take(k0 + u * 32 + lane, vv[u], qq[u], w[u]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            vv[u] = vv[u + 4];
+                            qq[u] = qq[u + 4];
+                            ll[u] = ll[u + 4];
+                        }
+                        __syncwarp();
                     }
+                }
+                if (!tested) {
+                    if (__any_sync(0xffffffffu, range_bad) && lane == 0) atomicOr(&sh.bad, (int)ST_RANGE);
+                    continue;
                 }
                 const double px = wt(lx) / Z;
                 range_bad = __any_sync(0xffffffffu, range_bad);
                 smin = warp_sum(smin);
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) kx = min(kx, __shfl_xor_sync(0xffffffffu, kx, d));
+                kx = __reduce_min_sync(0xffffffffu, kx);
                 // the stored probability of the first entry that names the draft token sits in lane kx % 32
-                qx = __shfl_sync(0xffffffffu, qx_mine, kx & 31);
+                float qx = __shfl_sync(0xffffffffu, qx_mine, kx & 31);
                 if (kx == 0x7fffffff) qx = 0.f;
                 if (lane == 0) {
                     if (range_bad) {
                         atomicOr(&sh.bad, (int)ST_RANGE);
                     } else {
                         const double u = (double)ux;
-                        int acc = 1, amb = 0, bord = 0;
+                        bool acc = true, amb = false, bord = false;
                         if (qx > 0.f) {
                             const double ratio = px / (double)qx;
                             acc = u < fmin(1.0, ratio);
@@ -498,47 +673,56 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                             else
                                 amb = dist <= (BORDER_REL + GUARD_Z) * fmax(u, ratio);
                         }
-                        sh.acc[i] = acc;
-                        sh.amb[i] = amb;
-                        sh.bord[i] = bord;
                         double R = 1.0 - smin;
                         if (R < 0.0) R = 0.0;
                         // 1 - sum min(p, q~) inherits the absolute error of the fp32-accumulated
                         // normaliser: a small residual mass is reported from the exact sums instead
-                        sh.small[i] = !PRECISE && R < RESID_EXACT_BELOW;
+                        const bool small = !PRECISE && R < RESID_EXACT_BELOW;
+                        sh.test[i] = (unsigned char)((acc ? TEST_ACC : 0) | (amb ? TEST_AMB : 0) | (bord ? TEST_BORD : 0) |
+                                                     (small ? TEST_SMALL : 0));
                         a.p_draft[ri] = (float)px;
                         a.resid_mass[ri] = (float)R;
                     }
                 }
             }
         }
+        grid_dependency_sync();
+        // (requested now, looked at when the outputs are written)
+        const unsigned status_word = *(volatile unsigned*)a.status;
         __syncthreads();
         st_bits |= (unsigned)sh.bad;
         if (mass_only) return;          // (bad data was reported by the fast pass already)
 
-        // ---- 3. first-rejection scan -----------------------------------------------------
+        // ---- 2. first-rejection scan -----------------------------------------------------
         // A rejection inside the range decides the sequence; so does accepting every position
         // when the bonus row g is in the range.  Otherwise it waits for the next rows.
-        int alen = lo, nborder = 0;
+        int alen = lo, nborder = 0, first_amb = -1;
         bool flagged = false, rejected = false, decided = true;
+        unsigned long long small_rows = 0ull;
         if (draw_only) {
             // (no accept test was ambiguous, so none is borderline either)
             alen = alen_fast;
             rejected = alen < hi;
         } else if (!st_bits && !a.sample_only) {
-            while (alen < hi && sh.acc[alen]) ++alen;
-            rejected = alen < hi;
+            const int t0 = lane >= lo && lane < hi ? sh.test[lane] : TEST_ACC;
+            const int t1 = lane + 32 >= lo && lane + 32 < hi ? sh.test[lane + 32] : TEST_ACC;
+            auto bits = [&](int which) {
+                return (unsigned long long)__ballot_sync(0xffffffffu, t0 & which) |
+                       (unsigned long long)__ballot_sync(0xffffffffu, t1 & which) << 32;
+            };
+            const unsigned long long refused = ~bits(TEST_ACC);
+            rejected = refused != 0ull;
+            alen = rejected ? __ffsll((long long)refused) - 1 : hi;
             decided = rejected || g < a.r1;
-            const int last = rejected ? alen : hi - 1;
-            for (int i = lo; i <= last; ++i) {
-                flagged |= sh.amb[i] != 0;
-                nborder += sh.bord[i];
-            }
-            if (!PRECISE)
-                for (int i = lo; i < hi; ++i) flagged |= sh.small[i] != 0;
+            const unsigned long long seen = bit_range(lo, rejected ? alen + 1 : hi);     // every decision that counts
+            if (PRECISE) nborder = __popcll(bits(TEST_BORD) & seen);
+            const unsigned long long amb = bits(TEST_AMB) & seen;
+            if (amb) first_amb = __ffsll((long long)amb) - 1;
+            small_rows = bits(TEST_SMALL);
+            flagged = amb != 0ull || small_rows != 0ull;
         }
 
-        // ---- 4. residual / bonus sample --------------------------------------------------
+        // ---- 3. residual / bonus sample --------------------------------------------------
         int token = -1;
         int pick_row = 0, pick_chunk = -1;      // vocabulary-parallel: what the picked chunk's owner needs
         bool pick_resid = false;
@@ -547,108 +731,57 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
         if (!st_bits && want_token && decided) {
             const int j = a.sample_only ? jpos : alen;
             const int rj = b * G + j;
-            int n = 0;
-            if (a.sample_only ? j < G : rejected) {
-                n = a.q_count[rj];
-                if (n < 0 || n > a.k_max) {
-                    n = 0;
-                    st_bits |= ST_RANGE;
-                }
+            int n = (a.sample_only ? j < G : rejected) ? a.q_count[rj] : 0;
+            if (n < 0 || n > a.k_max) {
+                n = 0;
+                st_bits |= ST_RANGE;
             }
             const int* idx = a.q_idx + (long long)rj * a.k_max;
             const float* prob = a.q_prob + (long long)rj * a.k_max;
             const T* row = seq + (long long)j * a.row_stride;
-            Weight<PRECISE> wt;
-            wt.init(Tb, sh.mx[j]);
-            const double Z = sh.Z[j];
-            const double invZ = 1.0 / Z;
+            const bool exact = PRECISE && row_needed(need, j);
             bool use_resid = n > 0;
+            int cstar = -1;
+            double* mj = cm;
+            if (a.cm_rows) mj = cm + (long long)(j - i_lo) * a.nch;
+            else chunk_masses<T, PRECISE, SHARDED>(a, sh, cm, b, j, exact, use_resid, n);
+            st_bits |= (unsigned)sh.bad;
             for (int pass = 0; pass < 2 && !st_bits; ++pass) {
-                // chunk masses (in units where the row sums to one)
-                if (PRECISE && row_needed(need, j)) {
-                    for (int c = tid; c < a.nch; c += THREADS) cm[c] = a.dsum[record_index(a, b * G1 + j, c)] * invZ;
-                } else {
-                    const double off = (double)__fmul_rn(sh.mx[j], c32);
-                    const double Zraw = sh.Zraw[j];
-                    for (int c = tid; c < a.nch; c += THREADS) {
-                        float2 v = a.stats[record_index(a, b * G1 + j, c)];
-                        cm[c] = v.x > -CUDART_INF_F ? (double)v.y * exp2((double)__fmul_rn(v.x, c32) - off) / Zraw : 0.0;
-                    }
+                // level 1, by every warp for itself: lanes own contiguous blocks of chunks
+                const int per = (a.nch + 31) / 32;
+                const int c0 = lane * per;
+                double s = 0.0;
+#pragma unroll 1
+                for (int c = c0; c < c0 + per; ++c)
+                    if (c < a.nch) s += fmax(mj[c], 0.0);
+                __syncwarp();
+                double incl = s;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const double y = __shfl_up_sync(0xffffffffu, incl, d);
+                    incl += lane >= d ? y : 0.0;
                 }
-                __syncthreads();
-                if (use_resid) {
-                    bool rb = false;
-                    {
-                        // n <= 1024: at most four entries per thread, loads first
-                        int vv[4];
-                        float qq[4], ll[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int k = tid + u * THREADS;
-                            vv[u] = k < n ? idx[k] : -2;
-                            qq[u] = k < n ? prob[k] : 0.f;
-                        }
-                        const float* ent = SHARDED ? a.entry_logits + (long long)rj * (a.k_max + 1) : nullptr;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const bool ok = vv[u] >= 0 && vv[u] < a.V;
-                            if (vv[u] != -2 && !ok) rb = true;
-                            ll[u] = ok ? (SHARDED ? ent[tid + u * THREADS] : load_logit(row, vv[u])) : -CUDART_INF_F;
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (vv[u] >= 0 && vv[u] < a.V)
-                                atomicAdd(&cm[vv[u] / CHUNK], -fmin(wt(ll[u]) * invZ, (double)qq[u]));
-                    }
-                    if (rb) atomicOr(&sh.bad, (int)ST_RANGE);
-                }
-                __syncthreads();
-                // level 1 by warp 0: lanes own contiguous blocks of chunks
-                if (warp == 0) {
-                    const int per = (a.nch + 31) / 32;
-                    const int c0 = lane * per, c1 = min(a.nch, c0 + per);
-                    double s = 0.0;
-                    for (int c = c0; c < c1; ++c) {
-                        double m = cm[c];
-                        if (m < 0.0) {
-                            m = 0.0;
-                            cm[c] = 0.0;
-                        }
-                        s += m;
-                    }
-                    double incl = s;
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        double y = __shfl_up_sync(0xffffffffu, incl, d);
-                        if (lane >= d) incl += y;
-                    }
-                    const double R = __shfl_sync(0xffffffffu, incl, 31);
-                    const double thr = (double)u_chunk * R;
-                    double run = incl - s;
-                    int first = 0x7fffffff, lastpos = -1;
-                    double mind = 1e300;
-                    for (int c = c0; c < c1; ++c) {
-                        const double m = cm[c];
+                Rtot = __shfl_sync(0xffffffffu, incl, 31);
+                const double thr = (double)u_chunk * Rtot;
+                double run = incl - s;
+                int first = 0x7fffffff, lastpos = -1;
+                bool close = false;
+#pragma unroll 1
+                for (int c = c0; c < c0 + per; ++c) {
+                    if (c < a.nch) {
+                        const double m = fmax(mj[c], 0.0);
                         run += m;
                         if (m > 0.0) lastpos = c;
-                        if (run > thr && first == 0x7fffffff) first = c;
-                        mind = fmin(mind, fabs(run - thr));
-                    }
-#pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) {
-                        first = min(first, __shfl_xor_sync(0xffffffffu, first, d));
-                        lastpos = max(lastpos, __shfl_xor_sync(0xffffffffu, lastpos, d));
-                        mind = fmin(mind, __shfl_xor_sync(0xffffffffu, mind, d));
-                    }
-                    if (lane == 0) {
-                        sh.cstar = first != 0x7fffffff ? first : lastpos;
-                        sh.Rtot = R;
+                        if (run > thr) first = min(first, c);
                         // every prefix and the total carry an absolute error <= GUARD_Z
-                        if (!PRECISE && mind <= GUARD_Z) sh.flag = 1;
+                        close |= fabs(run - thr) <= GUARD_Z;
                     }
                 }
-                __syncthreads();
-                Rtot = sh.Rtot;
+                __syncwarp();
+                first = __reduce_min_sync(0xffffffffu, first);
+                lastpos = __reduce_max_sync(0xffffffffu, lastpos);
+                cstar = first != 0x7fffffff ? first : lastpos;
+                if (!PRECISE && __any_sync(0xffffffffu, close) && tid == 0) sh.flag = 1;
                 if (!use_resid) break;
                 // the residual may vanish (q~ >= p everywhere): then the draw is from p itself
                 const double tiny = PRECISE ? RESID_ZERO_BELOW : 4.0 * GUARD_Z;
@@ -661,20 +794,21 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                 }
                 use_resid = false;  // precise: residual is zero, fall back to p
                 __syncthreads();
+                mj = cm;
+                chunk_masses<T, PRECISE, SHARDED>(a, sh, cm, b, j, exact, false, 0);
             }
-            st_bits |= (unsigned)sh.bad;
-            const int cs = st_bits ? -1 : sh.cstar;
             pick_row = j;
-            pick_chunk = cs;
+            pick_chunk = cstar;
             pick_resid = use_resid;
-            if (!st_bits && cs >= 0 && !SHARDED) {
-                token = level2_draw<T, PRECISE>(a, row, 0, cs, idx, prob, n, use_resid, wt, invZ,
-                                                u_entry, sh);
+            if (cstar >= 0 && !st_bits && !SHARDED) {
+                Weight<PRECISE> wt;
+                wt.init(Tb, sh.mx[j]);
+                token = level2_draw<T, PRECISE>(a, row, 0, cstar, idx, prob, n, use_resid, wt, 1.0 / sh.Z[j], u_entry, sh);
             }
             flagged |= sh.flag != 0;
         }
 
-        // ---- 5. outputs --------------------------------------------------------------------
+        // ---- 4. outputs --------------------------------------------------------------------
         // a wait of the streaming pass ran out (now or in a call since the status word was last
         // cleared): its statistics are not complete, nothing of this call is valid
         if (status_word & ST_INTERNAL) st_bits |= ST_INTERNAL;
@@ -722,24 +856,22 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                         nrows = 1;
                         a.rowq[atomicAdd(a.rowq_count, 1)] = b * G1 + jpos;
                     } else {
-                        int first_amb = -1;
-                        const int last = rejected ? alen : hi - 1;
-                        for (int i = lo; i <= last && first_amb < 0; ++i)
-                            if (sh.amb[i]) first_amb = i;
-                        bool any_small = false;
-                        for (int i = lo; i < hi; ++i) any_small |= sh.small[i] != 0;
+                        const bool any_small = small_rows != 0ull;
                         draw_only_flag = first_amb < 0 && !any_small;
                         mass_only_flag = first_amb < 0 && any_small && !sh.flag;
-                        for (int i = lo; i < row_hi; ++i) {
-                            // (vocabulary-parallel: whether the draw inside the chunk is too close to call is
-                            // only known to the chunk's owner later, so the sampled row is always listed)
-                            const bool nr = i >= 64 || (first_amb >= 0 && i >= first_amb) || (i < hi && sh.small[i]) ||
-                                            ((sh.flag || SHARDED) && want_token && decided && i == alen);
-                            if (nr) {
-                                if (i < 64) nd |= 1ull << i;
-                                ++nrows;
-                                if (!SHARDED) a.rowq[atomicAdd(a.rowq_count, 1)] = b * G1 + i;
-                            }
+                        nd = small_rows;
+                        if (first_amb >= 0) nd |= ~0ull << first_amb;
+                        // (vocabulary-parallel: whether the draw inside the chunk is too close to call is
+                        // only known to the chunk's owner later, so the sampled row is always listed)
+                        if ((sh.flag || SHARDED) && want_token && decided && alen < 64) nd |= 1ull << alen;
+                        nd &= bit_range(lo, row_hi);
+                        const bool row64 = row_hi > 64;         // (row 64 has no bit: it always counts as listed)
+                        nrows = __popcll(nd) + (row64 ? 1 : 0);
+                        if (!SHARDED && nrows > 0) {
+                            int at = atomicAdd(a.rowq_count, nrows);
+                            for (unsigned long long left = nd; left; left &= left - 1ull)
+                                a.rowq[at++] = b * G1 + __ffsll((long long)left) - 1;
+                            if (row64) a.rowq[at] = b * G1 + 64;
                         }
                     }
                     a.need_rows[b] = nd;
@@ -762,12 +894,16 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
 }
 
 template <typename T, bool PRECISE, bool SHARDED = false>
-__global__ void __launch_bounds__(THREADS, 2) verify_finish_kernel(VerifyArgs a) {
-    extern __shared__ double cm[];  // [nch] chunk masses of the sampled row
+__global__ void __launch_bounds__(THREADS, 2) verify_finish_kernel(const __grid_constant__ VerifyArgs a) {
+    extern __shared__ double cm[];  // chunk masses: of every row that is read (a.cm_rows), or of the sampled one
     __shared__ FinishShared sh;
-    grid_dependency_sync();
+    // Only the chunk statistics / exact sums come from the kernel before this one; whatever was written
+    // before that kernel is visible as soon as this one runs, because that kernel let it start only after
+    // its own wait.  (The sharded form follows an exchange and waits at once.)
+    if (SHARDED) grid_dependency_wait();
     const int nloop = PRECISE ? *a.queue_count : a.B;
     for (int slot = blockIdx.x; slot < nloop; slot += gridDim.x) verify_finish_slot<T, PRECISE, SHARDED>(a, slot, sh, cm);
+    grid_dependency_sync();
 }
 
 }  // namespace picospec

@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(THREADS) vp_draw_kernel(VerifyArgs a, int v0, 
             sh.flag = 0;
             sbad = 0;
         }
+        zero_qloc(sh);
         __syncthreads();
         if (mine) {
             const float Tb = a.temperature[b];
