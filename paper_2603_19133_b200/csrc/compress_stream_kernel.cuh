@@ -1,35 +1,32 @@
 // Draft-side compression, staged variant: rows that hold at least one full tile.  Two kernels.
 //
-// compress_filter_kernel streams the rows (one CTA per row at a time, tiles of 8 chunks staged in
-// shared memory by bulk async copies; the producer lane runs ahead into the next row) and keeps
-// every element that can still be among the k largest:
-//   - the CTA holds a running lower bound `thr` on the k-th largest logit of the row;
+// compress_filter_kernel streams the rows (one CTA per row at a time, in tiles of 8 chunks, one per
+// warp, staged in shared memory by bulk async copies; the producer lanes run ahead into the next row)
+// and keeps every element that can still be among the k largest:
+//   - the CTA holds a running bound `thr` below which elements are dropped (how it is chosen, and which
+//     chunks make a tile: bound_rank);
 //   - per chunk a lane compares its 32 values with thr (packed compares for bf16) into a 32-bit
-//     mask; the warp then takes one set bit per lane per step, ranks the lanes by ballot and
-//     appends the values (64-bit keys: logit, then lower index first; the value is re-read from the
-//     staged tile) to the warp's own region of the candidate buffer: no atomics with a return
-//     value, no CTA barrier.  About 15 of the 1024 values of a chunk pass, so this is two or three
-//     steps per chunk;
+//     mask and appends the passing values (64-bit keys: logit, then lower index first; the value is
+//     re-read from the staged tile) to the warp's own region of the candidate buffer;
 //   - every stored candidate is counted in a two-level histogram whose bins count up from the
 //     first tile's bound, one bin per 16-bit logit code (the top 16 bits of the orderable key: a
 //     bf16 value, 2^-7 relative for fp32), magnitudes below 2^-10 sharing one bin on each side of
 //     zero so that a window that crosses zero does not spend itself on tiny exponents; 4096 bins
 //     reach 32 binades up, whatever lies beyond shares the last bin; thr is the lower edge of the
-//     highest bin whose suffix count reaches k, so it is a valid bound whenever it is computed,
-//     by any warp, from whatever has been counted so far.
+//     highest bin whose suffix count reaches the wanted rank.
 //     The warps take turns refreshing it, once per tile; a warp whose region fills refreshes it
 //     and drops its candidates below it;
-//   - the first tile of a row gets its bound without the histogram: every warp finds, by a
-//     16-step bisection over its own chunk, a value that at least ceil(k/8) of its small groups
-//     of elements reach with their maximum; the smallest of the eight values is reached by at
-//     least k elements of the tile (one CTA barrier, the only one inside a row);
-//   - a row whose candidates do not fit (heavy ties, adversarial order) is handed to the direct
-//     kernel through a redo list;
+//   - the first tile of a row gets its bound without the histogram: every warp finds a value that an
+//     eighth of the wanted rank of small groups of its elements reach with their maximum; the smallest
+//     of the eight values is reached by the wanted rank of elements (one CTA barrier, the only one
+//     inside a row);
+//   - a row whose candidates do not fit (heavy ties), or whose bound rose past its k-th largest, is
+//     handed to the direct kernel through a redo list;
 //   - with top-p the same pass accumulates the softmax normaliser relative to the first tile's
 //     maximum (a row whose later logits overflow that reference also goes to the redo list).
-// At the end of a row the candidates at or above thr (at least k; for 16-bit logits the k best plus
-// the ties of the k-th, for 32-bit logits plus what shares its 16-bit code) go to a per-row scratch
-// area in global memory, with the bound itself.
+// At the end of a row the candidates at or above thr (for 16-bit logits the k best plus the ties of the
+// k-th, for 32-bit logits plus what shares its 16-bit code) go to a per-row scratch area in global
+// memory, with the bound itself.
 //
 // compress_finish_kernel (a warp or a CTA per row) selects the k best of them and puts them in order
 // with a counting sort over the 16-bit logit codes, then calls finish_row (top-p cut,
@@ -323,9 +320,9 @@ __device__ __noinline__ int maintain_region(int wcount, int region_off, int hist
 // the CTAs read one window of memory that moves forward, as a copy would).  The rem rows that
 // are left would keep only some of the CTAs busy for a whole row's time, so each of them is cut into
 // `split` pieces of consecutive tiles and the rem * split pieces are dealt round-robin: piece n goes
-// to CTA n % grid.  A piece is filtered on its own: it keeps a bound that at least k of ITS elements
-// reach, which is a valid bound for the row, and leaves its survivors in its own scratch area (whole
-// row r: area r; tail piece n: area rows + n).  The finish kernel puts the pieces of a row together.
+// to CTA n % grid.  A piece is filtered on its own, with the bound of its share of the row
+// (bound_rank), and leaves its survivors in its own scratch area (whole row r: area r; tail piece n:
+// area rows + n).  The finish kernel puts the pieces of a row together.
 // No piece starts at a row's last tile when that tile is ragged (the first tile of a piece must be a
 // full one, up to the few entries that a row's offset from a 16-byte boundary takes from it).
 struct FilterPlan {
@@ -398,6 +395,29 @@ inline FilterPlan make_filter_plan(int rows, int tiles_per_row, bool ragged_last
     return p;
 }
 
+// ---- how far a bound may reach ahead -------------------------------------------------------------
+// A bound that k elements seen so far reach is certain, but while little of the row has been seen it
+// lets k / (tiles seen) elements of every tile pass, k (1 + ln tiles) in all, and handling those was most
+// of the kernel's instructions at large k.  The bound used is the value that
+//     rank(f) = 1.5 k f + 5 sqrt(1.5 k f) + 12        (at most k)
+// of the elements seen reach, f being the fraction of the row that has been seen: were the k largest spread
+// evenly over the tiles, it would be lower than the k-th largest by a factor 1.5 and five standard
+// deviations in the count.  A tile takes one chunk from each eighth of the row, so that rows whose large
+// logits crowd at one end are spread too.  It is not certain; it is checked: every element dropped
+// was below the final bound, so the row is right if k survivors reach that, and goes to the direct
+// kernel if not.  4096 rows of 262144 entries, k = 1024: 560 -> 473 us; 1536 rows of 128256, top-p with
+// k = 256: 116 -> 111 us; 512 rows of 151936, k = 128: 43 -> 40.7 us.
+__host__ __device__ __forceinline__ int bound_rank(int k, float f) {
+    const float e = 1.5f * (float)k * f;
+    const int r = (int)(e + 5.0f * sqrtf(e)) + 12;
+    return r < k ? r : k;
+}
+// Where one tile's rank is k already (small k) the tiles are contiguous instead: one copy of 16 KB a tile
+// (4096 rows of 32000 entries, k = 8: 69 us against 75 us with eight copies of 2 KB).
+__host__ __device__ __forceinline__ bool bound_spreads(int k, float per_tile) { return bound_rank(k, per_tile) < k; }
+// spread tiles: first of the chunks of a row of `nch` that warp w of the CTA streams
+__device__ __forceinline__ int warp_chunk0(int nch, int w) { return (int)(((long long)nch * w) >> 3); }
+
 // First-tile bound of one warp when it needs at most 32 elements (k <= 256): the lanes form at
 // least `need` groups of `group_lanes` lanes (a power of two); every group's largest value is
 // reached by one element of the group, so the smallest of the group maxima is reached by at least
@@ -431,10 +451,13 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
     if (k_eff > a.k_max) k_eff = a.k_max;
     if (k_eff > a.V) k_eff = a.V;
     const int surv_cap = cs_survivor_cap(a.k_max);
+    // (the fewest tiles that a row of V entries takes: a fraction that is too large only makes a bound lower)
+    const float per_tile = 1.0f / (float)((a.nch + TILE_CHUNKS - 1) / TILE_CHUNKS);
+    const bool spread = bound_spreads(k_eff, per_tile);
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], WARPS);
             mbar_init(&empty[s], WARPS);
         }
         mbar_init_fence();
@@ -452,8 +475,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
     __syncthreads();
 
     if (warp == WARPS) {
-        // ---- producer: every tile of every piece of this CTA, in order ---------------------------
-        if (lane != 0) return;
+        // ---- producer: every tile of every piece of this CTA, in order; a lane per chunk of the tile ----
+        if (lane >= WARPS) return;
         const uint64_t pol = l2_evict_first_policy();
         uint32_t i = 0;
         FilterPiece pc;
@@ -461,6 +484,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
             const long long srow = source_row(a, pc.row);
             // (a row with a bad temperature is copied for nothing: its workers look the temperature up)
             const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (srow < 0 ? 0 : srow) * a.row_stride, a.V);
+            const int row_chunks = (sr.end + CHUNK - 1) / CHUNK;
+            const int c0 = spread ? warp_chunk0(row_chunks, lane) : 0, c1 = spread ? warp_chunk0(row_chunks, lane + 1) : 0;
             for (int ti = pc.tile0; ti < pc.tile1; ++ti, ++i) {
                 const int s = (int)(i % STAGES);
                 const uint32_t round = i / STAGES;
@@ -469,8 +494,13 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     if (wr != WAIT_OK) atomicOr(a.status, ST_INTERNAL);
                     if (wr == WAIT_LOST) return;      // nothing more is issued
                 }
-                constexpr int GRANULES = TILE_BYTES / 16;
-                if (srow >= 0) stage_tile<T>(stage_mem + s * TILE_BYTES, sr, ti * GRANULES, GRANULES, &full[s], pol);
+                constexpr int GRANULES = CHUNK * (int)sizeof(T) / 16;
+                if (!spread) {
+                    if (srow >= 0 && lane == 0)
+                        stage_tile<T>(stage_mem + s * TILE_BYTES, sr, ti * (TILE_CHUNKS * GRANULES), TILE_CHUNKS * GRANULES, &full[s], pol);
+                } else if (srow >= 0 && c0 + ti < c1) {
+                    stage_tile<T>(stage_mem + s * TILE_BYTES + lane * (GRANULES * 16), sr, (c0 + ti) * GRANULES, GRANULES, &full[s], pol);
+                }
                 mbar_arrive(&full[s]);
             }
         }
@@ -481,15 +511,16 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
     u64* region = cand + warp * CS_REGION;
     const int region_off = (int)(reinterpret_cast<unsigned char*>(region) - dyn);
     const int hist_off = (int)(reinterpret_cast<unsigned char*>(hist) - dyn);
-    // first-tile bound.  k <= 128 (every warp needs at most 16 elements): from the lane maxima, over
-    // groups of two or more lanes.  Larger k: the exact need-th largest maximum of groups of g elements,
-    // at least 4 k groups in the tile (cheaper bounds from lane maxima or lane pairs let 10 to 25 % of
-    // a tile pass: the extra candidates cost more than the search).
-    const int need = (k_eff + WARPS - 1) / WARPS;
+    // first-tile bound.  Rank up to 128 (every warp needs at most 16 elements): from the lane maxima, over
+    // groups of two or more lanes.  Beyond (a k that is large for the row): the exact need-th largest maximum
+    // of groups of g elements, at least 4 rank groups in the tile (cheaper bounds from lane maxima or lane
+    // pairs let 10 to 25 % of a tile pass: the extra candidates cost more than the search).
+    const int rank1 = bound_rank(k_eff, per_tile);
+    const int need = (rank1 + WARPS - 1) / WARPS;
     int group_lanes = 1;
     while (2 * group_lanes * need <= 32) group_lanes <<= 1;
     int g = VEC;
-    while (g > 2 && (TILE_CHUNKS * CHUNK) / g < 4 * k_eff) g >>= 1;
+    while (g > 2 && (TILE_CHUNKS * CHUNK) / g < 4 * rank1) g >>= 1;
 
     bool dead = false;      // a wait ran out: this warp computes no more, but takes every tile and joins every barrier
     bool lost = false;      // a wait did not complete at all: the warp stops waiting as well
@@ -507,6 +538,9 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         // chunks are counted from the row's first granule here: which 1024 entries make one is no matter
         const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (in_range ? srow : 0) * a.row_stride, a.V);
         const int mis = sr.mis, end = sr.end;
+        const int row_chunks = (end + CHUNK - 1) / CHUNK;
+        const int c0 = spread ? warp_chunk0(row_chunks, warp) : warp;
+        const int c1 = spread ? warp_chunk0(row_chunks, warp + 1) : row_chunks;
         const bool valid = temp_ok(Tb) && in_range;
         const float c32 = temp_scale(Tb);
         float ref_off = 0.f, acc = 0.f;
@@ -528,8 +562,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     }
                 }
             }
-            const int c = ti * TILE_CHUNKS + warp;
-            const bool work = !dead && valid && !full_region && c * CHUNK < end;
+            const int c = spread ? c0 + ti : ti * TILE_CHUNKS + warp;
+            const bool work = !dead && valid && !full_region && c < c1;
             const unsigned char* chunk = stage_mem + s * TILE_BYTES + warp * (CHUNK * (int)sizeof(T));
             ChunkRegs<T> regs;
             if (work) load_staged(regs, chunk, c * CHUNK, end, lane);
@@ -538,7 +572,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 if (work) {
                     unsigned k16;
                     float wm = 0.f;
-                    if (SMALL && group_lanes >= 2) {
+                    if (group_lanes >= 2) {
                         const float lm = regs.lane_max_plain();
                         k16 = first_tile_key_groups(lm, group_lanes);
                         if (STATS) wm = warp_max_redux(lm);
@@ -572,7 +606,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 if (added) {
                     if (wcount + added > CS_REGION) {
                         // no room: bring the bound up to date and drop what fell below it
-                        wcount = maintain_region(wcount, region_off, hist_off, &cs, &cta.wcnt[warp], k_eff);
+                        wcount = maintain_region(wcount, region_off, hist_off, &cs, &cta.wcnt[warp],
+                                                 bound_rank(k_eff, per_tile * (float)(ti - pc.tile0 + 1)));
                         if (wcount + added > CS_REGION) {     // ties, a coarse bin too full, or a very loose bound
                             full_region = true;
                             mask = 0u;
@@ -611,7 +646,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 // latest values may not be counted yet, which only makes it a little lower)
                 if (warp == (ti & (WARPS - 1))) {
                     __syncwarp();
-                    refresh_bound(hist_off, &cs, k_eff);
+                    refresh_bound(hist_off, &cs, bound_rank(k_eff, per_tile * (float)(ti - pc.tile0 + 1)));
                 }
             }
         }
@@ -627,7 +662,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         unsigned thr_final = *(volatile unsigned*)&cs.thr_key;
         if (piece_ok) {
             // the final bound, by every warp for itself (all get the same): no second barrier for it
-            const int found = kth_bin(hist, k_eff, lane);
+            const int found = kth_bin(hist, bound_rank(k_eff, per_tile * (float)(pc.tile1 - pc.tile0)), lane);
             if (found >= 0) thr_final = max(thr_final, coord_code(g0 + found) << 16);
             // every warp filters its own region and appends to the piece's scratch area
             u64* dst = a.surv_keys + (long long)pc.area * surv_cap;
@@ -647,7 +682,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
             else if (!valid) flags = CSF_TEMPERATURE;
             else if (cs.overflow || m > surv_cap) flags = CSF_REDO;      // too many candidates or ties at the bound
             else if (cs.nan) flags = CSF_LOGIT;
-            else if (m < k_eff) flags = CSF_REDO;                        // cannot happen with a valid bound; be safe
+            else if (pc.tile1 - pc.tile0 == plan.tiles_per_row && m < k_eff) flags = CSF_REDO;   // the bound reached too far
             double zs = 0.0;
             if (STATS)
                 for (int w = 0; w < WARPS; ++w) zs += cs.wsum[w];
@@ -678,10 +713,10 @@ constexpr int CS_MAX_PIECES = 8;    // most pieces a row is dealt in
 //           bound, i.e. BINS / 128 binades for values away from zero; the last one is open-ended
 template <int TPR> struct FinishGeom;
 template <> struct FinishGeom<32> {
-    static constexpr int ROWS = 4, CAP = 512, KCAP = 128, BINS = 512, AHEAD = 4, CTAS = 7;
+    static constexpr int ROWS = 4, CAP = 512, KCAP = 128, BINS = 512, AHEAD = 4, HOLD = 4, CTAS = 7;
 };
 template <> struct FinishGeom<THREADS> {
-    static constexpr int ROWS = 1, CAP = 2 * MAX_K, KCAP = MAX_K, BINS = 2048, AHEAD = 2, CTAS = 6;
+    static constexpr int ROWS = 1, CAP = 2 * MAX_K, KCAP = MAX_K, BINS = 2048, AHEAD = 2, HOLD = 6, CTAS = 5;
 };
 template <int TPR> constexpr int finish_smem_bytes() {
     return FinishGeom<TPR>::ROWS * (FinishGeom<TPR>::CAP * 8 + FinishGeom<TPR>::KCAP * 8 + FinishGeom<TPR>::BINS * 4);
@@ -695,9 +730,8 @@ struct CsFinishShared {
 };
 
 // A row's survivors lie in one scratch area, or in those of its pieces if it was dealt in pieces.  A
-// survivor set holds all of a piece's elements at or above its final bound, i.e. its k best plus
-// whatever shares the bound's 16-bit code with the k-th; the largest of the pieces' bounds is a bound
-// for the row.  The k best are found and put in order by a counting sort over the 16-bit codes: count
+// survivor set holds all of a piece's elements at or above its final bound; the row's k best are among
+// the survivors if k of them reach the largest of the pieces' bounds.  The k best are found and put in order by a counting sort over the 16-bit codes: count
 // the keys per bin, sum from the top, move every key that is not below the bin of the k-th into its
 // bin's stretch, then place each by its rank among the keys of its own stretch (all pairs: a
 // stretch holds the ties of one code, a few keys).  Bound by latency for few rows (meta, survivors, six
@@ -710,7 +744,7 @@ template <typename T, bool STATS, int TPR>
 __global__ void __launch_bounds__(TPR * FinishGeom<TPR>::ROWS, FinishGeom<TPR>::CTAS)
 compress_finish_kernel(CompressArgs a, FilterPlan plan) {
     typedef FinishGeom<TPR> Geom;
-    constexpr int AHEAD = Geom::AHEAD, PER = Geom::BINS / TPR;
+    constexpr int AHEAD = Geom::AHEAD, HOLD = Geom::HOLD, PER = Geom::BINS / TPR;
     extern __shared__ __align__(16) unsigned char fin_mem[];
     __shared__ CsFinishShared shared[Geom::ROWS];
     const int tid = group_tid<TPR>(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -735,9 +769,9 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
     if (row >= plan.rows) return;       // (a warp beyond the last row)
     const u64* src = a.surv_keys + (long long)area0 * surv_cap;
     // the first area's first slots exist for every k_max: requested before their number is known
-    u64 ahead[AHEAD];
+    u64 held[HOLD];
 #pragma unroll
-    for (int x = 0; x < AHEAD; ++x) ahead[x] = src[x * TPR + tid];
+    for (int x = 0; x < AHEAD; ++x) held[x] = src[x * TPR + tid];
     const float Tb = a.temperature[row / a.G];
     // ---- the pieces, one per lane: flags, the row's bound, where each piece's survivors begin -------
     CsRowMeta meta;
@@ -773,15 +807,21 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
                 }
             return src[(long long)p * surv_cap + (i - b)];
         };
-        const int held = nareas == 1 ? AHEAD * TPR : 0;      // survivors the group holds in registers
+        // the first HOLD survivors of each thread stay in registers, those below the bound as zero
+#pragma unroll
+        for (int x = 0; x < HOLD; ++x) {
+            const int i = x * TPR + tid;
+            if (x >= AHEAD || nareas > 1) held[x] = i < m ? key_at(i) : 0ull;
+            if (i >= m || (unsigned)(held[x] >> 32) < thr_key) held[x] = 0ull;
+        }
         group_sync<TPR>();      // the bins are zero
         // ---- count ------------------------------------------------------------------------------
         auto bin_of = [&](u64 key) { return hist_bin_in<Geom::BINS>((unsigned)(key >> 32), g0); };
 #pragma unroll
-        for (int x = 0; x < AHEAD; ++x)
-            if (nareas == 1 && x * TPR + tid < m && (unsigned)(ahead[x] >> 32) >= thr_key) atomicAdd(&bins[bin_of(ahead[x])], 1);
+        for (int x = 0; x < HOLD; ++x)
+            if (held[x]) atomicAdd(&bins[bin_of(held[x])], 1);
 #pragma unroll 4
-        for (int i = held + tid; i < m; i += TPR) {
+        for (int i = HOLD * TPR + tid; i < m; i += TPR) {
             const u64 key = key_at(i);
             if ((unsigned)(key >> 32) >= thr_key) atomicAdd(&bins[bin_of(key)], 1);
         }
@@ -829,7 +869,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
             fs.kth = Geom::BINS - (tid + 1) * PER + x;
             if (end > Geom::CAP) fs.overflow = 1;         // too many ties with the k-th
         }
-        if (tid == TPR - 1 && live < k_eff) fs.overflow = 1;          // cannot happen with valid bounds; be safe
+        if (tid == TPR - 1 && live < k_eff) fs.overflow = 1;          // a piece's bound reached too far ahead
 #pragma unroll
         for (int x = 0; x < PER / 4; ++x) mine[x] = make_int4(cnt[4 * x], cnt[4 * x + 1], cnt[4 * x + 2], cnt[4 * x + 3]);
         group_sync<TPR>();
@@ -838,16 +878,17 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
             // ---- move: afterwards bins[b] is the end of bin b's stretch, which begins where bin b + 1's ends
             const int kth = fs.kth;
             auto move = [&](u64 key) {
-                if ((unsigned)(key >> 32) >= thr_key) {
-                    const int b = bin_of(key);
-                    if (b >= kth) stretch[atomicAdd(&bins[b], 1)] = key;
-                }
+                const int b = bin_of(key);
+                if (b >= kth) stretch[atomicAdd(&bins[b], 1)] = key;
             };
 #pragma unroll
-            for (int x = 0; x < AHEAD; ++x)
-                if (nareas == 1 && x * TPR + tid < m) move(ahead[x]);
+            for (int x = 0; x < HOLD; ++x)
+                if (held[x]) move(held[x]);
 #pragma unroll 4
-            for (int i = held + tid; i < m; i += TPR) move(key_at(i));
+            for (int i = HOLD * TPR + tid; i < m; i += TPR) {
+                const u64 key = key_at(i);
+                if ((unsigned)(key >> 32) >= thr_key) move(key);
+            }
             group_sync<TPR>();
             // ---- rank inside the stretch
             const int total = bins[kth];
@@ -856,6 +897,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
                 const int b = bin_of(key);
                 const int s0 = b + 1 < Geom::BINS ? bins[b + 1] : 0, s1 = bins[b];
                 int rank = s0;
+#pragma unroll 4
                 for (int x = s0; x < s1; ++x) rank += stretch[x] > key ? 1 : 0;
                 if (rank < k_eff) keys[rank] = key;         // keys are distinct: every rank is taken once
             }

@@ -213,7 +213,7 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
             // A warp per row while the row that has most survivors has few of them: a row dealt in 8 pieces
             // at k = 64 (560 survivors) took 15.9 us of a call by warps, 7.0 by CTAs; 4096 whole rows at
             // k = 8 take 9.1 us by warps and took 41 with a CTA and a sort network each.
-            const int survivors = plan.rem > 0 ? k_eff * plan.split : k_eff;
+            const int survivors = plan.rem > 0 ? plan.split * bound_rank(k_eff, 1.0f / (float)plan.split) : k_eff;
             if (survivors <= FinishGeom<32>::KCAP) launch_compress_finish<T, 32>(a, plan, stats, s);
             else launch_compress_finish<T, THREADS>(a, plan, stats, s);
         }

@@ -45,3 +45,43 @@ def test_select_and_order(rows, V, k, above, ties, binades, redo, dtype):
     for a, b in ((got[0], want[0]), (got[2], want[2]), (got[3], want[3])):
         assert np.array_equal(a, b)
     np.testing.assert_allclose(got[1], want[1], rtol=1e-5)
+
+
+@pytest.mark.parametrize("top_p", [1.0, 0.9])
+@pytest.mark.parametrize("rows,V,k,head,redo", [
+    (460, 65536, 256, 1.0 / 8, False),       # the large logits spread over the row (whole rows and pieces)
+    (5, 131072, 100, 0.6, False),            # six in ten of them in the first eighth
+    (5, 65536, 256, 1.0, False),             # all of them in the first eighth, spread over it
+    (5, 65536, 256, -1.0, True),             # all of them in 512 neighbouring entries: the bound rises past the k-th
+])
+def test_bound_ahead_of_the_rows_end(rows, V, k, head, redo, top_p):
+    # where the k largest lie must not show in the result, only in whether the direct kernel is needed
+    import paper_2603_19133_b200 as ps
+    g = torch.Generator(device="cuda").manual_seed(rows + V + k)
+    dl = torch.randn((rows, 1, V), generator=g, device="cuda").clamp_(max=3.9)
+    n = 2 * k
+    for r in range(rows):
+        if head < 0:
+            at = 1024 * (r % 3) + torch.randperm(n, generator=g, device="cuda")
+        else:
+            m = int(round(n * head))
+            first = torch.randperm(V // 8, generator=g, device="cuda")[:m]
+            rest = V // 8 + torch.randperm(V - V // 8, generator=g, device="cuda")[:n - m]
+            at = torch.cat([first, rest])
+        dl[r, 0, at] = 4.0 + 3.0 * torch.rand(n, generator=g, device="cuda")
+    dl = dl.to(torch.bfloat16)
+    T = torch.full((rows,), 0.8, device="cuda")
+    u = torch.rand((rows, 1), generator=g, device="cuda")
+    top_k = k if top_p >= 1.0 else 0
+    ctx = ps.Context(rows, 1, V, k)
+    try:
+        got = [t.cpu().numpy() for t in ctx.compress(dl, T, top_k, top_p, k, u)]
+        redone = ctx.counters(clear=True)[1]
+        assert ctx.status(clear=True)[0] == 0
+    finally:
+        ctx.close()
+    assert redone == (rows if redo else 0)
+    want = oracle.compress(dl.float().cpu().numpy(), T.cpu().numpy(), top_k, top_p, k, u.cpu().numpy(), nthreads=oracle.cores())
+    for a, b in ((got[0], want[0]), (got[2], want[2]), (got[3], want[3])):
+        assert np.array_equal(a, b)
+    np.testing.assert_allclose(got[1], want[1], rtol=1e-5)
