@@ -416,7 +416,7 @@ __host__ __device__ __forceinline__ int bound_rank(int k, float f) {
 // (4096 rows of 32000 entries, k = 8: 69 us against 75 us with eight copies of 2 KB).
 __host__ __device__ __forceinline__ bool bound_spreads(int k, float per_tile) { return bound_rank(k, per_tile) < k; }
 // spread tiles: first of the chunks of a row of `nch` that warp w of the CTA streams
-__device__ __forceinline__ int warp_chunk0(int nch, int w) { return (int)(((long long)nch * w) >> 3); }
+__device__ __forceinline__ int warp_chunk0(int nch, int w) { return (nch * w) >> 3; }
 
 // First-tile bound of one warp when it needs at most 32 elements (k <= 256): the lanes form at
 // least `need` groups of `group_lanes` lanes (a power of two); every group's largest value is
@@ -457,7 +457,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], WARPS);
+            mbar_init(&full[s], spread ? WARPS : 1);
             mbar_init(&empty[s], WARPS);
         }
         mbar_init_fence();
@@ -475,8 +475,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
     __syncthreads();
 
     if (warp == WARPS) {
-        // ---- producer: every tile of every piece of this CTA, in order; a lane per chunk of the tile ----
-        if (lane >= WARPS) return;
+        // ---- producer: every tile of every piece of this CTA, in order; a lane per copy of the tile ----
+        if (lane >= (spread ? WARPS : 1)) return;
         const uint64_t pol = l2_evict_first_policy();
         uint32_t i = 0;
         FilterPiece pc;
@@ -496,7 +496,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 }
                 constexpr int GRANULES = CHUNK * (int)sizeof(T) / 16;
                 if (!spread) {
-                    if (srow >= 0 && lane == 0)
+                    if (srow >= 0)
                         stage_tile<T>(stage_mem + s * TILE_BYTES, sr, ti * (TILE_CHUNKS * GRANULES), TILE_CHUNKS * GRANULES, &full[s], pol);
                 } else if (srow >= 0 && c0 + ti < c1) {
                     stage_tile<T>(stage_mem + s * TILE_BYTES + lane * (GRANULES * 16), sr, (c0 + ti) * GRANULES, GRANULES, &full[s], pol);
@@ -538,9 +538,11 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         // chunks are counted from the row's first granule here: which 1024 entries make one is no matter
         const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (in_range ? srow : 0) * a.row_stride, a.V);
         const int mis = sr.mis, end = sr.end;
-        const int row_chunks = (end + CHUNK - 1) / CHUNK;
+        // this warp's chunk of tile ti: c0 + ti * c_step, if below c1
+        const int row_chunks = (unsigned)(end + CHUNK - 1) / CHUNK;
         const int c0 = spread ? warp_chunk0(row_chunks, warp) : warp;
         const int c1 = spread ? warp_chunk0(row_chunks, warp + 1) : row_chunks;
+        const int c_step = spread ? 1 : TILE_CHUNKS;
         const bool valid = temp_ok(Tb) && in_range;
         const float c32 = temp_scale(Tb);
         float ref_off = 0.f, acc = 0.f;
@@ -562,7 +564,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     }
                 }
             }
-            const int c = spread ? c0 + ti : ti * TILE_CHUNKS + warp;
+            const int c = c0 + ti * c_step;
             const bool work = !dead && valid && !full_region && c < c1;
             const unsigned char* chunk = stage_mem + s * TILE_BYTES + warp * (CHUNK * (int)sizeof(T));
             ChunkRegs<T> regs;
@@ -646,7 +648,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 // latest values may not be counted yet, which only makes it a little lower)
                 if (warp == (ti & (WARPS - 1))) {
                     __syncwarp();
-                    refresh_bound(hist_off, &cs, bound_rank(k_eff, per_tile * (float)(ti - pc.tile0 + 1)));
+                    refresh_bound(hist_off, &cs, spread ? bound_rank(k_eff, per_tile * (float)(ti - pc.tile0 + 1)) : k_eff);
                 }
             }
         }
@@ -662,7 +664,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         unsigned thr_final = *(volatile unsigned*)&cs.thr_key;
         if (piece_ok) {
             // the final bound, by every warp for itself (all get the same): no second barrier for it
-            const int found = kth_bin(hist, bound_rank(k_eff, per_tile * (float)(pc.tile1 - pc.tile0)), lane);
+            const int found = kth_bin(hist, spread ? bound_rank(k_eff, per_tile * (float)(pc.tile1 - pc.tile0)) : k_eff, lane);
             if (found >= 0) thr_final = max(thr_final, coord_code(g0 + found) << 16);
             // every warp filters its own region and appends to the piece's scratch area
             u64* dst = a.surv_keys + (long long)pc.area * surv_cap;
@@ -716,7 +718,7 @@ template <> struct FinishGeom<32> {
     static constexpr int ROWS = 4, CAP = 512, KCAP = 128, BINS = 512, AHEAD = 4, HOLD = 4, CTAS = 7;
 };
 template <> struct FinishGeom<THREADS> {
-    static constexpr int ROWS = 1, CAP = 2 * MAX_K, KCAP = MAX_K, BINS = 2048, AHEAD = 2, HOLD = 6, CTAS = 5;
+    static constexpr int ROWS = 1, CAP = 2 * MAX_K, KCAP = MAX_K, BINS = 2048, AHEAD = 2, HOLD = 4, CTAS = 6;
 };
 template <int TPR> constexpr int finish_smem_bytes() {
     return FinishGeom<TPR>::ROWS * (FinishGeom<TPR>::CAP * 8 + FinishGeom<TPR>::KCAP * 8 + FinishGeom<TPR>::BINS * 4);
