@@ -418,14 +418,20 @@ __host__ __device__ __forceinline__ bool bound_spreads(int k, float per_tile) { 
 // spread tiles: first of the chunks of a row of `nch` that warp w of the CTA streams
 __device__ __forceinline__ int warp_chunk0(int nch, int w) { return (nch * w) >> 3; }
 
-// First-tile bound of one warp when it needs at most 32 elements (k <= 256): the lanes form at
-// least `need` groups of `group_lanes` lanes (a power of two); every group's largest value is
-// reached by one element of the group, so the smallest of the group maxima is reached by at least
-// `need` elements of the warp's chunk.  Returns its 16-bit orderable code (rounded down).
-__device__ __forceinline__ unsigned first_tile_key_groups(float lane_max, int group_lanes) {
-    unsigned key = orderable(lane_max) >> 16;
-    for (int d = 1; d < group_lanes; d <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, d));
-    return __reduce_min_sync(0xffffffffu, key);
+// First-tile bound of one warp when it needs at most 16 elements: the need-th largest of its 32 lanes'
+// maxima, as a 16-bit orderable code (rounded down).  (The smallest of the maxima of `need` groups of
+// lanes is cheaper and also certain, but now and then so low that a fifth of the tile passes and a
+// warp's region overflows: one row in five thousand at need = 15.)
+__device__ __forceinline__ unsigned first_tile_key_lanes(float lane_max, int need) {
+    const unsigned key = orderable(lane_max) >> 16;
+    if (need == 1) return __reduce_max_sync(0xffffffffu, key);
+    unsigned prefix = 0u;
+#pragma unroll 4
+    for (int bit = 15; bit >= 0; --bit) {
+        const unsigned t = prefix | (1u << bit);
+        if (__popc(__ballot_sync(0xffffffffu, key >= t)) >= need) prefix = t;
+    }
+    return prefix;
 }
 
 template <typename T, bool STATS, bool SMALL>
@@ -511,14 +517,12 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
     u64* region = cand + warp * CS_REGION;
     const int region_off = (int)(reinterpret_cast<unsigned char*>(region) - dyn);
     const int hist_off = (int)(reinterpret_cast<unsigned char*>(hist) - dyn);
-    // first-tile bound.  Rank up to 128 (every warp needs at most 16 elements): from the lane maxima, over
-    // groups of two or more lanes.  Beyond (a k that is large for the row): the exact need-th largest maximum
-    // of groups of g elements, at least 4 rank groups in the tile (cheaper bounds from lane maxima or lane
-    // pairs let 10 to 25 % of a tile pass: the extra candidates cost more than the search).
+    // first-tile bound.  Rank up to 128 (every warp needs at most 16 elements): from the lane maxima.
+    // Beyond (a k that is large for the row): the exact need-th largest maximum of groups of g elements, at
+    // least 4 rank groups in the tile (cheaper bounds from lane maxima or lane pairs let 10 to 25 % of a
+    // tile pass: the extra candidates cost more than the search).
     const int rank1 = bound_rank(k_eff, per_tile);
     const int need = (rank1 + WARPS - 1) / WARPS;
-    int group_lanes = 1;
-    while (2 * group_lanes * need <= 32) group_lanes <<= 1;
     int g = VEC;
     while (g > 2 && (TILE_CHUNKS * CHUNK) / g < 4 * rank1) g >>= 1;
 
@@ -574,9 +578,9 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 if (work) {
                     unsigned k16;
                     float wm = 0.f;
-                    if (group_lanes >= 2) {
+                    if (need <= 16) {
                         const float lm = regs.lane_max_plain();
-                        k16 = first_tile_key_groups(lm, group_lanes);
+                        k16 = first_tile_key_lanes(lm, need);
                         if (STATS) wm = warp_max_redux(lm);
                     } else {
                         k16 = first_tile_key(regs, g, need);
