@@ -499,8 +499,10 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
         const bool mass_only = PRECISE && (qe & QUEUE_MASS_ONLY) != 0;
         const int alen_fast = draw_only ? a.accept_len[b] : 0;
         const unsigned long long need = PRECISE ? a.need_rows[b] : 0ull;   // rows with exact chunk sums
-        if (!a.sample_only && a.state_in && a.state_in[b] == 0) {
+        if (!PRECISE && !a.sample_only && a.state_in && a.state_in[b] == 0) {
             // decided by an earlier call: nothing of this sequence is read or written
+            // (the queue of the double-precision pass holds none of these; there state_in may be the
+            // array in which the fast pass has just marked the sequence as decided by this call)
             grid_dependency_sync();
             if (tid == 0 && a.state_out) a.state_out[b] = 0;
             return;

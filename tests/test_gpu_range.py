@@ -190,3 +190,53 @@ def test_argument_checks(ps):
                                  inp["u_accept"], inp["u_resample"])
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_thresholds_in_a_later_window_of_a_shared_state_array(ps, dtype):
+    # Accept uniforms and draws within a few fp32 ulps of their thresholds, in the windows after the first,
+    # where state_in and state_out are one array: those sequences are decided in double precision.
+    w = gen.scaled(gen.WORKLOADS["config3"], B=48, V=40000, dtype=dtype)
+    inp, (qi, qp, qc, tok) = _case(w, seed=6700)
+    tl, T = _np(inp["target_logits"]), _np(inp["temperature"])
+    rng = np.random.default_rng(67)
+    ua, ur = np.zeros((w.B, w.G), np.float32), _np(inp["u_resample"]).copy()
+    near = 0
+    for b in range(w.B):
+        i = 2 + b % (w.G - 2)                   # the position that decides; u = 0 accepts all before it
+        x = tl[b, i].astype(np.float64) / float(T[b])
+        p = np.exp(x - x.max())
+        p /= p.sum()
+        q = np.zeros_like(p)
+        n = int(qc[b, i])
+        q[qi[b, i, :n]] = qp[b, i, :n].astype(np.float64)
+        ratio = p[tok[b, i]] / q[tok[b, i]]
+        if b % 2 == 0 and ratio < 1.0:
+            ua[b, i] = np.float32(ratio * (1 + int(rng.integers(-2, 3)) * 6e-8))
+            near += 1
+        else:
+            ua[b, i] = np.float32(1.0 - 2.0 ** -24)
+            cum = np.cumsum(np.add.reduceat(np.maximum(p - q, 0.0), np.arange(0, w.V, 1024)))
+            c = int(rng.integers(0, len(cum) - 1))
+            ur[b, 0] = np.float32(cum[c] / cum[-1] * (1 + int(rng.integers(-2, 3)) * 6e-8))
+    assert near >= 8
+    d = [_cuda(x) for x in (tok, qi, qp, qc, ua, ur)]
+    ctx = ps.Context(w.B, w.G, w.V, w.k_max)
+    try:
+        o, o_state, g, g_state, borderline, slow = None, None, None, None, 0, 0
+        for r0, r1 in ((0, 2), (2, 5), (5, w.G + 1)):
+            o = oracle.verify_range(tl, T, None, r0, r1, o_state, tok, qi, qp, qc, ua, ur, out=o, nthreads=oracle.cores())
+            g = ctx.verify_range(inp["target_logits"], inp["temperature"], None, r0, r1, g_state, *d, out=g)
+            o_state, g_state = o["state"], g["state"]
+            st, slow = ctx.status()
+            assert st == 0
+            for k in ("state", "accept_len", "token"):
+                assert np.array_equal(_np(g[k]), o[k]), (k, r0, r1)
+            assert int(g["borderline_count"].item()) == o["borderline_count"], (r0, r1)
+            borderline += o["borderline_count"]
+            m = ~np.isnan(o["resid_mass"])
+            np.testing.assert_allclose(_np(g["p_draft"])[m], o["p_draft"][m], rtol=RTOL, atol=0)
+            np.testing.assert_allclose(_np(g["resid_mass"])[m], o["resid_mass"][m], rtol=RTOL, atol=ATOL_MASS)
+        assert borderline >= near and slow >= near
+    finally:
+        ctx.close()
