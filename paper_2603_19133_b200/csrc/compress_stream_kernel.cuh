@@ -14,12 +14,12 @@
 //     zero so that a window that crosses zero does not spend itself on tiny exponents; 4096 bins
 //     reach 32 binades up, whatever lies beyond shares the last bin; thr is the lower edge of the
 //     highest bin whose suffix count reaches the wanted rank.
-//     The warps take turns refreshing it, once per tile; a warp whose region fills refreshes it
-//     and drops its candidates below it;
-//   - the first tile of a row gets its bound without the histogram: every warp finds a value that an
-//     eighth of the wanted rank of small groups of its elements reach with their maximum; the smallest
-//     of the eight values is reached by the wanted rank of elements (one CTA barrier, the only one
-//     inside a row);
+//     One warp or another refreshes it, after ever more tiles;
+//   - the first tile of a row gets its bound without the histogram: every warp finds a value that its
+//     share of the wanted rank of small groups of its elements reach with their maximum; the smallest of
+//     the eight values, or the third smallest with a larger share, is reached by the wanted rank of
+//     elements (one CTA barrier, the only one inside a row);
+//   - a chunk of which too much passes goes a slower way (crowded_chunk);
 //   - a row whose candidates do not fit (heavy ties), or whose bound rose past its k-th largest, is
 //     handed to the direct kernel through a redo list;
 //   - with top-p the same pass accumulates the softmax normaliser relative to the first tile's
@@ -66,6 +66,31 @@ struct CsRowMeta {
     double z_stream;  // sum of 2^(l * c32 - ref_off) over the row (top-p only)
 };
 
+// capacity of a row's scratch area (keys) for a sparse-row capacity k_max
+__host__ __device__ __forceinline__ int cs_survivor_cap(int k_max) { return 2 * k_max > 512 ? 2 * k_max : 512; }
+
+struct __align__(8) CsShared {
+    unsigned thr_key;   // orderable form of the current lower bound on the k-th largest logit
+    unsigned certain;   // counts are no longer capped (crowded_chunk): only k of them make a bound
+    unsigned first_key[WARPS];  // the warps' own bounds of the first tile
+    unsigned top_key;   // largest orderable logit of the first tile
+    int g0;             // bin coordinate of the first tile's bound: origin of the histogram
+    int area;           // scratch area of the piece
+    int seen;           // chunks whose entries are counted, or are being counted
+    int overflow;       // the scratch area ran out of room: the row goes to the redo list
+    int nan;
+    int m;              // survivors written at the end of the piece
+    double wsum[WARPS];
+};
+// state of the CTA that outlives a piece
+struct CsCta {
+    int abort;          // a bounded wait ran out somewhere in the CTA
+    int k, surv_cap, quota;     // as in FilterBound
+    u64* surv_keys;
+    int wcnt[WARPS];    // per warp: entries in its region (the slot counter its lanes draw from)
+    int marked[WARPS];  // per warp: its region may hold entries that are not counted yet
+    int2 arg[WARPS];    // per warp: what crowded_chunk takes besides its arguments (chunk's offset, its first index)
+};
 // bf16 SMALL: CAP 2048, 3 stages x 16 KB; bf16 LARGE: CAP 4096, 2 stages x 16 KB (72.5 KB either way:
 // 3 CTAs / SM).  fp32: 2 stages x 32 KB (88.5 / 104.5 KB: 2 CTAs / SM).
 template <typename T, bool SMALL> struct CsGeom {
@@ -75,38 +100,19 @@ template <typename T, bool SMALL> struct CsGeom {
     static constexpr int CTAS = sizeof(T) == 2 ? 3 : 2;
     static constexpr int TILE_BYTES = TILE_CHUNKS * CHUNK * (int)sizeof(T);
     static constexpr int STAGE_BYTES = STAGES * TILE_BYTES;
-    static constexpr int SMEM_BYTES = STAGE_BYTES + CAP * 8 + CS_HIST_WORDS * 4;
+    static constexpr int HIST_OFF = STAGE_BYTES + CAP * 8;
+    static constexpr int SHARED_OFF = HIST_OFF + CS_HIST_WORDS * 4;    // CsShared[2], CsCta
+    static constexpr int SMEM_BYTES = SHARED_OFF + 2 * (int)sizeof(CsShared) + (int)sizeof(CsCta);
 };
 
-// capacity of a row's scratch area (keys) for a sparse-row capacity k_max
-__host__ __device__ __forceinline__ int cs_survivor_cap(int k_max) { return 2 * k_max > 512 ? 2 * k_max : 512; }
-
-struct CsShared {
-    unsigned thr_key;   // orderable form of the current lower bound on the k-th largest logit
-    unsigned thr0_key;  // first-tile bound: minimum over the warps' own bounds
-    unsigned top_key;   // largest orderable logit of the first tile
-    int overflow;       // a region ran out of room: the row goes to the redo list
-    int nan;
-    int m;              // survivors written at the end of the piece
-    double wsum[WARPS];
-};
-// state of the CTA that outlives a piece
-struct CsCta {
-    int abort;          // a bounded wait ran out somewhere in the CTA
-    int wcnt[WARPS];    // per warp: entries in its region (the slot counter its lanes draw from)
-};
 __device__ __forceinline__ void cs_reset(CsShared& cs) {
     cs.thr_key = 0u;
-    cs.thr0_key = 0xffffffffu;
+    cs.certain = 0u;
+    cs.seen = 0;
     cs.top_key = 0u;
     cs.overflow = 0;
     cs.nan = 0;
     cs.m = 0;
-}
-
-// threshold (a float) of an orderable key; keys below 0x00800000 are -inf and the negative NaN patterns
-__device__ __forceinline__ float thr_of_key(unsigned key) {
-    return key < 0x00800000u ? -CUDART_INF_F : from_orderable(key);
 }
 
 // ---- per-dtype pieces --------------------------------------------------------------------------
@@ -273,13 +279,29 @@ __device__ __forceinline__ int kth_bin(const unsigned* hist, int k, int lane) {
     return hit2 ? 32 * s + (31 - __clz(hit2)) : 32 * s;
 }
 
-// One warp: raise thr to the lower edge of the highest bin whose suffix count reaches k.
-__device__ __forceinline__ void refresh_threshold(const unsigned* hist, CsShared& cs, int k, int lane) {
-    const int found = kth_bin(hist, k, lane);
-    if (found >= 0 && lane == 0) {
-        const int g0 = bin_coord(*(volatile unsigned*)&cs.thr0_key >> 16);
-        atomicMax(&cs.thr_key, coord_code(g0 + found) << 16);
+// One warp: raise thr to the lower edge of the highest bin whose suffix count reaches `rank` (or k, if
+// counts that are not capped may be among those read: the flag is set before the first of them is added).
+__device__ __forceinline__ void refresh_threshold(const unsigned* hist, CsShared& cs, int rank, int k, int lane) {
+    int found = kth_bin(hist, rank, lane);
+    if (rank < k) {
+        __threadfence_block();
+        if (__any_sync(0xffffffffu, *(volatile unsigned*)&cs.certain)) found = kth_bin(hist, k, lane);
     }
+    if (found >= 0 && lane == 0) atomicMax(&cs.thr_key, coord_code(*(volatile int*)&cs.g0 + found) << 16);
+}
+
+// A candidate's low word is ~index, whose top bit is set; cleared, it marks an entry that is not counted yet.
+constexpr u64 CS_COUNTED = 0x80000000ull;
+// One warp: count the entries of its region that are not counted yet.
+__device__ __forceinline__ void count_marked(unsigned* hist, u64* region, int n, int g0, int lane) {
+    for (int x = lane; x < n; x += 32) {
+        const u64 key = region[x];
+        if (!(key & CS_COUNTED)) {
+            region[x] = key | CS_COUNTED;
+            hist_add(hist, hist_bin((unsigned)(key >> 32), g0));
+        }
+    }
+    __syncwarp();
 }
 
 // Warp-local: drop the entries of this warp's region below thr (stable, in place).
@@ -297,22 +319,126 @@ __device__ __forceinline__ int compact_region(u64* region, int n, unsigned thr_k
     return out;
 }
 
+// The out-of-line functions find the shared state by its place in the dynamic shared memory (`copy`: which of
+// the two of the per-piece state): every argument is a register that is live in the kernel's loop.
 // Refresh the bound (one warp; out of line).
-__device__ __noinline__ void refresh_bound(int hist_off, CsShared* cs, int k_eff) {
+template <typename Geom> __device__ __noinline__ void refresh_bound(int copy, int rank, int k) {
     extern __shared__ __align__(1024) unsigned char dyn[];
-    refresh_threshold(reinterpret_cast<const unsigned*>(dyn + hist_off), *cs, k_eff, threadIdx.x & 31);
+    CsShared& cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF)[copy];
+    refresh_threshold(reinterpret_cast<const unsigned*>(dyn + Geom::HIST_OFF), cs, rank, k, threadIdx.x & 31);
 }
-// Region nearly full: bring the bound up to date and drop what fell below it (one warp; out of line).
-// The warp's slot counter follows.
-__device__ __noinline__ int maintain_region(int wcount, int region_off, int hist_off, CsShared* cs, int* wcnt, int k_eff) {
+// First tile of a piece: the bound is the NTH smallest of the warps' own (one warp, every warp with the same
+// result; out of line).
+template <typename Geom, int NTH> __device__ __noinline__ void first_bound(int copy, int area) {
     extern __shared__ __align__(1024) unsigned char dyn[];
+    CsShared* cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF) + copy;
     const int lane = threadIdx.x & 31;
-    refresh_threshold(reinterpret_cast<const unsigned*>(dyn + hist_off), *cs, k_eff, lane);
+    // (the lane number makes the keys distinct)
+    unsigned key = lane < WARPS ? *(volatile unsigned*)&cs->first_key[lane] | lane : 0xffffffffu;
+    unsigned bound = __reduce_min_sync(0xffffffffu, key);
+#pragma unroll
+    for (int x = 1; x < NTH; ++x) {
+        if (key == bound) key = 0xffffffffu;
+        bound = __reduce_min_sync(0xffffffffu, key);
+    }
+    bound &= 0xffff0000u;
+    if (lane == 0) {
+        *(volatile int*)&cs->g0 = bin_coord(bound >> 16);
+        *(volatile int*)&cs->area = area;
+        atomicMax(&cs->thr_key, bound);
+    }
     __syncwarp();
-    const int n = compact_region(reinterpret_cast<u64*>(dyn + region_off), wcount, *(volatile unsigned*)&cs->thr_key, lane);
-    if (lane == 0) *wcnt = n;
+}
+// orderable form of a staged value (-0 becomes +0)
+template <typename T> __device__ __forceinline__ uint32_t staged_key(const unsigned char* chunk, int off) {
+    const uint32_t bits = __float_as_uint(staged_value(chunk, off, (const T*)nullptr) + 0.0f);
+    return bits ^ ((uint32_t)((int32_t)bits >> 31) | 0x80000000u);
+}
+// A chunk of which more passes (`mask` per lane) than it may count with, or than the warp's region (n entries)
+// has room for (one warp; out of line).
+//   - If there is room, as many as the quota are counted, the others are marked.
+//   - Else the bound is brought up to date and what falls below it is dropped.  With spread tiles all that
+//     the warp holds is counted before, the chunk's values included, so that k of them make a bound that
+//     is certain and as high as the counts allow; and if the rest still does not fit, the region is emptied
+//     into the piece's scratch area, and the chunk's values follow if they are more than the region holds.
+// Returns the entries in the region, or -1: the row goes to the direct kernel.
+template <typename T, typename Geom, bool SPREAD>
+__device__ __noinline__ int crowded_chunk(unsigned mask, int n, int copy) {
+    extern __shared__ __align__(1024) unsigned char dyn[];
+    constexpr int REGION = Geom::REGION;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    CsShared* cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF) + copy;
+    CsCta* cta = reinterpret_cast<CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
+    const unsigned char* chunk = dyn + cta->arg[warp].x;
+    const int vchunk = cta->arg[warp].y;
+    unsigned* hist = reinterpret_cast<unsigned*>(dyn + Geom::HIST_OFF);
+    u64* region = reinterpret_cast<u64*>(dyn + Geom::STAGE_BYTES) + warp * REGION;
+    u64* to = region;
+    int* wcnt = &cta->wcnt[warp];
+    const int g0 = *(volatile int*)&cs->g0, k = cta->k;
+    int own = __popc(mask), added = __reduce_add_sync(0xffffffffu, own);
+    int held = n;                   // slots taken at `to`
+    int count = 0;                  // entries of the chunk that are counted below
+    if (n + added <= REGION) {
+        const bool certain = __any_sync(0xffffffffu, *(volatile unsigned*)&cs->certain);
+        count = certain ? added : cta->quota;
+        if (lane == 0) cta->marked[warp] = 1;
+    } else if (!SPREAD) {
+        refresh_threshold(hist, *cs, k, k, lane);
+        __syncwarp();
+    } else {
+        if (lane == 0) *(volatile unsigned*)&cs->certain = 1u;
+        __threadfence_block();
+        __syncwarp();
+        count_marked(hist, region, n, g0, lane);
+        for (unsigned m = mask; m; m &= m - 1u)
+            hist_add(hist, hist_bin(staged_key<T>(chunk, bit_offset(__ffs(m) - 1, lane, (const T*)nullptr)), g0));
+        __syncwarp();
+        refresh_threshold(hist, *cs, k, k, lane);
+        __syncwarp();
+    }
+    if (n + added > REGION) {
+        const unsigned thr_key = __shfl_sync(0xffffffffu, *(volatile unsigned*)&cs->thr_key, 0);
+        held = n = compact_region(region, n, thr_key, lane);
+        unsigned left = 0u;
+        for (unsigned m = mask; m; m &= m - 1u)
+            if (staged_key<T>(chunk, bit_offset(__ffs(m) - 1, lane, (const T*)nullptr)) >= thr_key) left |= m & (0u - m);
+        __syncwarp();
+        mask = left;
+        own = __popc(mask);
+        added = __reduce_add_sync(0xffffffffu, own);
+        if (!SPREAD) count = added;
+        if (n + added > REGION) {
+            if (!SPREAD) return -1;
+            const bool direct = added > REGION;
+            const int spilled = n + (direct ? added : 0), surv_cap = cta->surv_cap;
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&cs->m, spilled);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (base + spilled > surv_cap) return -1;
+            u64* dst = cta->surv_keys + (long long)cs->area * surv_cap + base;
+            for (int x = lane; x < n; x += 32) dst[x] = region[x];
+            held = direct ? n : 0;
+            if (direct) to = dst;
+        }
+        __syncwarp();
+        if (lane == 0) *wcnt = held;
+        __syncwarp();
+    }
+    int pos = atomicAdd(wcnt, own);
+    for (; mask; mask &= mask - 1u) {
+        const int off = bit_offset(__ffs(mask) - 1, lane, (const T*)nullptr);
+        const uint32_t okey = staged_key<T>(chunk, off);
+        u64 key = ((u64)okey << 32) | (u64)(~(uint32_t)(vchunk + off));
+        if (pos - held < count) hist_add(hist, hist_bin(okey, g0));
+        else if (count) key &= ~CS_COUNTED;
+        to[pos++] = key;
+    }
     __syncwarp();
-    return n;
+    if (to == region) return held + added;
+    if (lane == 0) *wcnt = 0;
+    __syncwarp();
+    return 0;
 }
 
 // ---- how the rows of a call are dealt to the CTAs of the filter kernel ----------------------------
@@ -402,21 +528,67 @@ inline FilterPlan make_filter_plan(int rows, int tiles_per_row, bool ragged_last
 //     rank(f) = 1.5 k f + 5 sqrt(1.5 k f) + 12        (at most k)
 // of the elements seen reach, f being the fraction of the row that has been seen: were the k largest spread
 // evenly over the tiles, it would be lower than the k-th largest by a factor 1.5 and five standard
-// deviations in the count.  A tile takes one chunk from each eighth of the row, so that rows whose large
-// logits crowd at one end are spread too.  It is not certain; it is checked: every element dropped
-// was below the final bound, so the row is right if k survivors reach that, and goes to the direct
-// kernel if not.  4096 rows of 262144 entries, k = 1024: 560 -> 473 us; 1536 rows of 128256, top-p with
-// k = 256: 116 -> 111 us; 512 rows of 151936, k = 128: 43 -> 40.7 us.
-__host__ __device__ __forceinline__ int bound_rank(int k, float f) {
+// deviations in the count.
+// They are not: vocabularies have an order (frequent pieces first, languages and unused ids in blocks).
+// A tile takes one chunk from each eighth of the row, so that each eighth is seen to the same fraction, and
+//   - no chunk counts with more than a quarter of the first tile's rank and eight (chunk_quota; the entries
+//     beyond it are marked and counted at the row's end): a crowded place cannot lift the bound above
+//     what three quarters of the rank reach elsewhere, which is still 1.125 k f and more;
+//   - the first tile's bound is the third smallest of the warps' own, a sixth of the rank each: it is neither
+//     lifted by five crowded chunks nor dropped by two empty ones (an unused end of the vocabulary);
+//   - eighth e is streamed by warp (e + tile) % 8, so that a crowded eighth does not fill one warp's region;
+//   - a region that is too full makes the rest of the row go by certain bounds, and empties itself into
+//     the row's scratch area if need be (crowded_chunk).
+// It is not certain; it is checked: every element dropped was below the final bound, so the row is right if
+// k survivors reach that, and goes to the direct kernel if not.  Against certain bounds throughout, compress
+// takes 156 instead of 217 us for 1024 rows of 262144 entries (k = 1024) and 156 instead of 170 for 1536 rows
+// of 128256 (top-p, k = 256) where the large logits lie evenly, 167 instead of 215 and 158 instead of 169 with a
+// quarter of the k largest below index 1024.  (Without the precautions all rows of those two went to the
+// direct kernel: 726 and 662 us.)
+__host__ __device__ __forceinline__ int open_rank(int k, float f) {
     const float e = 1.5f * (float)k * f;
-    const int r = (int)(e + 5.0f * sqrtf(e)) + 12;
+    return (int)(e + 5.0f * sqrtf(e)) + 12;
+}
+__host__ __device__ __forceinline__ int bound_rank(int k, float f) {
+    const int r = open_rank(k, f);
     return r < k ? r : k;
 }
+// what one chunk may count with
+__host__ __device__ __forceinline__ int chunk_quota(int k, float per_tile) { return (open_rank(k, per_tile) + 3) / 4 + 8; }
 // Where one tile's rank is k already (small k) the tiles are contiguous instead: one copy of 16 KB a tile
 // (4096 rows of 32000 entries, k = 8: 69 us against 75 us with eight copies of 2 KB).
-__host__ __device__ __forceinline__ bool bound_spreads(int k, float per_tile) { return bound_rank(k, per_tile) < k; }
-// spread tiles: first of the chunks of a row of `nch` that warp w of the CTA streams
-__device__ __forceinline__ int warp_chunk0(int nch, int w) { return (nch * w) >> 3; }
+// (Rows of two tiles: too few of the eighths may have a chunk in the first.)
+__host__ __device__ __forceinline__ bool bound_spreads(int k, int tiles) { return tiles > 2 && bound_rank(k, 1.0f / (float)tiles) < k; }
+// What the kernel needs of all this, worked out once per call (in the constant bank: no registers).
+struct FilterBound {
+    int k;                  // entries wanted of a row
+    int surv_cap;           // keys in a scratch area
+    bool spread;            // a tile takes a chunk from each eighth of the row (chunks [e, e + 1) * tiles), not eight consecutive
+                            // ones; chunk `tile` of eighth e is streamed by warp (e + tile) % 8
+    float per_tile, per_chunk;  // fractions of a row
+    int need, group;        // first tile: elements that a warp's own bound is reached by, elements per group of its search
+    int quota;              // chunk_quota
+};
+inline FilterBound make_filter_bound(int k, int k_max, int nch, int vec) {
+    FilterBound f;
+    f.k = k;
+    f.surv_cap = cs_survivor_cap(k_max);
+    // (the fewest tiles that a row of V entries takes: a fraction that is too large only makes a bound lower)
+    const int tiles = (nch + TILE_CHUNKS - 1) / TILE_CHUNKS;
+    f.per_tile = 1.0f / (float)tiles;
+    f.per_chunk = f.per_tile / (float)TILE_CHUNKS;
+    f.spread = bound_spreads(k, tiles);
+    // First tile: up to 16 elements per warp from the lane maxima.  Beyond (a k that is large for the row)
+    // the exact need-th largest maximum of groups of elements, at least 4 rank groups in the tile (cheaper
+    // bounds from lane maxima or lane pairs let 10 to 25 % of a tile pass: the extra candidates cost
+    // more than the search).
+    const int rank1 = f.spread ? bound_rank(k, f.per_tile) : k;
+    f.need = f.spread ? (rank1 + 5) / 6 : (rank1 + WARPS - 1) / WARPS;
+    f.group = vec;
+    while (f.group > 2 && (TILE_CHUNKS * CHUNK) / f.group < 4 * rank1) f.group >>= 1;
+    f.quota = f.spread ? chunk_quota(k, f.per_tile) : CHUNK;
+    return f;
+}
 
 // First-tile bound of one warp when it needs at most 16 elements: the need-th largest of its 32 lanes'
 // maxima, as a 16-bit orderable code (rounded down).  (The smallest of the maxima of `need` groups of
@@ -434,44 +606,40 @@ __device__ __forceinline__ unsigned first_tile_key_lanes(float lane_max, int nee
     return prefix;
 }
 
-template <typename T, bool STATS, bool SMALL>
+// SPREAD: bound_spreads for the call's rows
+template <typename T, bool STATS, bool SMALL, bool SPREAD>
 __global__ void __launch_bounds__(STREAM_THREADS, CsGeom<T, SMALL>::CTAS)
-compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_limit_ns) {
+compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned long long wait_limit_ns) {
     extern __shared__ __align__(1024) unsigned char dyn[];
     typedef CsGeom<T, SMALL> Geom;
     constexpr int STAGES = Geom::STAGES;
     constexpr int TILE_BYTES = Geom::TILE_BYTES;
     constexpr int CS_CAND_CAP = Geom::CAP, CS_REGION = Geom::REGION;
-    constexpr int VEC = ChunkRegs<T>::VEC;
     unsigned char* stage_mem = dyn;
     u64* cand = reinterpret_cast<u64*>(dyn + Geom::STAGE_BYTES);
     unsigned* hist = reinterpret_cast<unsigned*>(cand + CS_CAND_CAP);          // bins, then super-bins
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES];
     // Two copies of the per-piece state, used in turn: the copy of the piece that has just ended is
     // reset by one thread while the other warps already start on the next piece.
-    __shared__ CsShared css[2];
-    __shared__ CsCta cta;
+    CsShared* css = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF);
+    CsCta& cta = *reinterpret_cast<CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
-    if (k_eff > a.k_max) k_eff = a.k_max;
-    if (k_eff > a.V) k_eff = a.V;
-    const int surv_cap = cs_survivor_cap(a.k_max);
-    // (the fewest tiles that a row of V entries takes: a fraction that is too large only makes a bound lower)
-    const float per_tile = 1.0f / (float)((a.nch + TILE_CHUNKS - 1) / TILE_CHUNKS);
-    const bool spread = bound_spreads(k_eff, per_tile);
-
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], spread ? WARPS : 1);
+            mbar_init(&full[s], SPREAD ? WARPS : 1);
             mbar_init(&empty[s], WARPS);
         }
         mbar_init_fence();
         cs_reset(css[0]);
         cs_reset(css[1]);
         cta.abort = 0;
+        cta.k = fb.k;
+        cta.surv_cap = fb.surv_cap;
+        cta.quota = fb.quota;
+        cta.surv_keys = a.surv_keys;
     }
-    if (tid < WARPS) cta.wcnt[tid] = 0;
+    if (tid < WARPS) cta.wcnt[tid] = cta.marked[tid] = 0;
     for (int i = tid; i < CS_HIST_WORDS; i += STREAM_THREADS) hist[i] = 0u;
     grid_dependency_sync();
     if (tid == 0 && blockIdx.x == 0) {
@@ -482,7 +650,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
 
     if (warp == WARPS) {
         // ---- producer: every tile of every piece of this CTA, in order; a lane per copy of the tile ----
-        if (lane >= (spread ? WARPS : 1)) return;
+        if (lane >= (SPREAD ? WARPS : 1)) return;
         const uint64_t pol = l2_evict_first_policy();
         uint32_t i = 0;
         FilterPiece pc;
@@ -491,7 +659,6 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
             // (a row with a bad temperature is copied for nothing: its workers look the temperature up)
             const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (srow < 0 ? 0 : srow) * a.row_stride, a.V);
             const int row_chunks = (sr.end + CHUNK - 1) / CHUNK;
-            const int c0 = spread ? warp_chunk0(row_chunks, lane) : 0, c1 = spread ? warp_chunk0(row_chunks, lane + 1) : 0;
             for (int ti = pc.tile0; ti < pc.tile1; ++ti, ++i) {
                 const int s = (int)(i % STAGES);
                 const uint32_t round = i / STAGES;
@@ -501,11 +668,13 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     if (wr == WAIT_LOST) return;      // nothing more is issued
                 }
                 constexpr int GRANULES = CHUNK * (int)sizeof(T) / 16;
-                if (!spread) {
+                if (!SPREAD) {
                     if (srow >= 0)
                         stage_tile<T>(stage_mem + s * TILE_BYTES, sr, ti * (TILE_CHUNKS * GRANULES), TILE_CHUNKS * GRANULES, &full[s], pol);
-                } else if (srow >= 0 && c0 + ti < c1) {
-                    stage_tile<T>(stage_mem + s * TILE_BYTES + lane * (GRANULES * 16), sr, (c0 + ti) * GRANULES, GRANULES, &full[s], pol);
+                } else if (srow >= 0 && lane * plan.tiles_per_row + ti < row_chunks) {
+                    // (a lane per eighth)
+                    stage_tile<T>(stage_mem + s * TILE_BYTES + ((lane + ti) & (WARPS - 1)) * (GRANULES * 16), sr,
+                                  (lane * plan.tiles_per_row + ti) * GRANULES, GRANULES, &full[s], pol);
                 }
                 mbar_arrive(&full[s]);
             }
@@ -515,17 +684,6 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
 
     // ---- workers ------------------------------------------------------------------------------
     u64* region = cand + warp * CS_REGION;
-    const int region_off = (int)(reinterpret_cast<unsigned char*>(region) - dyn);
-    const int hist_off = (int)(reinterpret_cast<unsigned char*>(hist) - dyn);
-    // first-tile bound.  Rank up to 128 (every warp needs at most 16 elements): from the lane maxima.
-    // Beyond (a k that is large for the row): the exact need-th largest maximum of groups of g elements, at
-    // least 4 rank groups in the tile (cheaper bounds from lane maxima or lane pairs let 10 to 25 % of a
-    // tile pass: the extra candidates cost more than the search).
-    const int rank1 = bound_rank(k_eff, per_tile);
-    const int need = (rank1 + WARPS - 1) / WARPS;
-    int g = VEC;
-    while (g > 2 && (TILE_CHUNKS * CHUNK) / g < 4 * rank1) g >>= 1;
-
     bool dead = false;      // a wait ran out: this warp computes no more, but takes every tile and joins every barrier
     bool lost = false;      // a wait did not complete at all: the warp stops waiting as well
     uint32_t i = 0;
@@ -542,17 +700,12 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         // chunks are counted from the row's first granule here: which 1024 entries make one is no matter
         const StagedRow<T> sr(reinterpret_cast<const T*>(a.logits) + (in_range ? srow : 0) * a.row_stride, a.V);
         const int mis = sr.mis, end = sr.end;
-        // this warp's chunk of tile ti: c0 + ti * c_step, if below c1
-        const int row_chunks = (unsigned)(end + CHUNK - 1) / CHUNK;
-        const int c0 = spread ? warp_chunk0(row_chunks, warp) : warp;
-        const int c1 = spread ? warp_chunk0(row_chunks, warp + 1) : row_chunks;
-        const int c_step = spread ? 1 : TILE_CHUNKS;
         const bool valid = temp_ok(Tb) && in_range;
+        // chunks of the row; 0 once nothing more of it is to be worked on
+        int row_chunks = valid && !dead ? (unsigned)(end + CHUNK - 1) / CHUNK : 0;
         const float c32 = temp_scale(Tb);
         float ref_off = 0.f, acc = 0.f;
         int wcount = 0;             // candidates in this warp's region (cs.wcnt[warp] holds the same number)
-        int g0 = 0;                 // bin coordinate of the first tile's bound: origin of the histogram
-        bool full_region = false;   // the region ran out of room (the row goes to the direct kernel)
 
         for (int ti = pc.tile0; ti < pc.tile1; ++ti, ++i) {
             const int s = (int)(i % STAGES);
@@ -561,6 +714,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                 const int wr = mbar_wait_twice(&full[s], round & 1, wait_limit_ns);
                 if (wr != WAIT_OK) {
                     dead = true;
+                    row_chunks = 0;
                     lost = wr == WAIT_LOST;
                     if (lane == 0) {
                         cta.abort = 1;
@@ -568,69 +722,67 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     }
                 }
             }
-            const int c = c0 + ti * c_step;
-            const bool work = !dead && valid && !full_region && c < c1;
+            // this warp's chunk of the tile
+            const int c = SPREAD ? ((warp - ti) & (WARPS - 1)) * plan.tiles_per_row + ti : ti * TILE_CHUNKS + warp;
+            const bool work = c < row_chunks;
             const unsigned char* chunk = stage_mem + s * TILE_BYTES + warp * (CHUNK * (int)sizeof(T));
             ChunkRegs<T> regs;
             if (work) load_staged(regs, chunk, c * CHUNK, end, lane);
             if (ti == pc.tile0 && valid) {
-                // first tile of a piece (every warp holds a full chunk): each warp's own bound, then the minimum
+                // first tile of a piece: each warp's own bound (none without a chunk), then the smallest of them, or the
+                // third smallest
+                if (lane == 0) cs.first_key[warp] = 0u;
                 if (work) {
                     unsigned k16;
                     float wm = 0.f;
-                    if (need <= 16) {
+                    if (fb.need <= 16) {
                         const float lm = regs.lane_max_plain();
-                        k16 = first_tile_key_lanes(lm, need);
+                        k16 = first_tile_key_lanes(lm, fb.need);
                         if (STATS) wm = warp_max_redux(lm);
                     } else {
-                        k16 = first_tile_key(regs, g, need);
+                        k16 = first_tile_key(regs, fb.group, fb.need);
                         if (STATS) wm = warp_max_redux(regs.lane_max_plain());
                     }
                     if (lane == 0) {
-                        atomicMin(&cs.thr0_key, k16 << 16);
+                        cs.first_key[warp] = k16 << 16;
                         if (STATS && wm == wm) atomicMax(&cs.top_key, orderable(wm));
                     }
                 }
                 workers_sync();
-                const unsigned thr0 = *(volatile unsigned*)&cs.thr0_key;
-                g0 = bin_coord(thr0 >> 16);
-                if (lane == 0) atomicMax(&cs.thr_key, thr0);
+                first_bound<Geom, SPREAD ? 3 : 1>(parity ^ 1, pc.area);
                 if (STATS) ref_off = __fmul_rn(from_orderable(*(volatile unsigned*)&cs.top_key), c32);
+                if (*(volatile unsigned*)&cs.thr_key < 0x00800000u) {
+                    // no finite bound (rows of -inf): everything would pass, padding included
+                    if (lane == 0) cs.overflow = 1;
+                    row_chunks = 0;
+                }
                 __syncwarp();
             }
             int added = 0;          // what this chunk appends to the region
-            if (work) {
-                const unsigned thr_key = *(volatile unsigned*)&cs.thr_key;
-                unsigned mask = pass_mask(regs, thr_of_key(thr_key));
-                if (thr_key < 0x00800000u) {
-                    // no finite bound (rows of -inf): everything would pass, padding included
-                    full_region = true;
-                    mask = 0u;
-                }
+            if (work && row_chunks) {
+                if (SPREAD && lane == 0) atomicAdd(&cs.seen, 1);
+                unsigned mask = pass_mask(regs, from_orderable(*(volatile unsigned*)&cs.thr_key));
                 const int n = __popc(mask);
                 added = __reduce_add_sync(0xffffffffu, n);
                 if (added) {
-                    if (wcount + added > CS_REGION) {
-                        // no room: bring the bound up to date and drop what fell below it
-                        wcount = maintain_region(wcount, region_off, hist_off, &cs, &cta.wcnt[warp],
-                                                 bound_rank(k_eff, per_tile * (float)(ti - pc.tile0 + 1)));
-                        if (wcount + added > CS_REGION) {     // ties, a coarse bin too full, or a very loose bound
-                            full_region = true;
-                            mask = 0u;
-                            added = 0;
-                        }
-                    }
                     const int vchunk = c * CHUNK - mis;
-                    // every lane appends its own passing values: its slots come from the warp's counter
-                    if (mask) {
+                    if (added > (SPREAD ? min(fb.quota, CS_REGION - wcount) : CS_REGION - wcount)) {
+                        if (lane == 0) cta.arg[warp] = make_int2((int)(chunk - dyn), vchunk);
+                        __syncwarp();
+                        wcount = crowded_chunk<T, Geom, SPREAD>(mask, wcount, parity ^ 1);
+                        if (wcount < 0) {
+                            if (lane == 0) cs.overflow = 1;
+                            row_chunks = wcount = 0;
+                        }
+                        added = 0;
+                    } else if (mask) {
+                        // every lane appends its own passing values: its slots come from the warp's counter
                         int pos = atomicAdd(&cta.wcnt[warp], n);
                         do {
                             const int bit = __ffs(mask) - 1;
                             mask &= mask - 1u;
                             const int off = bit_offset(bit, lane, (const T*)nullptr);
-                            const uint32_t bits = __float_as_uint(staged_value(chunk, off, (const T*)nullptr) + 0.0f);   // -0 becomes +0
-                            const uint32_t okey = bits ^ ((uint32_t)((int32_t)bits >> 31) | 0x80000000u);
-                            region[pos++] = ((u64)okey << 32) | (u64)(~(uint32_t)(vchunk + off));
+                            region[pos++] = ((u64)staged_key<T>(chunk, off) << 32) | (u64)(~(uint32_t)(vchunk + off));
                         } while (mask);
                     }
                 }
@@ -645,20 +797,28 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
                     const float lm = regs.lane_max();
                     if (lm != lm) cs.nan = 1;
                 }
-                // count the new entries in the histogram
+                // count the new entries in the histogram (those of a crowded chunk are counted already)
+                const int g0 = *(volatile int*)&cs.g0;
                 for (int x = wcount + lane; x < wcount + added; x += 32) hist_add(hist, hist_bin((unsigned)(region[x] >> 32), g0));
                 wcount += added;
-                // the bound is refreshed after every tile, each time by another warp (the others'
-                // latest values may not be counted yet, which only makes it a little lower)
-                if (warp == (ti & (WARPS - 1))) {
+                // The bound is refreshed after tiles 1, 2, 3, 4, 6, 8, 12, 16, 24, ..., by one warp or another.  (After
+                // every tile it took 157 -> 162 us of compress for 1024 rows of 262144 entries, k = 1024.)
+                // The rank goes by the chunks that all warps have counted: some are tiles ahead of this one.
+                const int t = ti - pc.tile0 + 1;
+                if (warp == ((t + (t >> 3)) & (WARPS - 1)) && ((t & (t - 1)) == 0 || (t & 7) == 0 || t == 3 || t == 6 || t == 12)) {
                     __syncwarp();
-                    refresh_bound(hist_off, &cs, spread ? bound_rank(k_eff, per_tile * (float)(ti - pc.tile0 + 1)) : k_eff);
+                    const int rank = SPREAD ? bound_rank(fb.k, fb.per_chunk * (float)*(volatile int*)&cs.seen) : fb.k;
+                    refresh_bound<Geom>(parity ^ 1, rank, fb.k);
                 }
             }
         }
 
         // ---- end of the piece: survivors and statistics to the piece's scratch area ------------------
-        if (lane == 0 && full_region) cs.overflow = 1;
+        const bool whole = pc.tile1 - pc.tile0 == plan.tiles_per_row;
+        __syncwarp();
+        if (SPREAD && whole && *(volatile int*)&cta.marked[warp]) {
+            count_marked(hist, region, wcount, *(volatile int*)&cs.g0, lane);
+        }
         if (STATS) {
             const double sw = (double)warp_sum(acc);
             if (lane == 0) cs.wsum[warp] = sw;
@@ -668,16 +828,17 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         unsigned thr_final = *(volatile unsigned*)&cs.thr_key;
         if (piece_ok) {
             // the final bound, by every warp for itself (all get the same): no second barrier for it
-            const int found = kth_bin(hist, spread ? bound_rank(k_eff, per_tile * (float)(pc.tile1 - pc.tile0)) : k_eff, lane);
-            if (found >= 0) thr_final = max(thr_final, coord_code(g0 + found) << 16);
+            const bool certain = !SPREAD || whole || *(volatile unsigned*)&cs.certain;
+            const int found = kth_bin(hist, certain ? fb.k : bound_rank(fb.k, fb.per_tile * (float)(pc.tile1 - pc.tile0)), lane);
+            if (found >= 0) thr_final = max(thr_final, coord_code(*(volatile int*)&cs.g0 + found) << 16);
             // every warp filters its own region and appends to the piece's scratch area
-            u64* dst = a.surv_keys + (long long)pc.area * surv_cap;
+            u64* dst = a.surv_keys + (long long)pc.area * fb.surv_cap;
             const int n = compact_region(region, wcount, thr_final, lane);
             int base = 0;
             if (lane == 0 && n) base = atomicAdd(&cs.m, n);
             base = __shfl_sync(0xffffffffu, base, 0);
             for (int x = lane; x < n; x += 32)
-                if (base + x < surv_cap) dst[base + x] = region[x];
+                if (base + x < fb.surv_cap) dst[base + x] = region[x] | CS_COUNTED;
         }
         workers_sync();     // the survivors are counted; nobody reads the histogram any more
         if (tid == 0) {
@@ -686,9 +847,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
             if (cta.abort) flags = CSF_ABORT;
             else if (!in_range) flags = CSF_RANGE;
             else if (!valid) flags = CSF_TEMPERATURE;
-            else if (cs.overflow || m > surv_cap) flags = CSF_REDO;      // too many candidates or ties at the bound
+            else if (cs.overflow || m > fb.surv_cap) flags = CSF_REDO;      // too many candidates, or ties at the bound
             else if (cs.nan) flags = CSF_LOGIT;
-            else if (pc.tile1 - pc.tile0 == plan.tiles_per_row && m < k_eff) flags = CSF_REDO;   // the bound reached too far
             double zs = 0.0;
             if (STATS)
                 for (int w = 0; w < WARPS; ++w) zs += cs.wsum[w];
@@ -705,7 +865,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, unsigned long long wait_
         }
         // Ready for the next piece, without a barrier of its own: the histogram is not written before
         // the barrier of that piece's first tile, which every warp reaches after its share of this.
-        if (lane == 0) cta.wcnt[warp] = 0;
+        if (lane == 0) cta.wcnt[warp] = cta.marked[warp] = 0;
         for (int x = tid; x < CS_HIST_WORDS; x += THREADS) hist[x] = 0u;
     }
 }

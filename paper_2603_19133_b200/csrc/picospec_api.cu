@@ -28,7 +28,7 @@ struct picospec_ctx {
     unsigned long long wait_limit_ns;   // first limit of the staged kernels' waits
     int last_cuda_error;
     unsigned long long compress_calls;
-    int filter_ctas[2][2][2];           // resident CTAs per SM of the filter kernel's variants (0: not asked yet)
+    int filter_ctas[2][2][2][2];        // resident CTAs per SM of the filter kernel's variants (0: not asked yet)
     // optional per-kernel timing (picospec_profile_*): rings of event pairs per kernel kind
     int prof_level;
     cudaEvent_t prof_ev[PICOSPEC_PROF_KINDS][PROF_RING][2];
@@ -104,18 +104,18 @@ template <typename T> void set_compress_attrs() {
     cudaFuncSetAttribute(compress_kernel<T, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
 }
 
+template <typename T, bool SMALL, bool SPREAD> cudaError_t set_filter_attrs() {
+    constexpr int bytes = CsGeom<T, SMALL>::SMEM_BYTES;
+    cudaError_t e = cudaFuncSetAttribute(compress_filter_kernel<T, true, SMALL, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(compress_filter_kernel<T, false, SMALL, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e;
+}
 template <typename T> cudaError_t set_filter_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(compress_filter_kernel<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         CsGeom<T, true>::SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(compress_filter_kernel<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 CsGeom<T, true>::SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(compress_filter_kernel<T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 CsGeom<T, false>::SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(compress_filter_kernel<T, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 CsGeom<T, false>::SMEM_BYTES);
+    cudaError_t e = set_filter_attrs<T, true, true>();
+    if (e == cudaSuccess) e = set_filter_attrs<T, true, false>();
+    if (e == cudaSuccess) e = set_filter_attrs<T, false, true>();
+    if (e == cudaSuccess) e = set_filter_attrs<T, false, false>();
     return e;
 }
 
@@ -170,6 +170,10 @@ void launch_compress_finish(const CompressArgs& a, const FilterPlan& plan, bool 
     else launch_chained(compress_finish_kernel<T, false, TPR>, grid, TPR * ROWS, finish_smem_bytes<TPR>(), s, a, plan);
 }
 
+template <typename T, bool STATS, bool SMALL> auto filter_kernel(const FilterBound& fb) {
+    return fb.spread ? compress_filter_kernel<T, STATS, SMALL, true> : compress_filter_kernel<T, STATS, SMALL, false>;
+}
+
 template <typename T>
 cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool aligned, cudaStream_t s) {
     const int rows = a.B * a.G;
@@ -184,12 +188,13 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
         if (k_eff > a.k_max) k_eff = a.k_max;
         const bool small = k_eff <= CS_K_SMALL;
-        void (*kern)(CompressArgs, FilterPlan, unsigned long long) =
-            small ? (stats ? compress_filter_kernel<T, true, true> : compress_filter_kernel<T, false, true>)
-                  : (stats ? compress_filter_kernel<T, true, false> : compress_filter_kernel<T, false, false>);
+        const FilterBound fb = make_filter_bound(k_eff, a.k_max, a.nch, ChunkRegs<T>::VEC);
+        void (*kern)(CompressArgs, FilterPlan, FilterBound, unsigned long long) =
+            small ? (stats ? filter_kernel<T, true, true>(fb) : filter_kernel<T, false, true>(fb))
+                  : (stats ? filter_kernel<T, true, false>(fb) : filter_kernel<T, false, false>(fb));
         const int smem = small ? CsGeom<T, true>::SMEM_BYTES : CsGeom<T, false>::SMEM_BYTES;
         // resident CTAs per SM for this kernel's registers and shared memory (asking costs a microsecond: once)
-        int& per_sm = ctx->filter_ctas[sizeof(T) == 2][small][stats];
+        int& per_sm = ctx->filter_ctas[sizeof(T) == 2][small][stats][fb.spread];
         if (per_sm == 0) {
             cudaError_t eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, STREAM_THREADS, smem);
             if (eo != cudaSuccess) return eo;
@@ -204,7 +209,7 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
                                                  (long long)ctx->num_sms * per_sm);
         {
             ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_STREAM, 1, s);
-            launch_chained(kern, plan.grid, STREAM_THREADS, smem, s, a, plan, ctx->wait_limit_ns);
+            launch_chained(kern, plan.grid, STREAM_THREADS, smem, s, a, plan, fb, ctx->wait_limit_ns);
         }
         cudaError_t e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;

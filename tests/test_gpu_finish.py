@@ -48,14 +48,14 @@ def test_select_and_order(rows, V, k, above, ties, binades, redo, dtype):
 
 
 @pytest.mark.parametrize("top_p", [1.0, 0.9])
-@pytest.mark.parametrize("rows,V,k,head,redo", [
-    (460, 65536, 256, 1.0 / 8, False),       # the large logits spread over the row (whole rows and pieces)
-    (5, 131072, 100, 0.6, False),            # six in ten of them in the first eighth
-    (5, 65536, 256, 1.0, False),             # all of them in the first eighth, spread over it
-    (5, 65536, 256, -1.0, True),             # all of them in 512 neighbouring entries: the bound rises past the k-th
+@pytest.mark.parametrize("rows,V,k,head", [
+    (460, 65536, 256, 1.0 / 8),              # the large logits spread over the row (whole rows and pieces)
+    (5, 131072, 100, 0.6),                   # six in ten of them in the first eighth
+    (5, 65536, 256, 1.0),                    # all of them in the first eighth, spread over it
+    (5, 65536, 256, -1.0),                   # all of them in 512 neighbouring entries
 ])
-def test_bound_ahead_of_the_rows_end(rows, V, k, head, redo, top_p):
-    # where the k largest lie must not show in the result, only in whether the direct kernel is needed
+def test_bound_ahead_of_the_rows_end(rows, V, k, head, top_p):
+    # where the k largest lie must show neither in the result nor in whether the direct kernel is needed
     import paper_2603_19133_b200 as ps
     g = torch.Generator(device="cuda").manual_seed(rows + V + k)
     dl = torch.randn((rows, 1, V), generator=g, device="cuda").clamp_(max=3.9)
@@ -69,8 +69,14 @@ def test_bound_ahead_of_the_rows_end(rows, V, k, head, redo, top_p):
             rest = V // 8 + torch.randperm(V - V // 8, generator=g, device="cuda")[:n - m]
             at = torch.cat([first, rest])
         dl[r, 0, at] = 4.0 + 3.0 * torch.rand(n, generator=g, device="cuda")
-    dl = dl.to(torch.bfloat16)
-    T = torch.full((rows,), 0.8, device="cuda")
+    _check_compress(dl.to(torch.bfloat16), k, top_p, 0.8, g)
+
+
+def _check_compress(dl, k, top_p, temperature, g, staged=True):
+    """Against the oracle; `staged`: no row is handed to the direct kernel."""
+    import paper_2603_19133_b200 as ps
+    rows, _, V = dl.shape
+    T = torch.full((rows,), temperature, device="cuda")
     u = torch.rand((rows, 1), generator=g, device="cuda")
     top_k = k if top_p >= 1.0 else 0
     ctx = ps.Context(rows, 1, V, k)
@@ -80,8 +86,43 @@ def test_bound_ahead_of_the_rows_end(rows, V, k, head, redo, top_p):
         assert ctx.status(clear=True)[0] == 0
     finally:
         ctx.close()
-    assert redone == (rows if redo else 0)
+    assert redone == 0 or not staged
     want = oracle.compress(dl.float().cpu().numpy(), T.cpu().numpy(), top_k, top_p, k, u.cpu().numpy(), nthreads=oracle.cores())
     for a, b in ((got[0], want[0]), (got[2], want[2]), (got[3], want[3])):
         assert np.array_equal(a, b)
     np.testing.assert_allclose(got[1], want[1], rtol=1e-5)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V,k,top_p", [(128256, 64, 0.95), (128256, 1024, 1.0), (262144, 256, 0.9), (32000, 8, 1.0),
+                                       (32000, 256, 1.0), (17409, 500, 1.0), (50381, 512, 0.95)])
+@pytest.mark.parametrize("order", ["quarter", "half", "rank", "mixed", "reversed", "unused", "block"])
+def test_vocabularies_with_an_order(V, k, top_p, order, dtype):
+    # a vocabulary numbered by frequency, with an unused end, with a block of one language: the rows are as
+    # right as any, and (but for logits that follow the numbers altogether) none of them is read a
+    # second time by the direct kernel
+    g = torch.Generator(device="cuda").manual_seed(V + k)
+    rows = 6
+    ids = torch.arange(V, device="cuda").float()
+    noise = 1.5 * torch.randn((rows, V), generator=g, device="cuda")
+    free = -1.1 * torch.log(torch.floor(torch.rand((rows, V), generator=g, device="cuda") * V) + 1.0)
+    x = free + noise
+    if order == "rank":
+        x = noise - 1.1 * torch.log(ids + 1.0)
+    elif order == "mixed":
+        x = noise + 0.5 * free - 0.55 * torch.log(ids + 1.0)
+    elif order == "reversed":
+        x = noise - 1.1 * torch.log(V - ids)
+    elif order == "unused":
+        x[:, V * 7 // 8:] = -30.0
+    elif order == "block":
+        x[:, V // 4:V * 43 // 100] += 2.0
+    else:
+        # a quarter or a half of the k largest among the ids below 1024
+        m = max(1, int(k * (0.25 if order == "quarter" else 0.5)))
+        at = torch.rand((rows, 1024), generator=g, device="cuda").argsort(dim=1)[:, :m]
+        kth = torch.topk(x, k - m + 1, dim=1).values[:, -1:]
+        top = x.amax(dim=1, keepdim=True)
+        x.scatter_(1, at, kth + 0.02 + 0.9 * (top - kth) * torch.rand((rows, m), generator=g, device="cuda"))
+    _check_compress(x[:, None].to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, top_p, 0.9, g,
+                    staged=order not in ("rank", "reversed"))
