@@ -104,7 +104,9 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
     constexpr int TCH = TileGeom<T>::CHUNKS;
     constexpr int TILE_BYTES = TileGeom<T>::TILE_BYTES, STAGE_BYTES = TileGeom<T>::STAGE_BYTES;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES];
-    __shared__ TileDesc desc[STAGES];
+    // Twice as many descriptors as stages: a warp uses the descriptor of a tile after it has handed the
+    // stage back, and certainly no longer once it hands back the stage's next tile.
+    __shared__ TileDesc desc[2][STAGES];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
             d.c32 = temp_scale(Tb);
             d.c0 = tc * TCH;
             d.mis = sr.mis;
-            desc[s] = d;
+            desc[round & 1][s] = d;
             mbar_arrive(&full[s]);
             r += step_r;
             tc += step_tc;
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, StreamCfg<T>::CTAS_PER_SM) chu
             if (lane == 0) atomicOr(a.status, ST_INTERNAL);
             if (wr == WAIT_LOST) break;
         }
-        const TileDesc d = desc[s];
+        const TileDesc d = desc[round & 1][s];
 #pragma unroll
         for (int q = 0; q < CPW; ++q) {
             const int c = d.c0 + warp * CPW + q;

@@ -717,3 +717,14 @@ def test_random_shapes_and_scales(ps, seed):
         inputs[key] = (inputs[key].float() * scale + shift).to(td)
     r = run_both(ps, w, inputs)
     assert r["status"] == 0
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 1000), ("bf16", 9000), ("f32", 1000), ("f32", 9000)])
+def test_every_tile_of_the_statistics_pass_has_another_temperature(ps, dtype, V):
+    # rows of one and two tiles, many per CTA: each tile comes with the scale and the place of another row
+    w = gen.Workload("t", V=V, B=500, G=8, dtype=dtype, s=1.1, sigma_d=1.5, corr=0.8, sigma_t=1.0, T=None, top_k=16,
+                     top_p=1.0, k_max=16)
+    inputs = gen.make_inputs(w, seed=V, device="cuda")
+    inputs["temperature"] = 0.1 + 3.0 * torch.rand_like(inputs["temperature"])
+    for _ in range(3):
+        assert run_both(ps, w, inputs, check_compress=False)["status"] == 0
