@@ -8,6 +8,8 @@ fallback: a missing library or a non-CUDA tensor raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional, Tuple
 
@@ -23,14 +25,22 @@ _lib = None
 _marshal = None
 
 
+def _import(name: str, path: str):
+    """The extension module `name` from the file `path`."""
+    loader = importlib.machinery.ExtensionFileLoader(name, path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_file_location(name, path, loader=loader))
+    loader.exec_module(module)
+    return module
+
+
 def lib() -> ctypes.CDLL:
     """Load libpicospec.so (built in-tree by build.build()); fail loudly if it is absent."""
     global _lib, _marshal
     if _lib is None:
         path = _build.LIB
-        if not os.path.exists(path) or not os.path.exists(_build.MARSHAL):
+        if not os.path.exists(path) or not os.path.exists(_build.marshal_path()):
             path = _build.build()
-        from . import _marshal as native
+        native = _import(__package__ + "._marshal", _build.marshal_path())
         native.open(path)
         _marshal = native
         L = ctypes.CDLL(path)

@@ -3,6 +3,7 @@ needed to compile)."""
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 import sys
 import sysconfig
@@ -10,7 +11,6 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpicospec.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
 MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 SOURCES = [os.path.join(CSRC, "picospec_api.cu")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -45,12 +45,21 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def marshal_path() -> str:
+    """File of the marshaller for the running Python and the installed torch: it is tied to the binary interface
+    of both, so both are in its name and a build for others is never loaded."""
+    import torch
+    return os.path.join(HERE, "_marshal_torch" + re.sub(r"\W", "_", torch.__version__) + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
 def build_marshal(force: bool = False) -> str:
-    """Compile _marshal.so (csrc/marshal.cpp) against the installed torch."""
+    """Compile the marshaller (csrc/marshal.cpp) against the installed torch if it is missing or older than
+    its sources."""
+    path = marshal_path()
     header = os.path.join(os.path.dirname(HERE), "include", "picospec.h")
-    if not force and os.path.exists(MARSHAL) and all(
-            os.path.getmtime(p) <= os.path.getmtime(MARSHAL) for p in (MARSHAL_SOURCE, header)):
-        return MARSHAL
+    if not force and os.path.exists(path) and all(
+            os.path.getmtime(p) <= os.path.getmtime(path) for p in (MARSHAL_SOURCE, header)):
+        return path
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
@@ -58,13 +67,13 @@ def build_marshal(force: bool = False) -> str:
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
            "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
-           "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], MARSHAL_SOURCE, "-o", MARSHAL,
+           "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"], MARSHAL_SOURCE, "-o", path,
            "-L" + lib, "-Wl,-rpath," + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         sys.stderr.write(res.stdout + res.stderr)
-        raise RuntimeError("g++ failed building _marshal.so")
-    return MARSHAL
+        raise RuntimeError("g++ failed building the marshaller (csrc/marshal.cpp)")
+    return path
 
 
 if __name__ == "__main__":

@@ -6,6 +6,7 @@ import os
 import re
 import subprocess
 import sys
+import sysconfig
 
 import numpy as np
 import pytest
@@ -49,6 +50,24 @@ def test_host_argument_checks_need_no_gpu():
     assert lib.picospec_create(ctypes.byref(h), 0, 0, 1, 1000, 8) == -1          # max_batch <= 0
     assert lib.picospec_create(ctypes.byref(h), 0, 1, 1, 1000, 5000) == -1       # max_k too large
     assert lib.picospec_destroy(None) == -1
+
+
+def test_a_marshaller_of_another_torch_is_not_loaded(monkeypatch):
+    from paper_2603_19133_b200 import binding, buildlib
+    binding.lib()
+    here = buildlib.marshal_path()
+    assert os.path.exists(here) and here.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    built = []
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", "0.0.1+other")
+        m.setattr(binding, "_lib", None)
+        m.setattr(binding, "_marshal", None)
+        m.setattr(buildlib, "build", lambda *a, **k: built.append(buildlib.marshal_path()) or buildlib.LIB)
+        assert buildlib.marshal_path() != here
+        with pytest.raises(ImportError):        # (nothing was built for that version here)
+            binding.lib()
+        assert built == [buildlib.marshal_path()] and binding._lib is None
+    binding.lib()
 
 
 @pytest.mark.skipif(torch.cuda.is_available(), reason="checks the behaviour without a GPU")
