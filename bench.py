@@ -10,6 +10,9 @@ compress filter pass or the verify streaming pass; the other one is listed under
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload config4] [--impl ours|reference]
 
+prints one line of JSON for that workload; the figures of the other workloads, the bandwidth sweep and the
+other entry points go to build/bench_details.json (--details), unless --only-main leaves them out.
+
 With N > 1 and no torchrun environment the script starts N ranks of itself (torch.distributed.run,
 one rank per GPU); every rank runs its own batch (the path shards by sequence, no collective on the
 data path), so scaling is weak.
@@ -746,12 +749,15 @@ def run_ours(args):
             "slow_path_rows_per_step": main["slow_rows_per_step"],
             "compress_redo_rows_per_step": main["redo_rows_per_step"],
             "device_status": main["status"],
-            "other_configs": others,
-            "pipelined": pipelined,
-            "paper_direction": paper_direction,
-            "wire_codec": wire_codec,
-            "vocab_parallel": vocab_parallel,
         }
+        details = {"other_configs": others, "pipelined": pipelined, "paper_direction": paper_direction,
+                   "wire_codec": wire_codec, "vocab_parallel": vocab_parallel}
+        # the line stays short enough for whoever reads it from a log; the other workloads go to a file
+        if any(details.values()):
+            os.makedirs(os.path.dirname(os.path.abspath(args.details)), exist_ok=True)
+            with open(args.details, "w") as f:
+                json.dump({**line, **details}, f, indent=1)
+            line["details"] = os.path.relpath(args.details, ROOT)
         print(json.dumps(line), flush=True)
     if world > 1:
         torch.distributed.barrier()
@@ -788,6 +794,8 @@ def main():
     ap.add_argument("--roofline-launches", type=int, default=64,
                     help="bracketed launches per kernel behind the roofline entry (at most 128 are kept)")
     ap.add_argument("--all-configs", action="store_true", default=True)
+    ap.add_argument("--details", default=os.path.join(ROOT, "build", "bench_details.json"),
+                    help="file for the other workloads' figures (the printed line holds the main workload)")
     ap.add_argument("--only-main", dest="all_configs", action="store_false")
     args = ap.parse_args()
     if args.gpus > 1 and "WORLD_SIZE" not in os.environ:
