@@ -256,7 +256,7 @@ class Context:
         """picospec_compress.  Returns (q_idx [B,G,k_max] i32, q_prob f32, q_count [B,G] i32,
         draft_tok [B,G] i32 or None)."""
         if out is None:
-            B, G, _ = draft_logits.shape
+            B, G, _ = _marshal.logits(draft_logits)
             dev = draft_logits.device
             q_idx = torch.empty((B, G, k_max), dtype=torch.int32, device=dev)
             q_prob = torch.empty((B, G, k_max), dtype=torch.float32, device=dev)
@@ -275,8 +275,8 @@ class Context:
         """picospec_verify.  Returns dict(accept_len [B], p_draft [B,G], resid_mass [B,G],
         borderline_count [1], token [B] or None)."""
         if out is None:
-            B, G = target_logits.shape[0], target_logits.shape[1] - 1
-            dev = target_logits.device
+            B, G1, _ = _marshal.logits(target_logits)
+            G, dev = G1 - 1, target_logits.device
             out = {
                 "accept_len": torch.empty((B,), dtype=torch.int32, device=dev),
                 "p_draft": torch.empty((B, G), dtype=torch.float32, device=dev),
@@ -297,8 +297,8 @@ class Context:
         (its arrays are updated in place; state may alias state_in) or None.  Returns dict(accept_len,
         p_draft, resid_mass, borderline_count, token or None, state [B] i32)."""
         if out is None:
-            B, G = target_logits.shape[0], target_logits.shape[1] - 1
-            dev = target_logits.device
+            B, G1, _ = _marshal.logits(target_logits)
+            G, dev = G1 - 1, target_logits.device
             out = {
                 "accept_len": torch.full((B,), -2, dtype=torch.int32, device=dev),
                 "p_draft": torch.full((B, G), float("nan"), dtype=torch.float32, device=dev),
@@ -321,7 +321,7 @@ class Context:
         if out is not None:
             p_idx, p_prob, p_count = out
         else:
-            B, dev = target_logits.shape[0], target_logits.device
+            B, dev = _marshal.logits(target_logits)[0], target_logits.device
             p_idx = torch.empty((B, k), dtype=torch.int32, device=dev)
             p_prob = torch.empty((B, k), dtype=torch.float32, device=dev)
             p_count = torch.empty((B,), dtype=torch.int32, device=dev)
@@ -337,7 +337,7 @@ class Context:
         if out is not None:
             token, mass = out
         else:
-            B, dev = draft_logits.shape[0], draft_logits.device
+            B, dev = _marshal.logits(draft_logits)[0], draft_logits.device
             token = torch.empty((B,), dtype=torch.int32, device=dev)
             mass = torch.empty((B,), dtype=torch.float32, device=dev) if want_mass else None
         _check(_marshal.edge_resample(self._h.value or 0, draft_logits, temperature, pos, p_idx, p_prob, p_count, u, token,
@@ -376,7 +376,7 @@ class Context:
                         q_idx: torch.Tensor, q_prob: torch.Tensor, q_count: torch.Tensor,
                         u_resample: torch.Tensor, want_mass: bool = True):
         """picospec_residual_sample.  Returns (token [B] i32, mass [B] f32 or None)."""
-        B, dev = target_logits.shape[0], target_logits.device
+        B, dev = _marshal.logits(target_logits)[0], target_logits.device
         token = torch.empty((B,), dtype=torch.int32, device=dev)
         mass = torch.empty((B,), dtype=torch.float32, device=dev) if want_mass else None
         _check(_marshal.residual_sample(self._h.value or 0, target_logits, temperature, pos, q_idx, q_prob, q_count, u_resample,

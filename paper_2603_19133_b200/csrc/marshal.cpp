@@ -291,6 +291,19 @@ PyObject* py_wire_unpack(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
+// logits -> (B, R, V), checked: for calls that allocate their outputs from the shape
+PyObject* py_logits(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    int64_t size[3] = {0, 0, 0};
+    PyObject* ok = guarded(n, 1, [&] {
+        const Logits l(a[0]);
+        size[0] = l.B; size[1] = l.R; size[2] = l.V;
+        return 0;
+    });
+    if (!ok) return nullptr;
+    Py_DECREF(ok);
+    return Py_BuildValue("(LLL)", (long long)size[0], (long long)size[1], (long long)size[2]);
+}
+
 // path of libpicospec.so
 PyObject* py_open(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 1, [&] {
@@ -319,6 +332,7 @@ PyObject* py_open(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 #define PICOSPEC_METHOD(f) {#f, (PyCFunction)(void (*)())py_##f, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PICOSPEC_METHOD(open),
+                         PICOSPEC_METHOD(logits),
                          PICOSPEC_METHOD(compress),
                          PICOSPEC_METHOD(verify),
                          PICOSPEC_METHOD(verify_range),
