@@ -558,7 +558,7 @@ def test_redo_list_does_not_leak_into_later_calls(ps):
         u5 = torch.rand((5, G), generator=g, device="cuda")
         ties = torch.randint(-2, 3, (5, G, V), generator=g, device="cuda").to(torch.bfloat16)
         assert compress_and_check(ties, T5, u5) == 5 * G              # heavy ties: every row is handed over
-        # rows that start 2 bytes off a 16-byte boundary take the direct kernel alone
+        # rows that start 2 bytes off a 16-byte boundary
         pad = (torch.randn((3 * G * (V + 8) + 1,), generator=g, device="cuda") * 2).to(torch.bfloat16)
         odd = pad[1:].view(3, G, V + 8)[:, :, :V]
         assert odd.data_ptr() % 16 != 0
@@ -728,3 +728,35 @@ def test_every_tile_of_the_statistics_pass_has_another_temperature(ps, dtype, V)
     inputs["temperature"] = 0.1 + 3.0 * torch.rand_like(inputs["temperature"])
     for _ in range(3):
         assert run_both(ps, w, inputs, check_compress=False)["status"] == 0
+
+
+@pytest.mark.parametrize("G,V,K", [
+    (2, 40000, 256), (2, 40000, 257),           # k_max: every row's chunk masses, or the sampled row's alone
+    (19, 262144, 16), (20, 262144, 16),         # 20 and 21 rows of 256 chunks: what 40960 bytes hold, and more
+])
+def test_both_sides_of_the_room_for_chunk_masses(ps, G, V, K):
+    w = gen.Workload("t", V=V, B=3, G=G, dtype="bf16", s=1.1, sigma_d=1.5, corr=0.8, sigma_t=1.0, T=None, top_k=K,
+                     top_p=1.0, k_max=K)
+    inputs = gen.make_inputs(w, seed=G + K, device="cuda")
+    # sequences that end at the first row, at a later one, and with the bonus row
+    inputs["u_accept"][0] = 1.0 - 2.0 ** -24
+    inputs["u_accept"][1, :G // 2] = 0.0
+    inputs["u_accept"][2] = 0.0
+    assert run_both(ps, w, inputs)["status"] == 0
+
+
+@pytest.mark.parametrize("K", [128, 129])
+def test_both_sides_of_the_room_for_chunk_masses_of_the_draw_alone(ps, K):
+    w = gen.Workload("t", V=40000, B=12, G=3, dtype="bf16", s=1.1, sigma_d=1.5, corr=0.8, sigma_t=1.0, T=None, top_k=K,
+                     top_p=1.0, k_max=K)
+    inputs = gen.make_inputs(w, seed=K, device="cuda")
+    T, tl, ur = (_np(inputs[n]) for n in ("temperature", "target_logits", "u_resample"))
+    qi, qp, qc, _ = oracle.compress(_np(inputs["draft_logits"]), T, K, 1.0, K, _np(inputs["u_draft"]))
+    pos = (np.arange(w.B) % (w.G + 1)).astype(np.int32)
+    o_tok, o_mass = oracle.residual_sample(tl, T, pos, qi, qp, qc, ur)
+    ctx = _ctx(ps, w.B, w.G, w.V, K)
+    tok, mass = ctx.residual_sample(inputs["target_logits"], inputs["temperature"], _cuda(pos), _cuda(qi), _cuda(qp),
+                                    _cuda(qc), inputs["u_resample"])
+    assert ctx.status(clear=True)[0] == 0
+    assert np.array_equal(_np(tok), o_tok)
+    np.testing.assert_allclose(_np(mass), o_mass, rtol=RTOL, atol=ATOL_MASS)

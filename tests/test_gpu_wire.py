@@ -144,3 +144,24 @@ def test_full_batch_of_the_benchmark_shape_round_trips(ps):
         assert ctx.status(clear=True)[0] == 0
     finally:
         ctx.close()
+
+
+def test_more_rows_than_a_cta_takes_at_a_time(ps):
+    # blocks of rows beyond 256 a CTA, moved in two turns, the last block not full
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    R, K = 8 * sms * 256 + 37, 1
+    rng = np.random.default_rng(82)
+    qc = rng.integers(-1, K + 1, size=R).astype(np.int32)
+    qi = np.where(qc[:, None] > 0, rng.integers(0, 64, size=(R, K)), -1).astype(np.int32)
+    qp = np.where(qc[:, None] > 0, rng.random((R, K)), 0.0).astype(np.float32)
+    ref = wire.pack(qi, qp, qc, 0)
+    ctx = ps.Context(R, 1, 64, K)
+    try:
+        buf, nbytes = ctx.wire_pack(_cuda(qi), _cuda(qp), _cuda(qc))
+        n = int(nbytes.item())
+        assert n == ref.size and np.array_equal(_np(buf[:n]), ref)
+        ui, up, uc = ctx.wire_unpack(buf, n, R, K)
+        assert np.array_equal(_np(ui), qi) and np.array_equal(_np(up), qp) and np.array_equal(_np(uc), qc)
+        assert ctx.status(clear=True)[0] == 0
+    finally:
+        ctx.close()
