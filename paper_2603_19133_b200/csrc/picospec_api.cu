@@ -249,7 +249,7 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
 }
 
 // Shared memory of the verify finish kernel: the chunk masses of every row that it reads where they fit
-// the 48 KB that need no opt-in beside the kernel's static 6 KB (up to 11 rows of 262144 entries) and the
+// the 48 KB that need no opt-in beside the kernel's static 6 KB (up to 20 rows of 262144 entries) and the
 // warp that reads a row has few entries to take out of them (about 200 cycles per 32); else those of the
 // sampled row, formed by the whole CTA once the row is known (about 3300 cycles).
 size_t finish_masses_bytes(VerifyArgs& a) {
