@@ -63,6 +63,7 @@ struct CsRowMeta {
     int flags;
     float ref_off;    // fp32(ref * c32): reference of the streamed normaliser
     unsigned thr_key; // the row's final bound: every survivor's orderable logit is at least this
+    int top;          // bin coordinate of the largest value counted
     double z_stream;  // sum of 2^(l * c32 - ref_off) over the row (top-p only)
 };
 
@@ -227,11 +228,8 @@ __device__ __forceinline__ unsigned coord_code(int G) {
     }
     return (unsigned)(0x7FFF - ((0x7FFF - G) + CS_DEAD));
 }
-// bin of an orderable key at or above the bound whose coordinate is g0, the last of N bins open-ended
-template <int N> __device__ __forceinline__ int hist_bin_in(unsigned okey, int g0) {
-    return min(bin_coord(okey >> 16) - g0, N - 1);
-}
-__device__ __forceinline__ int hist_bin(unsigned okey, int g0) { return hist_bin_in<CS_BINS>(okey, g0); }
+// bin of an orderable key at or above the bound whose coordinate is g0, the last one open-ended
+__device__ __forceinline__ int hist_bin(unsigned okey, int g0) { return min(bin_coord(okey >> 16) - g0, CS_BINS - 1); }
 __device__ __forceinline__ void hist_add(unsigned* hist, int bin) {
     atomicAdd(&hist[bin >> 1], (bin & 1) ? 0x10000u : 1u);
     atomicAdd(&hist[CS_BINS / 2 + (bin >> 5)], 1u);
@@ -387,6 +385,17 @@ __device__ __noinline__ int crowded_chunk(unsigned mask, int n, int copy) {
         refresh_threshold(hist, *cs, k, k, lane);
         __syncwarp();
     } else {
+        // Values that share the bound's own 16-bit code cannot be told apart by any bound: if, behind the first
+        // tile, they alone fill half a region, or if another warp has given up, so does this one.
+        const unsigned code = *(volatile unsigned*)&cs->thr_key >> 16;
+        int same = 0;
+        for (unsigned m = mask; m; m &= m - 1u)
+            same += staged_key<T>(chunk, bit_offset(__ffs(m) - 1, lane, (const T*)nullptr)) >> 16 == code ? 1 : 0;
+        __syncwarp();
+        same = __reduce_add_sync(0xffffffffu, same);
+        if ((same > REGION / 2 && __any_sync(0xffffffffu, *(volatile int*)&cs->seen > WARPS)) ||
+            __any_sync(0xffffffffu, *(volatile int*)&cs->overflow))
+            return -1;
         if (lane == 0) *(volatile unsigned*)&cs->certain = 1u;
         __threadfence_block();
         __syncwarp();
@@ -751,7 +760,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
                 workers_sync();
                 first_bound<Geom, SPREAD ? 3 : 1>(parity ^ 1, pc.area);
                 if (STATS) ref_off = __fmul_rn(from_orderable(*(volatile unsigned*)&cs.top_key), c32);
-                if (*(volatile unsigned*)&cs.thr_key < 0x00800000u) {
+                if (__any_sync(0xffffffffu, *(volatile unsigned*)&cs.thr_key < 0x00800000u)) {
                     // no finite bound (rows of -inf): everything would pass, padding included
                     if (lane == 0) cs.overflow = 1;
                     row_chunks = 0;
@@ -826,10 +835,12 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
         workers_sync();     // every candidate is counted, every flag is set
         const bool piece_ok = valid && !*(volatile int*)&cs.overflow && !*(volatile int*)&cta.abort;
         unsigned thr_final = *(volatile unsigned*)&cs.thr_key;
+        int top = 0;
         if (piece_ok) {
             // the final bound, by every warp for itself (all get the same): no second barrier for it
             const bool certain = !SPREAD || whole || *(volatile unsigned*)&cs.certain;
             const int found = kth_bin(hist, certain ? fb.k : bound_rank(fb.k, fb.per_tile * (float)(pc.tile1 - pc.tile0)), lane);
+            if (warp == 0) top = *(volatile int*)&cs.g0 + max(kth_bin(hist, 1, lane), 0);
             if (found >= 0) thr_final = max(thr_final, coord_code(*(volatile int*)&cs.g0 + found) << 16);
             // every warp filters its own region and appends to the piece's scratch area
             u64* dst = a.surv_keys + (long long)pc.area * fb.surv_cap;
@@ -859,6 +870,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
             meta.flags = flags;
             meta.ref_off = ref_off;
             meta.thr_key = thr_final;
+            meta.top = top;
             meta.z_stream = zs;
             a.surv_meta[pc.area] = meta;
             cs_reset(cs);       // this copy is used again by the piece after the next one
@@ -875,8 +887,8 @@ constexpr int CS_MAX_PIECES = 8;    // most pieces a row is dealt in
 // A group of TPR threads finishes a row: the CTA's 256 threads, or a warp (four rows per CTA).
 //   CAP     keys at or above the boundary bin the group can hold (more: the direct kernel)
 //   KCAP    largest k_eff
-//   BINS    bins of the counting sort: one per 16-bit logit code (bin_coord), counted up from the row's
-//           bound, i.e. BINS / 128 binades for values away from zero; the last one is open-ended
+//   BINS    bins of the counting sort, counted up from the row's bound: one or more per 16-bit logit code
+//           (bin_coord); BINS / 128 binades at least for values away from zero; the last one is open-ended
 template <int TPR> struct FinishGeom;
 template <> struct FinishGeom<32> {
     static constexpr int ROWS = 4, CAP = 512, KCAP = 128, BINS = 512, AHEAD = 4, HOLD = 4, CTAS = 7;
@@ -897,15 +909,18 @@ struct CsFinishShared {
 
 // A row's survivors lie in one scratch area, or in those of its pieces if it was dealt in pieces.  A
 // survivor set holds all of a piece's elements at or above its final bound; the row's k best are among
-// the survivors if k of them reach the largest of the pieces' bounds.  The k best are found and put in order by a counting sort over the 16-bit codes: count
-// the keys per bin, sum from the top, move every key that is not below the bin of the k-th into its
-// bin's stretch, then place each by its rank among the keys of its own stretch (all pairs: a
-// stretch holds the ties of one code, a few keys).  Bound by latency for few rows (meta, survivors, six
+// the survivors if k of them reach the largest of the pieces' bounds.  The k best are found and put in
+// order by a counting sort over the 16-bit codes and as much of what orders the keys of one code as the
+// bins have room for: count the keys per bin, sum from the top, move every key that is not below the
+// bin of the k-th into its bin's stretch, then place each by its rank among the keys of its own stretch
+// (all pairs: a few keys).  Bound by latency for few rows (meta, survivors, six
 // short phases: about 9 K cycles) and by issue for many.  It replaces a trim and a bitonic network over
 // the survivors, which was 32 of 51 K cycles of a row with k = 1024: 172 -> 72 us for 4096 rows with
 // k = 1024, 22 -> 15.5 us for 1536 rows with k = 256, 41 -> 9.1 us for 4096 rows with k = 8 (a warp
 // each), 16.4 -> 7.0 us for 40 rows in eight pieces with k = 64 (the pieces' records are read by one
 // lane each instead of one after the other).
+// With one bin per code, bf16 logits around 30 / 100 (k = 1024) took 95 / 267 us for 1536 rows; now 37 / 37, and
+// 33 around 0.
 template <typename T, bool STATS, int TPR>
 __global__ void __launch_bounds__(TPR * FinishGeom<TPR>::ROWS, FinishGeom<TPR>::CTAS)
 compress_finish_kernel(CompressArgs a, FilterPlan plan) {
@@ -941,7 +956,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
     const float Tb = a.temperature[row / a.G];
     // ---- the pieces, one per lane: flags, the row's bound, where each piece's survivors begin -------
     CsRowMeta meta;
-    meta.count = 0; meta.flags = 0; meta.thr_key = 0u; meta.ref_off = 0.f; meta.z_stream = 0.0;
+    meta.count = 0; meta.flags = 0; meta.thr_key = 0u; meta.top = 0; meta.ref_off = 0.f; meta.z_stream = 0.0;
     if (lane < nareas && (!split_row || lane == 0 || plan_piece_tile(plan, lane + 1) > plan_piece_tile(plan, lane)))
         meta = a.surv_meta[area0 + lane];
     __syncwarp();
@@ -973,6 +988,18 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
                 }
             return src[(long long)p * surv_cap + (i - b)];
         };
+        // As many bins per 16-bit code as the row's codes leave room for, by what orders the keys of one code: the
+        // low half of the logit, and for 16-bit logits, where these are all equal, the index (squeezed codes
+        // have one bin).
+        const int span = max(__reduce_max_sync(0xffffffffu, meta.top), g0) - g0 + 1;
+        const int lg = 31 - __clz(max(Geom::BINS / span, 1));
+        const int drop = max(32 - __clz(a.V) - lg, 0);
+        auto bin_of = [&](u64 key) {
+            const int c = bin_coord((unsigned)(key >> 48));
+            int sub = sizeof(T) == 2 ? (int)(((unsigned)(a.V - 1) - ~(unsigned)key) >> drop) : (int)(((unsigned)(key >> 32) & 0xffffu) << lg >> 16);
+            if ((unsigned)(c - 0x7FFF) <= 1u) sub = 0;
+            return min(((c - g0) << lg) + sub, Geom::BINS - 1);
+        };
         // the first HOLD survivors of each thread stay in registers, those below the bound as zero
 #pragma unroll
         for (int x = 0; x < HOLD; ++x) {
@@ -982,7 +1009,6 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
         }
         group_sync<TPR>();      // the bins are zero
         // ---- count ------------------------------------------------------------------------------
-        auto bin_of = [&](u64 key) { return hist_bin_in<Geom::BINS>((unsigned)(key >> 32), g0); };
 #pragma unroll
         for (int x = 0; x < HOLD; ++x)
             if (held[x]) atomicAdd(&bins[bin_of(held[x])], 1);

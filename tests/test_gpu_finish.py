@@ -126,3 +126,19 @@ def test_vocabularies_with_an_order(V, k, top_p, order, dtype):
         x.scatter_(1, at, kth + 0.02 + 0.9 * (top - kth) * torch.rand((rows, m), generator=g, device="cuda"))
     _check_compress(x[:, None].to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, top_p, 0.9, g,
                     staged=order not in ("rank", "reversed"))
+
+
+@pytest.mark.parametrize("dtype,rows,V,k,offset", [
+    ("bf16", 9, 32768, 1024, 100.0),         # several hundred keys of one code, for a CTA
+    ("f32", 9, 32768, 1024, 100.0),
+    ("f32", 5, 131072, 1024, 100.0),         # the same put together from pieces
+    ("f32", 9, 32768, 300, 30.0),            # stretches below and above the limit in one row
+    ("bf16", 9, 16384, 128, 100.0),          # for a warp
+    ("f32", 9, 16384, 128, 100.0),
+    ("f32", 9, 16384, 100, 100.0),
+])
+def test_many_keys_of_one_code(dtype, rows, V, k, offset):
+    # a common offset leaves few 16-bit codes to the k largest: a network orders them instead of the counts
+    g = torch.Generator(device="cuda").manual_seed(V + k)
+    x = 2.0 * torch.randn((rows, 1, V), generator=g, device="cuda") + offset
+    _check_compress(x.to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, 1.0, 0.9, g, staged=k > 128)
