@@ -52,6 +52,13 @@ struct CompressArgs {
     CsRowMeta* surv_meta;
 };
 
+// entries kept of a row before a top-p cut
+__device__ __forceinline__ int kept_entries(const CompressArgs& a) {
+    int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
+    if (k_eff > a.k_max) k_eff = a.k_max;
+    return k_eff > a.V ? a.V : k_eff;
+}
+
 // logits row behind output row `row`, or -1 if its position is out of range
 __device__ __forceinline__ long long source_row(const CompressArgs& a, int row) {
     if (!a.row_pos) return row;
@@ -398,162 +405,158 @@ __device__ __forceinline__ void finish_row(const CompressArgs& a, int row, const
     else finish_row_ranks<PRECISE, 4, TPR>(a, row, keys, k_eff, Tb, Z, sh);
 }
 
+// One row from its logits to its sparse row, by the 256 threads of a CTA.  cand [CAND_CAP], keep [MAX_K]: shared memory.
 template <typename T, bool ALIGNED, bool STATS>
-__global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
-    grid_dependency_sync();
-    extern __shared__ u64 smem64[];
-    u64* cand = smem64;
-    u64* keep = cand + CAND_CAP;
-    __shared__ CompressShared sh;
+__device__ __forceinline__ void compress_row(const CompressArgs& a, int row, int k_eff, u64* cand, u64* keep, CompressShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr bool LOGIT16 = sizeof(T) == 2;
-    const int rows = a.B * a.G;
     const int iters = (a.nch + WARPS - 1) / WARPS;
-    int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
-    if (k_eff > a.k_max) k_eff = a.k_max;
-    if (k_eff > a.V) k_eff = a.V;
-
-    // a call that goes through this kernel alone clears both of the next call's counters, as the
-    // staged filter kernel does (the redo-list launch of a staged call must not: the filter did)
-    if (blockIdx.x == 0 && tid == 0 && !a.use_redo_list) {
-        *a.queue_count_next = 0;
-        *a.redo_count_next = 0;
+    const int b = row / a.G;
+    const float Tb = a.temperature[b];
+    workers_sync();
+    if (!temp_ok(Tb)) {
+        emit_invalid_row<THREADS>(a, row);
+        if (tid == 0) atomicOr(a.status, ST_TEMPERATURE);
+        return;
     }
-    const int nwork = a.use_redo_list ? *a.redo_count : rows;
+    const float c32 = temp_scale(Tb);
+    const long long srow = source_row(a, row);
+    if (srow < 0) {
+        emit_invalid_row<THREADS>(a, row);
+        if (tid == 0) atomicOr(a.status, ST_RANGE);
+        return;
+    }
+    const T* rowp = reinterpret_cast<const T*>(a.logits) + srow * a.row_stride;
+    if (tid == 0) {
+        sh.count = 0;
+        sh.thr = -CUDART_INF_F;
+        sh.nan = 0;
+    }
+    workers_sync();
 
-    for (int wi = blockIdx.x; wi < nwork; wi += gridDim.x) {
-        const int row = a.use_redo_list ? a.redo_rows[wi] : wi;
-        const int b = row / a.G;
-        const float Tb = a.temperature[b];
-        workers_sync();
-        if (!temp_ok(Tb)) {
-            emit_invalid_row<THREADS>(a, row);
-            if (tid == 0) atomicOr(a.status, ST_TEMPERATURE);
-            continue;
-        }
-        const float c32 = temp_scale(Tb);
-        const long long srow = source_row(a, row);
-        if (srow < 0) {
-            emit_invalid_row<THREADS>(a, row);
-            if (tid == 0) atomicOr(a.status, ST_RANGE);
-            continue;
-        }
-        const T* rowp = reinterpret_cast<const T*>(a.logits) + srow * a.row_stride;
-        if (tid == 0) {
-            sh.count = 0;
-            sh.thr = -CUDART_INF_F;
-            sh.nan = 0;
-        }
-        workers_sync();
+    // running softmax statistics of this warp: fp32 lane sums relative to the warp's running
+    // maximum; when the maximum rises the sums are folded into a double and rescaled exactly
+    float runM = -CUDART_INF_F, runOff = 0.f, acc = 0.f;
+    double folded = 0.0;
 
-        // running softmax statistics of this warp: fp32 lane sums relative to the warp's running
-        // maximum; when the maximum rises the sums are folded into a double and rescaled exactly
-        float runM = -CUDART_INF_F, runOff = 0.f, acc = 0.f;
-        double folded = 0.0;
-
-        ChunkRegs<T> bufA, bufB;
-        if (warp < a.nch) bufA.template load<ALIGNED>(rowp, warp * CHUNK, a.V, lane);
-        auto body = [&](ChunkRegs<T>& cur, ChunkRegs<T>& nxt, int it) {
-            const int c = it * WARPS + warp;
-            const int cn = c + WARPS;
-            if (it + 1 < iters && cn < a.nch) nxt.template load<ALIGNED>(rowp, cn * CHUNK, a.V, lane);
-            const float thr = sh.thr;
-            if (c < a.nch) {
-                const int v0 = c * CHUNK;
-                const float lm = cur.lane_max();
-                if (lm != lm) sh.nan = 1;
-                if (STATS) {
-                    const float cmx = warp_max(lm);
-                    if (cmx > runM) {
-                        const float newOff = __fmul_rn(cmx, c32);
-                        const double s = (double)warp_sum(acc);
-                        folded = runM > -CUDART_INF_F ? (folded + s) * exp2((double)runOff - (double)newOff) : 0.0;
-                        acc = 0.f;
-                        runM = cmx;
-                        runOff = newOff;
-                    }
-                    if (runM > -CUDART_INF_F && runM < CUDART_INF_F) acc += lane_exp_sum(cur, c32, runOff);
+    ChunkRegs<T> bufA, bufB;
+    if (warp < a.nch) bufA.template load<ALIGNED>(rowp, warp * CHUNK, a.V, lane);
+    auto body = [&](ChunkRegs<T>& cur, ChunkRegs<T>& nxt, int it) {
+        const int c = it * WARPS + warp;
+        const int cn = c + WARPS;
+        if (it + 1 < iters && cn < a.nch) nxt.template load<ALIGNED>(rowp, cn * CHUNK, a.V, lane);
+        const float thr = sh.thr;
+        if (c < a.nch) {
+            const int v0 = c * CHUNK;
+            const float lm = cur.lane_max();
+            if (lm != lm) sh.nan = 1;
+            if (STATS) {
+                const float cmx = warp_max(lm);
+                if (cmx > runM) {
+                    const float newOff = __fmul_rn(cmx, c32);
+                    const double s = (double)warp_sum(acc);
+                    folded = runM > -CUDART_INF_F ? (folded + s) * exp2((double)runOff - (double)newOff) : 0.0;
+                    acc = 0.f;
+                    runM = cmx;
+                    runOff = newOff;
                 }
-                if (lm >= thr) {
+                if (runM > -CUDART_INF_F && runM < CUDART_INF_F) acc += lane_exp_sum(cur, c32, runOff);
+            }
+            if (lm >= thr) {
 #pragma unroll
-                    for (int j = 0; j < ChunkRegs<T>::NVEC; ++j) {
-                        if (cur.vec_max(j) >= thr) {
-                            constexpr int VEC = ChunkRegs<T>::VEC;
+                for (int j = 0; j < ChunkRegs<T>::NVEC; ++j) {
+                    if (cur.vec_max(j) >= thr) {
+                        constexpr int VEC = ChunkRegs<T>::VEC;
 #pragma unroll
-                            for (int e = 0; e < VEC; ++e) {
-                                const float l = cur.value(j * VEC + e);
-                                const int v = v0 + ChunkRegs<T>::offset(j * VEC + e, lane);
-                                if (l >= thr && v < a.V) cand[atomicAdd(&sh.count, 1)] = make_key(l, v);
-                            }
+                        for (int e = 0; e < VEC; ++e) {
+                            const float l = cur.value(j * VEC + e);
+                            const int v = v0 + ChunkRegs<T>::offset(j * VEC + e, lane);
+                            if (l >= thr && v < a.V) cand[atomicAdd(&sh.count, 1)] = make_key(l, v);
                         }
                     }
                 }
             }
-            workers_sync();
-            if (sh.count > CAND_CAP - ITER_ELEMS) {
-                const int count = sh.count;
-                workers_sync();
-                keep_top_k<LOGIT16>(cand, keep, count, k_eff, sh);
-                // sh.count == k_eff now; the k-th key's logit is the new admission threshold
-                float mn = CUDART_INF_F;
-                for (int i = tid; i < k_eff; i += THREADS) mn = fminf(mn, key_logit(cand[i]));
-                mn = -warp_max(-mn);
-                if (lane == 0) sh.wM[warp] = mn;
-                workers_sync();
-                if (tid == 0) {
-                    float m = sh.wM[0];
-                    for (int w = 1; w < WARPS; ++w) m = fminf(m, sh.wM[w]);
-                    sh.thr = m;
-                }
-                workers_sync();
-            }
-        };
-        for (int it = 0; it < iters; it += 2) {
-            body(bufA, bufB, it);
-            if (it + 1 < iters) body(bufB, bufA, it + 1);
-        }
-
-        // ---- row statistics -----------------------------------------------------------------
-        double Z = 0.0;
-        if (STATS) {
-            const double s = (double)warp_sum(acc);
-            if (lane == 0) {
-                sh.wM[warp] = runM;
-                sh.wS[warp] = folded + s;   // relative to runOff = fp32(runM * c32)
-            }
-            workers_sync();
-            float m = sh.wM[0];
-            for (int w = 1; w < WARPS; ++w) m = fmaxf(m, sh.wM[w]);
-            if (m > -CUDART_INF_F && m < CUDART_INF_F) {
-                const double off = (double)__fmul_rn(m, c32);
-                for (int w = 0; w < WARPS; ++w)
-                    if (sh.wM[w] > -CUDART_INF_F) Z += sh.wS[w] * exp2((double)__fmul_rn(sh.wM[w], c32) - off);
-                Z *= stream_sum_scale(m, c32);
-            }
         }
         workers_sync();
-
-        // ---- final selection and order --------------------------------------------------------
-        int count = sh.count;
-        workers_sync();
-        if (count > k_eff) {
+        if (sh.count > CAND_CAP - ITER_ELEMS) {
+            const int count = sh.count;
+            workers_sync();
             keep_top_k<LOGIT16>(cand, keep, count, k_eff, sh);
-            count = k_eff;
+            // sh.count == k_eff now; the k-th key's logit is the new admission threshold
+            float mn = CUDART_INF_F;
+            for (int i = tid; i < k_eff; i += THREADS) mn = fminf(mn, key_logit(cand[i]));
+            mn = -warp_max(-mn);
+            if (lane == 0) sh.wM[warp] = mn;
+            workers_sync();
+            if (tid == 0) {
+                float m = sh.wM[0];
+                for (int w = 1; w < WARPS; ++w) m = fminf(m, sh.wM[w]);
+                sh.thr = m;
+            }
+            workers_sync();
         }
-        int n2 = 1;
-        while (n2 < k_eff) n2 <<= 1;
-        for (int i = tid; i < n2; i += THREADS) keep[i] = i < count ? cand[i] : 0ull;
-        bitonic_sort_desc(keep, n2);
-
-        const float top = key_logit(keep[0]);
-        const bool bad = sh.nan || !(top > -CUDART_INF_F) || !(top < CUDART_INF_F) || (STATS && !(Z > 0.0));
-        if (bad) {
-            emit_invalid_row<THREADS>(a, row);
-            if (tid == 0) atomicOr(a.status, ST_LOGIT);
-            continue;
-        }
-        finish_row<false, THREADS>(a, row, keep, k_eff, Tb, Z, &sh.row);
+    };
+    for (int it = 0; it < iters; it += 2) {
+        body(bufA, bufB, it);
+        if (it + 1 < iters) body(bufB, bufA, it + 1);
     }
+
+    // ---- row statistics -----------------------------------------------------------------
+    double Z = 0.0;
+    if (STATS) {
+        const double s = (double)warp_sum(acc);
+        if (lane == 0) {
+            sh.wM[warp] = runM;
+            sh.wS[warp] = folded + s;   // relative to runOff = fp32(runM * c32)
+        }
+        workers_sync();
+        float m = sh.wM[0];
+        for (int w = 1; w < WARPS; ++w) m = fmaxf(m, sh.wM[w]);
+        if (m > -CUDART_INF_F && m < CUDART_INF_F) {
+            const double off = (double)__fmul_rn(m, c32);
+            for (int w = 0; w < WARPS; ++w)
+                if (sh.wM[w] > -CUDART_INF_F) Z += sh.wS[w] * exp2((double)__fmul_rn(sh.wM[w], c32) - off);
+            Z *= stream_sum_scale(m, c32);
+        }
+    }
+    workers_sync();
+
+    // ---- final selection and order --------------------------------------------------------
+    int count = sh.count;
+    workers_sync();
+    if (count > k_eff) {
+        keep_top_k<LOGIT16>(cand, keep, count, k_eff, sh);
+        count = k_eff;
+    }
+    int n2 = 1;
+    while (n2 < k_eff) n2 <<= 1;
+    for (int i = tid; i < n2; i += THREADS) keep[i] = i < count ? cand[i] : 0ull;
+    bitonic_sort_desc(keep, n2);
+
+    const float top = key_logit(keep[0]);
+    const bool bad = sh.nan || !(top > -CUDART_INF_F) || !(top < CUDART_INF_F) || (STATS && !(Z > 0.0));
+    if (bad) {
+        emit_invalid_row<THREADS>(a, row);
+        if (tid == 0) atomicOr(a.status, ST_LOGIT);
+        return;
+    }
+    finish_row<false, THREADS>(a, row, keep, k_eff, Tb, Z, &sh.row);
+}
+
+template <typename T, bool ALIGNED, bool STATS>
+__global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
+    grid_dependency_sync();
+    extern __shared__ u64 smem64[];
+    __shared__ CompressShared sh;
+    // a call that goes through this kernel alone clears both of the next call's counters, as the
+    // staged filter kernel does (the redo-list launch of a staged call must not: the filter did)
+    if (blockIdx.x == 0 && threadIdx.x == 0 && !a.use_redo_list) {
+        *a.queue_count_next = 0;
+        *a.redo_count_next = 0;
+    }
+    const int nwork = a.use_redo_list ? *a.redo_count : a.B * a.G, k_eff = kept_entries(a);
+    for (int wi = blockIdx.x; wi < nwork; wi += gridDim.x)
+        compress_row<T, ALIGNED, STATS>(a, a.use_redo_list ? a.redo_rows[wi] : wi, k_eff, smem64, smem64 + CAND_CAP, sh);
 }
 
 // Double-precision redo of the top-p cut for the rows in the queue, in one kernel: the exact chunk
@@ -573,9 +576,7 @@ __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs 
     if (nq == 0) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = warp >> 2, quarter = warp & 3;
-    int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
-    if (k_eff > a.k_max) k_eff = a.k_max;
-    if (k_eff > a.V) k_eff = a.V;
+    const int k_eff = kept_entries(a);
     const long long total = (long long)nq * a.nch;
     const long long pairs = (total + 1) / 2;
     for (long long pi = blockIdx.x; pi < pairs; pi += gridDim.x) {

@@ -921,23 +921,19 @@ struct CsFinishShared {
 // lane each instead of one after the other).
 // With one bin per code, bf16 logits around 30 / 100 (k = 1024) took 95 / 267 us for 1536 rows; now 37 / 37, and
 // 33 around 0.
+//
+// A group finishes a row: its part of the dynamic shared memory fin_mem is number `group`, its exchange area fs.
+// Returns false if the row has to go through compress_row: a piece's candidates did not fit, or there are too
+// many ties.
 template <typename T, bool STATS, int TPR>
-__global__ void __launch_bounds__(TPR * FinishGeom<TPR>::ROWS, FinishGeom<TPR>::CTAS)
-compress_finish_kernel(CompressArgs a, FilterPlan plan) {
+__device__ __forceinline__ bool finish_survivors(const CompressArgs& a, const FilterPlan& plan, int row, int k_eff, unsigned char* fin_mem,
+                                                 int group, CsFinishShared& fs) {
     typedef FinishGeom<TPR> Geom;
     constexpr int AHEAD = Geom::AHEAD, HOLD = Geom::HOLD, PER = Geom::BINS / TPR;
-    extern __shared__ __align__(16) unsigned char fin_mem[];
-    __shared__ CsFinishShared shared[Geom::ROWS];
     const int tid = group_tid<TPR>(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int group = TPR == 32 ? warp : 0;
-    const int row = blockIdx.x * Geom::ROWS + group;
-    CsFinishShared& fs = shared[group];
     u64* stretch = reinterpret_cast<u64*>(fin_mem) + group * (Geom::CAP + Geom::KCAP);
     u64* keys = stretch + Geom::CAP;
     int* bins = reinterpret_cast<int*>(reinterpret_cast<u64*>(fin_mem) + Geom::ROWS * (Geom::CAP + Geom::KCAP)) + group * Geom::BINS;
-    int k_eff = a.top_k > 0 ? a.top_k : a.k_max;
-    if (k_eff > a.k_max) k_eff = a.k_max;
-    if (k_eff > a.V) k_eff = a.V;
     const int surv_cap = cs_survivor_cap(a.k_max);
     // the scratch areas that hold this row: its own, or those of its pieces if it was dealt in pieces
     const int whole_rows = plan.q * plan.grid;
@@ -947,7 +943,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
     for (int x = tid; x < Geom::BINS / 4; x += TPR) reinterpret_cast<int4*>(bins)[x] = make_int4(0, 0, 0, 0);
     if (tid == 0) fs.overflow = 0;
     grid_dependency_sync();
-    if (row >= plan.rows) return;       // (a warp beyond the last row)
+    if (row >= plan.rows) return true;  // (a warp beyond the last row)
     const u64* src = a.surv_keys + (long long)area0 * surv_cap;
     // the first area's first slots exist for every k_max: requested before their number is known
     u64 held[HOLD];
@@ -966,7 +962,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
         emit_invalid_row<TPR>(a, row);
         if (tid == 0 && !(flags & CSF_ABORT))
             atomicOr(a.status, (flags & CSF_TEMPERATURE) ? ST_TEMPERATURE : (flags & CSF_RANGE) ? ST_RANGE : ST_LOGIT);
-        return;
+        return true;
     }
     int begin[CS_MAX_PIECES], m = 0;        // begin[p]: flat number of piece p's first survivor
 #pragma unroll
@@ -1096,14 +1092,7 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
             group_sync<TPR>();
         }
     }
-    if (redo) {
-        // a piece's candidates did not fit, or too many ties: the direct kernel writes this row
-        if (tid == 0) {
-            a.redo_rows[atomicAdd(a.redo_count, 1)] = row;
-            atomicAdd(a.redo_total, 1ull);
-        }
-        return;
-    }
+    if (redo) return false;
     const float top = key_logit(keys[0]);
     double Z = 0.0;
     if (STATS) {
@@ -1117,9 +1106,42 @@ compress_finish_kernel(CompressArgs a, FilterPlan plan) {
     if (bad) {
         emit_invalid_row<TPR>(a, row);
         if (tid == 0) atomicOr(a.status, ST_LOGIT);
-        return;
+        return true;
     }
     finish_row<false, TPR>(a, row, keys, k_eff, Tb, Z, &fs.row);
+    return true;
+}
+
+// Many rows: those that have to go through compress_row are listed for the kernel behind this one.
+template <typename T, bool STATS, int TPR>
+__global__ void __launch_bounds__(TPR * FinishGeom<TPR>::ROWS, FinishGeom<TPR>::CTAS)
+compress_finish_kernel(CompressArgs a, FilterPlan plan) {
+    extern __shared__ __align__(16) unsigned char fin_mem[];
+    __shared__ CsFinishShared shared[FinishGeom<TPR>::ROWS];
+    const int group = TPR == 32 ? threadIdx.x >> 5 : 0;
+    const int row = blockIdx.x * FinishGeom<TPR>::ROWS + group;
+    if (!finish_survivors<T, STATS, TPR>(a, plan, row, kept_entries(a), fin_mem, group, shared[group]) && group_tid<TPR>() == 0) {
+        a.redo_rows[atomicAdd(a.redo_count, 1)] = row;
+        atomicAdd(a.redo_total, 1ull);
+    }
+}
+
+// Few rows (all of them resident at two CTAs per SM, so that a row that is read again takes no longer than in a kernel
+// of its own): the CTA that finishes a row also takes it through compress_row if need be.  A kernel behind this one
+// for listed rows is a launch of 0.9 to 1.3 us that normally finds an empty list.  With it the finish was 7.4 us (8 x 5,
+// V = 128256, k = 64), 4.7 (1 x 4, V = 32000) and 9.3 (48 x 5, fp32, by warps); now 6.9, 4.3 and 6.6, and no launch behind it.
+template <typename T, bool ALIGNED, bool STATS>
+__global__ void __launch_bounds__(THREADS, 2)
+compress_finish_few_kernel(const __grid_constant__ CompressArgs a, const __grid_constant__ FilterPlan plan) {
+    extern __shared__ __align__(16) unsigned char fin_mem[];
+    __shared__ CsFinishShared fs;
+    __shared__ CompressShared sh;
+    const int row = blockIdx.x, k_eff = kept_entries(a);
+    if (!finish_survivors<T, STATS, THREADS>(a, plan, row, k_eff, fin_mem, 0, fs)) {
+        if (threadIdx.x == 0) atomicAdd(a.redo_total, 1ull);
+        u64* cand = reinterpret_cast<u64*>(fin_mem);
+        compress_row<T, ALIGNED, STATS>(a, row, k_eff, cand, cand + CAND_CAP, sh);
+    }
 }
 
 }  // namespace picospec

@@ -102,6 +102,10 @@ template <typename T> void set_compress_attrs() {
     cudaFuncSetAttribute(compress_kernel<T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
     cudaFuncSetAttribute(compress_kernel<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
     cudaFuncSetAttribute(compress_kernel<T, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
+    cudaFuncSetAttribute(compress_finish_few_kernel<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
+    cudaFuncSetAttribute(compress_finish_few_kernel<T, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
+    cudaFuncSetAttribute(compress_finish_few_kernel<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
+    cudaFuncSetAttribute(compress_finish_few_kernel<T, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, COMPRESS_SMEM);
 }
 
 template <typename T, bool SMALL, bool SPREAD> cudaError_t set_filter_attrs() {
@@ -170,6 +174,16 @@ void launch_compress_finish(const CompressArgs& a, const FilterPlan& plan, bool 
     else launch_chained(compress_finish_kernel<T, false, TPR>, grid, TPR * ROWS, finish_smem_bytes<TPR>(), s, a, plan);
 }
 
+// a CTA per row (few rows)
+template <typename T>
+void launch_compress_finish_few(const CompressArgs& a, const FilterPlan& plan, bool aligned, bool stats, cudaStream_t s) {
+    static_assert(finish_smem_bytes<THREADS>() <= COMPRESS_SMEM, "");
+    void (*kern)(CompressArgs, FilterPlan) =
+        aligned ? (stats ? compress_finish_few_kernel<T, true, true> : compress_finish_few_kernel<T, true, false>)
+                : (stats ? compress_finish_few_kernel<T, false, true> : compress_finish_few_kernel<T, false, false>);
+    launch_chained(kern, plan.rows, THREADS, COMPRESS_SMEM, s, a, plan);
+}
+
 template <typename T, bool STATS, bool SMALL> auto filter_kernel(const FilterBound& fb) {
     return fb.spread ? compress_filter_kernel<T, STATS, SMALL, true> : compress_filter_kernel<T, STATS, SMALL, false>;
 }
@@ -213,23 +227,27 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         }
         cudaError_t e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;
+        const bool few = rows <= 2 * ctx->num_sms;      // (compress_finish_few_kernel)
         {
             ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_FINISH, 2, s);
             // A warp per row while the row that has most survivors has few of them: a row dealt in 8 pieces
             // at k = 64 (560 survivors) took 15.9 us of a call by warps, 7.0 by CTAs; 4096 whole rows at
             // k = 8 take 9.1 us by warps and took 41 with a CTA and a sort network each.
             const int survivors = plan.rem > 0 ? plan.split * bound_rank(k_eff, 1.0f / (float)plan.split) : k_eff;
-            if (survivors <= FinishGeom<32>::KCAP) launch_compress_finish<T, 32>(a, plan, stats, s);
+            if (few) launch_compress_finish_few<T>(a, plan, aligned, stats, s);
+            else if (survivors <= FinishGeom<32>::KCAP) launch_compress_finish<T, 32>(a, plan, stats, s);
             else launch_compress_finish<T, THREADS>(a, plan, stats, s);
         }
         e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;
-        // rows whose candidates did not fit (normally none: every CTA returns at once)
-        CompressArgs r = a;
-        r.use_redo_list = 1;
+        // rows whose candidates did not fit (normally none: every CTA returns at once; few rows: an empty bracket)
         ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_REDO, 2, s);
-        if (aligned) launch_compress_direct<T, true>(r, grid, stats, s);
-        else launch_compress_direct<T, false>(r, grid, stats, s);
+        if (!few) {
+            CompressArgs r = a;
+            r.use_redo_list = 1;
+            if (aligned) launch_compress_direct<T, true>(r, grid, stats, s);
+            else launch_compress_direct<T, false>(r, grid, stats, s);
+        }
     } else {
         ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_STREAM, 1, s);
         if (aligned) launch_compress_direct<T, true>(a, grid, stats, s);
@@ -238,6 +256,7 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !stats) return e;
     ProfScope ps2(ctx, PICOSPEC_PROF_COMPRESS_PRECISE, 2, s);
+    if (a.top_p >= 1.0f) return e;      // only a cut can be too close to call (the bracket is empty)
     // rows whose top-p cut was too close to call: exact normaliser, then redo the cut
     PreciseArgs p;
     p.logits = a.logits; p.row_stride = a.row_stride; p.V = a.V; p.nch = a.nch;

@@ -142,3 +142,16 @@ def test_many_keys_of_one_code(dtype, rows, V, k, offset):
     g = torch.Generator(device="cuda").manual_seed(V + k)
     x = 2.0 * torch.randn((rows, 1, V), generator=g, device="cuda") + offset
     _check_compress(x.to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, 1.0, 0.9, g, staged=k > 128)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("k,top_p", [(64, 1.0), (64, 0.9), (300, 0.9)])
+@pytest.mark.parametrize("more", [0, 1])
+def test_rows_to_read_again_among_few_and_many(more, k, top_p, dtype):
+    # as many rows as are finished by a CTA that reads a row again itself (two per SM), and one more: then by
+    # a warp (k = 64) or a CTA that lists such rows for another kernel.  Every ninth row is full of ties.
+    rows, V = 2 * torch.cuda.get_device_properties(0).multi_processor_count + more, 16384
+    g = torch.Generator(device="cuda").manual_seed(rows + k)
+    x = 1.5 * torch.randn((rows, 1, V), generator=g, device="cuda")
+    x[::9, :, :V // 2] = 3.0
+    _check_compress(x.to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, top_p, 0.8, g, staged=False)
