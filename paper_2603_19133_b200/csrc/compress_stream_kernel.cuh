@@ -18,15 +18,15 @@
 //   - the first tile of a row gets its bound without the histogram: every warp finds a value that its
 //     share of the wanted rank of small groups of its elements reach with their maximum; the smallest of
 //     the eight values, or the third smallest with a larger share, is reached by the wanted rank of
-//     elements (one CTA barrier, the only one inside a row);
+//     elements (one CTA barrier, the only one of a row);
 //   - a chunk of which too much passes goes a slower way (crowded_chunk);
 //   - a row whose candidates do not fit (heavy ties), or whose bound rose past its k-th largest, is
 //     handed to the direct kernel through a redo list;
 //   - with top-p the same pass accumulates the softmax normaliser relative to the first tile's
 //     maximum (a row whose later logits overflow that reference also goes to the redo list).
-// At the end of a row the candidates at or above thr (for 16-bit logits the k best plus the ties of the
-// k-th, for 32-bit logits plus what shares its 16-bit code) go to a per-row scratch area in global
-// memory, with the bound itself.
+// At the end of a row every warp writes its candidates at or above thr to a per-row scratch area in global memory
+// (thr was refreshed last after two thirds of the row or more: about 1.4 k of them), which gets the bound as it is
+// when all have.
 //
 // compress_finish_kernel (a warp or a CTA per row) selects the k best of them and puts them in order
 // with a counting sort over the 16-bit logit codes, then calls finish_row (top-p cut,
@@ -42,9 +42,9 @@ namespace picospec {
 // Two shapes of the filter kernel, both sized for three CTAs per SM on 16-bit rows (the kernel is
 // bound by instruction issue, so resident warps count for more than tiles in flight: two stages
 // measure the same as three, three CTAs 15 % faster than two).  Rows with k <= 512 need few live
-// candidates: a small candidate buffer and three stages of 16 KB; larger k takes the big buffer and
-// two stages.  32-bit rows have 32 KB tiles: two stages and two CTAs per SM in both shapes.
-constexpr int CS_CAP_SMALL = 2048, CS_CAP_LARGE = 4096;    // candidate keys held in shared memory
+// candidates: a small candidate buffer; larger k takes the big buffer.  32-bit rows have 32 KB tiles:
+// two CTAs per SM in both shapes.
+constexpr int CS_CAP_SMALL = 2048, CS_CAP_LARGE = 3072;    // candidate keys held in shared memory
 constexpr int CS_K_SMALL = 512;                            // largest k served by the small shape
 constexpr int CS_BINS = 4096;        // histogram bins above the first tile's bound; the last one is open-ended
 constexpr int CS_DEAD = 117 << 7;    // 16-bit magnitude codes below 2^-10: one bin on each side of zero
@@ -62,25 +62,29 @@ struct CsRowMeta {
     int count;        // survivors written for the row
     int flags;
     float ref_off;    // fp32(ref * c32): reference of the streamed normaliser
-    unsigned thr_key; // the row's final bound: every survivor's orderable logit is at least this
-    int top;          // bin coordinate of the largest value counted
+    unsigned thr_key; // the piece's last bound: every entry of it whose orderable logit is at least this is a survivor
+    int top;          // bin coordinate of the largest survivor
     double z_stream;  // sum of 2^(l * c32 - ref_off) over the row (top-p only)
 };
 
-// capacity of a row's scratch area (keys) for a sparse-row capacity k_max
-__host__ __device__ __forceinline__ int cs_survivor_cap(int k_max) { return 2 * k_max > 512 ? 2 * k_max : 512; }
+// capacity of a row's scratch area (keys) for a sparse-row capacity k_max: twice what a row leaves there on average
+// (a bound refreshed last after 69 % of the row, as it is for 23 tiles, lets 1.45 k through)
+__host__ __device__ __forceinline__ int cs_survivor_cap(int k_max) { return 3 * k_max > 512 ? 3 * k_max : 512; }
 
 struct __align__(8) CsShared {
     unsigned thr_key;   // orderable form of the current lower bound on the k-th largest logit
     unsigned certain;   // counts are no longer capped (crowded_chunk): only k of them make a bound
     unsigned first_key[WARPS];  // the warps' own bounds of the first tile
-    unsigned top_key;   // largest orderable logit of the first tile
+    unsigned first_max[WARPS];  // the warps' largest orderable logits of the first tile (STATS)
     int g0;             // bin coordinate of the first tile's bound: origin of the histogram
     int area;           // scratch area of the piece
     int seen;           // chunks whose entries are counted, or are being counted
     int overflow;       // the scratch area ran out of room: the row goes to the redo list
     int nan;
-    int m;              // survivors written at the end of the piece
+    int m;              // survivors written
+    unsigned top;       // 16-bit code of the largest of them
+    int flags;          // CSF_TEMPERATURE / CSF_RANGE, known when the piece begins
+    float ref_off;
     double wsum[WARPS];
 };
 // state of the CTA that outlives a piece
@@ -89,20 +93,18 @@ struct CsCta {
     int k, surv_cap, quota;     // as in FilterBound
     u64* surv_keys;
     int wcnt[WARPS];    // per warp: entries in its region (the slot counter its lanes draw from)
-    int marked[WARPS];  // per warp: its region may hold entries that are not counted yet
     int2 arg[WARPS];    // per warp: what crowded_chunk takes besides its arguments (chunk's offset, its first index)
 };
-// bf16 SMALL: CAP 2048, 3 stages x 16 KB; bf16 LARGE: CAP 4096, 2 stages x 16 KB (72.5 KB either way:
-// 3 CTAs / SM).  fp32: 2 stages x 32 KB (88.5 / 104.5 KB: 2 CTAs / SM).
+// bf16: 2 stages x 16 KB, 66 KB SMALL, 74 KB LARGE (3 CTAs / SM).  fp32: 2 stages x 32 KB, 98 / 106 KB (2 CTAs / SM).
 template <typename T, bool SMALL> struct CsGeom {
     static constexpr int CAP = SMALL ? CS_CAP_SMALL : CS_CAP_LARGE;
     static constexpr int REGION = CAP / WARPS;             // each worker warp appends to its own region
-    static constexpr int STAGES = (sizeof(T) == 2 && SMALL) ? 3 : 2;
+    static constexpr int STAGES = 2;
     static constexpr int CTAS = sizeof(T) == 2 ? 3 : 2;
     static constexpr int TILE_BYTES = TILE_CHUNKS * CHUNK * (int)sizeof(T);
     static constexpr int STAGE_BYTES = STAGES * TILE_BYTES;
     static constexpr int HIST_OFF = STAGE_BYTES + CAP * 8;
-    static constexpr int SHARED_OFF = HIST_OFF + CS_HIST_WORDS * 4;    // CsShared[2], CsCta
+    static constexpr int SHARED_OFF = HIST_OFF + 2 * CS_HIST_WORDS * 4;    // CsShared[2], CsCta
     static constexpr int SMEM_BYTES = SHARED_OFF + 2 * (int)sizeof(CsShared) + (int)sizeof(CsCta);
 };
 
@@ -110,7 +112,7 @@ __device__ __forceinline__ void cs_reset(CsShared& cs) {
     cs.thr_key = 0u;
     cs.certain = 0u;
     cs.seen = 0;
-    cs.top_key = 0u;
+    cs.top = 0u;
     cs.overflow = 0;
     cs.nan = 0;
     cs.m = 0;
@@ -323,11 +325,11 @@ __device__ __forceinline__ int compact_region(u64* region, int n, unsigned thr_k
 template <typename Geom> __device__ __noinline__ void refresh_bound(int copy, int rank, int k) {
     extern __shared__ __align__(1024) unsigned char dyn[];
     CsShared& cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF)[copy];
-    refresh_threshold(reinterpret_cast<const unsigned*>(dyn + Geom::HIST_OFF), cs, rank, k, threadIdx.x & 31);
+    refresh_threshold(reinterpret_cast<const unsigned*>(dyn + Geom::HIST_OFF) + copy * CS_HIST_WORDS, cs, rank, k, threadIdx.x & 31);
 }
 // First tile of a piece: the bound is the NTH smallest of the warps' own (one warp, every warp with the same
-// result; out of line).
-template <typename Geom, int NTH> __device__ __noinline__ void first_bound(int copy, int area) {
+// result; out of line).  Returns the largest orderable logit of the tile (STATS).
+template <typename Geom, int NTH> __device__ __noinline__ unsigned first_bound(int copy, int area) {
     extern __shared__ __align__(1024) unsigned char dyn[];
     CsShared* cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF) + copy;
     const int lane = threadIdx.x & 31;
@@ -345,6 +347,32 @@ template <typename Geom, int NTH> __device__ __noinline__ void first_bound(int c
         *(volatile int*)&cs->area = area;
         atomicMax(&cs->thr_key, bound);
     }
+    __syncwarp();
+    return __reduce_max_sync(0xffffffffu, lane < WARPS ? *(volatile unsigned*)&cs->first_max[lane] : 0u);
+}
+// End of a piece, a warp: its entries at or above the bound go to the piece's scratch area (out of line).
+template <typename Geom> __device__ __noinline__ void hand_over(int copy, int n) {
+    extern __shared__ __align__(1024) unsigned char dyn[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    CsShared* cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF) + copy;
+    const CsCta* cta = reinterpret_cast<const CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
+    const u64* region = reinterpret_cast<const u64*>(dyn + Geom::STAGE_BYTES) + warp * Geom::REGION;
+    const int surv_cap = cta->surv_cap;
+    u64* dst = cta->surv_keys + (long long)*(volatile int*)&cs->area * surv_cap;
+    const unsigned thr_key = __shfl_sync(0xffffffffu, *(volatile unsigned*)&cs->thr_key, 0);
+    unsigned top = 0u;
+    for (int x0 = 0; x0 < n; x0 += 32) {
+        const u64 key = x0 + lane < n ? region[x0 + lane] : 0ull;
+        const unsigned okey = (unsigned)(key >> 32);
+        const unsigned keep = __ballot_sync(0xffffffffu, okey >= thr_key);      // (thr_key > 0: no empty slot)
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&cs->m, __popc(keep));
+        base = __shfl_sync(0xffffffffu, base, 0) + __popc(keep & ((1u << lane) - 1u));
+        if (okey >= thr_key && base < surv_cap) dst[base] = key | CS_COUNTED;
+        top = max(top, okey);
+    }
+    top = __reduce_max_sync(0xffffffffu, top) >> 16;
+    if (lane == 0) atomicMax(&cs->top, top);
     __syncwarp();
 }
 // orderable form of a staged value (-0 becomes +0)
@@ -369,7 +397,7 @@ __device__ __noinline__ int crowded_chunk(unsigned mask, int n, int copy) {
     CsCta* cta = reinterpret_cast<CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
     const unsigned char* chunk = dyn + cta->arg[warp].x;
     const int vchunk = cta->arg[warp].y;
-    unsigned* hist = reinterpret_cast<unsigned*>(dyn + Geom::HIST_OFF);
+    unsigned* hist = reinterpret_cast<unsigned*>(dyn + Geom::HIST_OFF) + copy * CS_HIST_WORDS;
     u64* region = reinterpret_cast<u64*>(dyn + Geom::STAGE_BYTES) + warp * REGION;
     u64* to = region;
     int* wcnt = &cta->wcnt[warp];
@@ -380,7 +408,6 @@ __device__ __noinline__ int crowded_chunk(unsigned mask, int n, int copy) {
     if (n + added <= REGION) {
         const bool certain = __any_sync(0xffffffffu, *(volatile unsigned*)&cs->certain);
         count = certain ? added : cta->quota;
-        if (lane == 0) cta->marked[warp] = 1;
     } else if (!SPREAD) {
         refresh_threshold(hist, *cs, k, k, lane);
         __syncwarp();
@@ -541,7 +568,7 @@ inline FilterPlan make_filter_plan(int rows, int tiles_per_row, bool ragged_last
 // They are not: vocabularies have an order (frequent pieces first, languages and unused ids in blocks).
 // A tile takes one chunk from each eighth of the row, so that each eighth is seen to the same fraction, and
 //   - no chunk counts with more than a quarter of the first tile's rank and eight (chunk_quota; the entries
-//     beyond it are marked and counted at the row's end): a crowded place cannot lift the bound above
+//     beyond it are marked and counted only if a region runs full): a crowded place cannot lift the bound above
 //     what three quarters of the rank reach elsewhere, which is still 1.125 k f and more;
 //   - the first tile's bound is the third smallest of the warps' own, a sixth of the rank each: it is neither
 //     lifted by five crowded chunks nor dropped by two empty ones (an unused end of the vocabulary);
@@ -626,10 +653,13 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
     constexpr int CS_CAND_CAP = Geom::CAP, CS_REGION = Geom::REGION;
     unsigned char* stage_mem = dyn;
     u64* cand = reinterpret_cast<u64*>(dyn + Geom::STAGE_BYTES);
-    unsigned* hist = reinterpret_cast<unsigned*>(cand + CS_CAND_CAP);          // bins, then super-bins
+    unsigned* hists = reinterpret_cast<unsigned*>(cand + CS_CAND_CAP);         // bins, then super-bins; two copies
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES];
-    // Two copies of the per-piece state, used in turn: the copy of the piece that has just ended is
-    // reset by one thread while the other warps already start on the next piece.
+    // Two copies of the per-piece state and of the histogram, used in turn, so that a piece has one barrier, that
+    // of its first tile: behind it every warp is done with the piece before, whose record is written and whose copies
+    // are cleared there.  (With three barriers a piece, a last exact bound and one histogram the kernel took 70.8 us for
+    // 4096 rows of 32000 entries at k = 8, 29.5 for 256 of 128256 at k = 10, 11.4 for 40 of 128256 at k = 64; now 67.8,
+    // 27.6 and 10.6, and the finish behind it 6.6 instead of 10.3 at k = 8.  Long rows: no difference.)
     CsShared* css = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF);
     CsCta& cta = *reinterpret_cast<CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
 
@@ -648,8 +678,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
         cta.quota = fb.quota;
         cta.surv_keys = a.surv_keys;
     }
-    if (tid < WARPS) cta.wcnt[tid] = cta.marked[tid] = 0;
-    for (int i = tid; i < CS_HIST_WORDS; i += STREAM_THREADS) hist[i] = 0u;
+    if (tid < WARPS) cta.wcnt[tid] = 0;
+    for (int i = tid; i < 2 * CS_HIST_WORDS; i += STREAM_THREADS) hists[i] = 0u;
     grid_dependency_sync();
     if (tid == 0 && blockIdx.x == 0) {
         *a.queue_count_next = 0;
@@ -697,10 +727,32 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
     bool lost = false;      // a wait did not complete at all: the warp stops waiting as well
     uint32_t i = 0;
     int parity = 0;         // which copy of the per-piece state this piece uses
+    // the record of a piece that every warp has done its share of (one thread)
+    auto write_record = [&](const CsShared& done) {
+        const int m = done.m;
+        int flags = done.flags;
+        if (cta.abort) flags = CSF_ABORT;
+        else if (flags == 0 && (done.overflow || m > fb.surv_cap)) flags = CSF_REDO;      // too many candidates, or ties at the bound
+        else if (flags == 0 && done.nan) flags = CSF_LOGIT;
+        double zs = 0.0;
+        if (STATS)
+            for (int w = 0; w < WARPS; ++w) zs += done.wsum[w];
+        // a reference that later logits overflowed, or NaN / +inf data: the direct kernel sorts it out
+        if (STATS && flags == 0 && !(zs > 0.0 && zs < CUDART_INF)) flags = CSF_REDO;
+        CsRowMeta meta;
+        meta.count = m;
+        meta.flags = flags;
+        meta.ref_off = done.ref_off;
+        meta.thr_key = done.thr_key;
+        meta.top = bin_coord(done.top);
+        meta.z_stream = zs;
+        a.surv_meta[done.area] = meta;
+    };
     FilterPiece pc;
     for (int k = 0; plan_piece(plan, blockIdx.x, k, pc); ++k) {
         if (pc.tile0 >= pc.tile1) continue;
         CsShared& cs = css[parity];
+        unsigned* hist = hists + parity * CS_HIST_WORDS;
         parity ^= 1;
         const int row = pc.row;
         const float Tb = a.temperature[row / a.G];
@@ -737,12 +789,11 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
             const unsigned char* chunk = stage_mem + s * TILE_BYTES + warp * (CHUNK * (int)sizeof(T));
             ChunkRegs<T> regs;
             if (work) load_staged(regs, chunk, c * CHUNK, end, lane);
-            if (ti == pc.tile0 && valid) {
+            if (ti == pc.tile0) {
                 // first tile of a piece: each warp's own bound (none without a chunk), then the smallest of them, or the
                 // third smallest
-                if (lane == 0) cs.first_key[warp] = 0u;
+                unsigned k16 = 0u, most = 0u;
                 if (work) {
-                    unsigned k16;
                     float wm = 0.f;
                     if (fb.need <= 16) {
                         const float lm = regs.lane_max_plain();
@@ -752,15 +803,24 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
                         k16 = first_tile_key(regs, fb.group, fb.need);
                         if (STATS) wm = warp_max_redux(regs.lane_max_plain());
                     }
-                    if (lane == 0) {
-                        cs.first_key[warp] = k16 << 16;
-                        if (STATS && wm == wm) atomicMax(&cs.top_key, orderable(wm));
-                    }
+                    if (STATS && wm == wm) most = orderable(wm);
+                }
+                if (lane == 0) {
+                    cs.first_key[warp] = k16 << 16;
+                    if (STATS) cs.first_max[warp] = most;
                 }
                 workers_sync();
-                first_bound<Geom, SPREAD ? 3 : 1>(parity ^ 1, pc.area);
-                if (STATS) ref_off = __fmul_rn(from_orderable(*(volatile unsigned*)&cs.top_key), c32);
-                if (__any_sync(0xffffffffu, *(volatile unsigned*)&cs.thr_key < 0x00800000u)) {
+                // the copies of the piece before
+                if (tid == 0) {
+                    if (i) write_record(css[parity]);
+                    cs_reset(css[parity]);
+                    cs.flags = !in_range ? CSF_RANGE : !valid ? CSF_TEMPERATURE : 0;
+                }
+                if (i)
+                    for (int x = tid; x < CS_HIST_WORDS; x += THREADS) hists[parity * CS_HIST_WORDS + x] = 0u;
+                const unsigned first_top = first_bound<Geom, SPREAD ? 3 : 1>(parity ^ 1, pc.area);
+                if (STATS) ref_off = __fmul_rn(from_orderable(first_top), c32);
+                if (valid && __any_sync(0xffffffffu, *(volatile unsigned*)&cs.thr_key < 0x00800000u)) {
                     // no finite bound (rows of -inf): everything would pass, padding included
                     if (lane == 0) cs.overflow = 1;
                     row_chunks = 0;
@@ -823,63 +883,18 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
         }
 
         // ---- end of the piece: survivors and statistics to the piece's scratch area ------------------
-        const bool whole = pc.tile1 - pc.tile0 == plan.tiles_per_row;
         __syncwarp();
-        if (SPREAD && whole && *(volatile int*)&cta.marked[warp]) {
-            count_marked(hist, region, wcount, *(volatile int*)&cs.g0, lane);
-        }
         if (STATS) {
             const double sw = (double)warp_sum(acc);
             if (lane == 0) cs.wsum[warp] = sw;
+            if (tid == 0) cs.ref_off = ref_off;
         }
-        workers_sync();     // every candidate is counted, every flag is set
-        const bool piece_ok = valid && !*(volatile int*)&cs.overflow && !*(volatile int*)&cta.abort;
-        unsigned thr_final = *(volatile unsigned*)&cs.thr_key;
-        int top = 0;
-        if (piece_ok) {
-            // the final bound, by every warp for itself (all get the same): no second barrier for it
-            const bool certain = !SPREAD || whole || *(volatile unsigned*)&cs.certain;
-            const int found = kth_bin(hist, certain ? fb.k : bound_rank(fb.k, fb.per_tile * (float)(pc.tile1 - pc.tile0)), lane);
-            if (warp == 0) top = *(volatile int*)&cs.g0 + max(kth_bin(hist, 1, lane), 0);
-            if (found >= 0) thr_final = max(thr_final, coord_code(*(volatile int*)&cs.g0 + found) << 16);
-            // every warp filters its own region and appends to the piece's scratch area
-            u64* dst = a.surv_keys + (long long)pc.area * fb.surv_cap;
-            const int n = compact_region(region, wcount, thr_final, lane);
-            int base = 0;
-            if (lane == 0 && n) base = atomicAdd(&cs.m, n);
-            base = __shfl_sync(0xffffffffu, base, 0);
-            for (int x = lane; x < n; x += 32)
-                if (base + x < fb.surv_cap) dst[base + x] = region[x] | CS_COUNTED;
-        }
-        workers_sync();     // the survivors are counted; nobody reads the histogram any more
-        if (tid == 0) {
-            int flags = 0;
-            const int m = cs.m;
-            if (cta.abort) flags = CSF_ABORT;
-            else if (!in_range) flags = CSF_RANGE;
-            else if (!valid) flags = CSF_TEMPERATURE;
-            else if (cs.overflow || m > fb.surv_cap) flags = CSF_REDO;      // too many candidates, or ties at the bound
-            else if (cs.nan) flags = CSF_LOGIT;
-            double zs = 0.0;
-            if (STATS)
-                for (int w = 0; w < WARPS; ++w) zs += cs.wsum[w];
-            // a reference that later logits overflowed, or NaN / +inf data: the direct kernel sorts it out
-            if (STATS && flags == 0 && !(zs > 0.0 && zs < CUDART_INF)) flags = CSF_REDO;
-            CsRowMeta meta;
-            meta.count = m;
-            meta.flags = flags;
-            meta.ref_off = ref_off;
-            meta.thr_key = thr_final;
-            meta.top = top;
-            meta.z_stream = zs;
-            a.surv_meta[pc.area] = meta;
-            cs_reset(cs);       // this copy is used again by the piece after the next one
-        }
-        // Ready for the next piece, without a barrier of its own: the histogram is not written before
-        // the barrier of that piece's first tile, which every warp reaches after its share of this.
-        if (lane == 0) cta.wcnt[warp] = cta.marked[warp] = 0;
-        for (int x = tid; x < CS_HIST_WORDS; x += THREADS) hist[x] = 0u;
+        if (valid && !__any_sync(0xffffffffu, *(volatile int*)&cs.overflow | *(volatile int*)&cta.abort)) hand_over<Geom>(parity ^ 1, wcount);
+        if (lane == 0) cta.wcnt[warp] = 0;
+        __syncwarp();
     }
+    workers_sync();
+    if (tid == 0 && i) write_record(css[parity ^ 1]);
 }
 
 // ---- finish: select, order, cut, emit ---------------------------------------------------------
