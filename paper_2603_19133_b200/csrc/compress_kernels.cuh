@@ -580,17 +580,17 @@ __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs 
     const long long total = (long long)nq * a.nch;
     const long long pairs = (total + 1) / 2;
     for (long long pi = blockIdx.x; pi < pairs; pi += gridDim.x) {
-        const long long item = 2 * pi + sub;
-        int qslot = -1;
-        const double s = precise_item_sum<T>(p, item, total, quarter, lane, qslot);
+        PreciseQuarter<T> q;
+        q.load(p, 2 * pi + sub, total, quarter, lane);
+        const double s = q.slot >= 0 ? q.sum() : 0.0;
         if (lane == 0) part[warp] = s;
         __syncthreads();
         if (quarter == 0 && lane == 0) {
             int mine = -1;
-            if (item < total) {
-                precise_item_store(p, item, (part[warp] + part[warp + 1]) + (part[warp + 2] + part[warp + 3]));
+            if (q.slot >= 0) {
+                precise_store(p, q, (part[warp] + part[warp + 1]) + (part[warp + 2] + part[warp + 3]));
                 __threadfence();
-                if (atomicAdd(&a.tickets[qslot], 1) == a.nch - 1) mine = qslot;
+                if (atomicAdd(&a.tickets[q.slot], 1) == a.nch - 1) mine = q.slot;
             }
             last_slot[sub] = mine;
         }

@@ -20,71 +20,73 @@ struct PreciseArgs {
     int pitch = 0;             // chunk sums per row in dsum (0: nch)
 };
 
-// One quarter of one item of the double-precision pass, by one warp.  Item = (listed row, chunk);
-// returns the partial sum and the position of the row in the list.
-template <typename T>
-__device__ __forceinline__ double precise_item_sum(const PreciseArgs& a, long long item, long long total, int quarter,
-                                                   int lane, int& qslot) {
-    qslot = -1;
-    double s = 0.0;
-    if (item < total) {
-        const int c = (int)(item % a.nch);
-        qslot = (int)(item / a.nch);
-        const int src_row = a.rows[qslot] & 0x1FFFFFFF;     // (a list may keep flags above the index)
-        const int b = src_row / a.seq_rows;
-        const T* row = reinterpret_cast<const T*>(a.logits) + (long long)src_row * a.row_stride;
-        // x = l * (1/T) instead of l / T: one rounding of 2^-53 more per term, far below every
-        // threshold this pass decides; four independent sums keep the exp pipeline busy
-        const double rT = 1.0 / (double)a.temperature[b];
-        const double m = (double)a.row_max[src_row] * rT;
-        const int v0 = c * CHUNK + quarter * (CHUNK / 4);
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+// A quarter of one item of the double-precision pass, held by a warp.  Item = (listed row, chunk).
+constexpr int PRECISE_HELD = CHUNK / 4 / 32;
+template <typename T> struct PreciseQuarter {
+    int slot, row, c;           // the row's place in the list (-1: no such item), the row, the chunk
+    float Tb, mx;
+    float l[PRECISE_HELD];
+    __device__ __forceinline__ void load(const PreciseArgs& a, long long item, long long total, int quarter, int lane) {
+        slot = -1;
+        if (item >= total) return;
+        slot = (int)(item / a.nch);
+        c = (int)(item - (long long)slot * a.nch);
+        row = a.rows[slot] & 0x1FFFFFFF;    // (a list may keep flags above the index)
+        Tb = a.temperature[row / a.seq_rows];
+        mx = a.row_max[row];
+        const T* p = reinterpret_cast<const T*>(a.logits) + (long long)row * a.row_stride;
+        const int v0 = c * CHUNK + quarter * (CHUNK / 4) + lane;
 #pragma unroll
-        for (int k = lane; k < CHUNK / 4; k += 128) {
-            const int v = v0 + k;
-            float l0 = -CUDART_INF_F, l1 = -CUDART_INF_F, l2 = -CUDART_INF_F, l3 = -CUDART_INF_F;
-            if (v < a.V) l0 = load_logit(row, v);
-            if (v + 32 < a.V) l1 = load_logit(row, v + 32);
-            if (v + 64 < a.V) l2 = load_logit(row, v + 64);
-            if (v + 96 < a.V) l3 = load_logit(row, v + 96);
-            s0 += exp((double)l0 * rT - m);
-            s1 += exp((double)l1 * rT - m);
-            s2 += exp((double)l2 * rT - m);
-            s3 += exp((double)l3 * rT - m);
-        }
-        s = warp_sum((s0 + s1) + (s2 + s3));
+        for (int x = 0; x < PRECISE_HELD; ++x) l[x] = v0 + x * 32 < a.V ? load_logit(p, v0 + x * 32) : -CUDART_INF_F;
     }
-    return s;
-}
+    // The sum of exp(l/T - mx/T).  x = l * (1/T) instead of l / T: one rounding of 2^-53 more per term, far below
+    // every threshold this pass decides; four independent sums keep the exp pipeline busy.
+    __device__ __forceinline__ double sum() {
+        const double rT = 1.0 / (double)Tb, m = (double)mx * rT;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+#pragma unroll 1
+        for (int x = 0; x < PRECISE_HELD; x += 4) {
+            s0 += exp((double)l[0] * rT - m);
+            s1 += exp((double)l[1] * rT - m);
+            s2 += exp((double)l[2] * rT - m);
+            s3 += exp((double)l[3] * rT - m);
+#pragma unroll
+            for (int y = 0; y + 4 < PRECISE_HELD; ++y) l[y] = l[y + 4];
+        }
+        return warp_sum((s0 + s1) + (s2 + s3));
+    }
+};
 // where the sum of an item goes
-__device__ __forceinline__ void precise_item_store(const PreciseArgs& a, long long item, double sum) {
-    const int c = (int)(item % a.nch);
-    const int src_row = a.rows[(int)(item / a.nch)] & 0x1FFFFFFF;
-    a.dsum[(long long)src_row * (a.pitch > 0 ? a.pitch : a.nch) + c] = sum;
+template <typename T> __device__ __forceinline__ void precise_store(const PreciseArgs& a, const PreciseQuarter<T>& q, double sum) {
+    a.dsum[(long long)q.row * (a.pitch > 0 ? a.pitch : a.nch) + q.c] = sum;
 }
 
+// A CTA takes two chunks at a time, four warps per chunk (a quarter of the chunk each, so that a handful of rows
+// still spreads over the whole GPU); the four partial sums of a chunk are added in a fixed order.  Where a CTA
+// takes several, the next one's logits are on the way while the exponentials of the one at hand are taken, so that
+// three CTAs per SM do what took six (40 rows of 128256 entries: 17 us either way, bound by the chain of one
+// item).  Few rows are bound by the launch: see precise_grid.
+constexpr int PRECISE_CTAS = 3;     // per SM
 template <typename T>
-__global__ void __launch_bounds__(THREADS) precise_chunk_sums_kernel(PreciseArgs a) {
+__global__ void __launch_bounds__(THREADS, PRECISE_CTAS) precise_chunk_sums_kernel(PreciseArgs a) {
     grid_dependency_sync();
     const int nq = *a.row_count;
     if (nq == 0) return;
-    // A CTA takes two chunks at a time, four warps per chunk (a quarter of the chunk each, so that a
-    // handful of rows still spreads over the whole GPU); the four partial sums of a chunk are added in
-    // a fixed order.
-    __shared__ double part[WARPS];
+    __shared__ double part[2][WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = warp >> 2, quarter = warp & 3;
     const long long total = (long long)nq * a.nch;
-    const long long pairs = (total + 1) / 2;
-    for (long long pi = blockIdx.x; pi < pairs; pi += gridDim.x) {
-        const long long item = 2 * pi + sub;
-        int qslot;
-        const double s = precise_item_sum<T>(a, item, total, quarter, lane, qslot);
-        if (lane == 0) part[warp] = s;
-        __syncthreads();
-        if (item < total && quarter == 0 && lane == 0)
-            precise_item_store(a, item, (part[warp] + part[warp + 1]) + (part[warp + 2] + part[warp + 3]));
-        __syncthreads();
+    PreciseQuarter<T> next;
+    next.load(a, 2ll * blockIdx.x + sub, total, quarter, lane);
+    int copy = 0;
+    for (long long pair = blockIdx.x; 2 * pair < total; pair += gridDim.x, copy ^= 1) {
+        PreciseQuarter<T> q = next;
+        next.load(a, 2 * (pair + gridDim.x) + sub, total, quarter, lane);
+        const double s = q.slot >= 0 ? q.sum() : 0.0;
+        if (lane == 0) part[copy][warp] = s;
+        __syncthreads();        // (one barrier an item: the copies take turns)
+        if (q.slot >= 0 && quarter == 0 && lane == 0)
+            precise_store(a, q, (part[copy][warp] + part[copy][warp + 1]) + (part[copy][warp + 2] + part[copy][warp + 3]));
     }
 }
 
