@@ -316,7 +316,10 @@ cudaError_t launch_verify(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s
     {
         ProfScope ps(ctx, PICOSPEC_PROF_VERIFY_FINISH, 2, s);
         if (edge) launch_chained(edge_finish_kernel<T, false>, a.B, THREADS, 0, s, a);
-        else launch_chained(verify_finish_kernel<T, false>, a.B, THREADS, dyn, s, f);
+        // more sequences than are resident at two CTAs per SM, few entries each: four (64 registers; 512 sequences of
+        // 8 positions, k = 8: 17.0 -> 12.3 us; one wave of sequences is bound by its chain and keeps 126 registers)
+        else launch_chained(a.B > 2 * ctx->num_sms && a.k_max <= 64 ? verify_finish_kernel<T, false, false, 2> : verify_finish_kernel<T, false>,
+                            a.B, THREADS, dyn, s, f);
     }
     ProfScope ps3(ctx, PICOSPEC_PROF_VERIFY_PRECISE, 2, s);
     PreciseArgs p;

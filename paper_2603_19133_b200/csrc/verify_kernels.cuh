@@ -487,7 +487,8 @@ __device__ __noinline__ void chunk_masses(const VerifyArgs& a, FinishShared& sh,
 // K = 128), 26 -> 13 (256 x 6, K = 256).  At K = 1024 (512 x 8: 197 -> 175 us) it is bound by the DRAM
 // sectors of the gathers instead.  Without the reads before the wait 256 x 6 takes 24.6 us, with the
 // streaming pass 5 us shorter for it.
-template <typename T, bool PRECISE, bool SHARDED>
+// HELD: entries per lane that stay in registers (rows of at most 64 entries need two).
+template <typename T, bool PRECISE, bool SHARDED, int HELD>
 __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot, FinishShared& sh, double* cm) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = a.G, G1 = a.G + 1;
@@ -552,8 +553,8 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                 const float* ent = SHARDED ? a.entry_logits + (long long)ri * (a.k_max + 1) : nullptr;
                 // the first batch of stored entries is requested before the row's count is known
                 // (every slot below k_max exists; slots at or beyond the count are dropped below)
-                int vv[8], x = -1, n = 0;
-                float qq[8], ll[8], ux = 0.f, lx = -CUDART_INF_F;
+                int vv[HELD], x = -1, n = 0;
+                float qq[HELD], ll[HELD], ux = 0.f, lx = -CUDART_INF_F;
                 bool range_bad = false;
                 if (entries) {
                     n = a.q_count[ri];
@@ -562,7 +563,7 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                         ux = a.u_accept[ri];
                     }
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
+                    for (int u = 0; u < HELD; ++u) {
                         const int k = u * 32 + lane;
                         vv[u] = k < a.k_max ? idx[k] : -2;
                         qq[u] = k < a.k_max ? prob[k] : 0.f;
@@ -571,7 +572,7 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                     // p(x) on every lane (the same instructions as on one lane, and no divergent tail)
                     if (tested && !range_bad) lx = SHARDED ? ent[a.k_max] : load_logit(row, x);
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
+                    for (int u = 0; u < HELD; ++u) {
                         const int k = u * 32 + lane;
                         if (k >= n || range_bad) vv[u] = -2;
                         const bool ok = vv[u] >= 0 && vv[u] < a.V;
@@ -613,7 +614,7 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                         }
                     }
                 };
-                if (n_read <= 64) {
+                if (HELD == 2 || n_read <= 64) {
                     // few entries: one copy of the body (see exp_call)
 #pragma unroll 1
                     for (int k0 = 0; k0 < n_read; k0 += 32) {
@@ -623,7 +624,7 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
                         ll[0] = ll[1];
                         __syncwarp();
                     }
-                } else {
+                } else if constexpr (HELD == 8) {
                     // many: four exponentials in flight
 #pragma unroll 1
                     for (int k0 = 0; k0 < n_read; k0 += 128) {
@@ -901,8 +902,8 @@ __device__ __forceinline__ void verify_finish_slot(const VerifyArgs& a, int slot
     }
 }
 
-template <typename T, bool PRECISE, bool SHARDED = false>
-__global__ void __launch_bounds__(THREADS, 2) verify_finish_kernel(const __grid_constant__ VerifyArgs a) {
+template <typename T, bool PRECISE, bool SHARDED = false, int HELD = 8>
+__global__ void __launch_bounds__(THREADS, HELD == 2 ? 4 : 2) verify_finish_kernel(const __grid_constant__ VerifyArgs a) {
     extern __shared__ double cm[];  // chunk masses: of every row that is read (a.cm_rows), or of the sampled one
     __shared__ FinishShared sh;
     // Only the chunk statistics / exact sums come from the kernel before this one; whatever was written
@@ -910,7 +911,7 @@ __global__ void __launch_bounds__(THREADS, 2) verify_finish_kernel(const __grid_
     // its own wait.  (The sharded form follows an exchange and waits at once.)
     if (SHARDED) grid_dependency_wait();
     const int nloop = PRECISE ? *a.queue_count : a.B;
-    for (int slot = blockIdx.x; slot < nloop; slot += gridDim.x) verify_finish_slot<T, PRECISE, SHARDED>(a, slot, sh, cm);
+    for (int slot = blockIdx.x; slot < nloop; slot += gridDim.x) verify_finish_slot<T, PRECISE, SHARDED, HELD>(a, slot, sh, cm);
     grid_dependency_sync();
 }
 

@@ -760,3 +760,13 @@ def test_both_sides_of_the_room_for_chunk_masses_of_the_draw_alone(ps, K):
     assert ctx.status(clear=True)[0] == 0
     assert np.array_equal(_np(tok), o_tok)
     np.testing.assert_allclose(_np(mass), o_mass, rtol=RTOL, atol=ATOL_MASS)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("more,k", [(0, 64), (1, 64), (1, 33), (1, 65)])
+def test_finish_of_more_sequences_than_are_resident(ps, more, k, dtype):
+    # two sequences per SM, and one more: four CTAs per SM while a row has at most 64 entries
+    B = 2 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    w = gen.Workload("m", V=9000, B=B, G=3, dtype=dtype, s=1.1, sigma_d=1.5, corr=0.8, sigma_t=1.0, T=None, top_k=k,
+                     top_p=1.0, k_max=k)
+    assert run_both(ps, w, gen.make_inputs(w, seed=B + k, device="cuda"), check_compress=False)["status"] == 0
