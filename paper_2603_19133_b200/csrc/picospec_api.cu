@@ -257,6 +257,12 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
             else launch_compress_direct<T, false>(r, grid, stats, s);
         }
     } else {
+        // a captured call may be replayed alone, with no call between that clears its queue
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusActive) {
+            const cudaError_t em = cudaMemsetAsync(a.queue_count, 0, sizeof(int), s);
+            if (em != cudaSuccess) return em;
+        }
         ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_STREAM, 1, s);
         if (aligned) launch_compress_direct<T, true>(a, grid, stats, s);
         else launch_compress_direct<T, false>(a, grid, stats, s);

@@ -155,3 +155,32 @@ def test_rows_to_read_again_among_few_and_many(more, k, top_p, dtype):
     x = 1.5 * torch.randn((rows, 1, V), generator=g, device="cuda")
     x[::9, :, :V // 2] = 3.0
     _check_compress(x.to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, top_p, 0.8, g, staged=False)
+
+
+@pytest.mark.parametrize("rows,V", [(400, 16384), (24, 16384), (24, 4096)])
+def test_a_captured_call_is_replayed_alone(rows, V):
+    # rows of equal logits whose cut falls on an entry's edge: each is read again by the direct kernel and takes
+    # the double-precision cut.  A replay has no other call before it that would clear the lists.
+    import paper_2603_19133_b200 as ps
+    k, keep = 64, 40
+    x = torch.zeros((rows, 1, V), dtype=torch.bfloat16, device="cuda")
+    T = torch.ones((rows,), device="cuda")
+    u = torch.rand((rows, 1), device="cuda")
+    i32 = torch.int32
+    out = (torch.empty((rows, 1, k), dtype=i32, device="cuda"), torch.empty((rows, 1, k), device="cuda"),
+           torch.empty((rows, 1), dtype=i32, device="cuda"), torch.empty((rows, 1), dtype=i32, device="cuda"))
+    ctx = ps.Context(rows, 1, V, k)
+    try:
+        ctx.compress(x, T, 0, keep / V, k, u, out=out)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            ctx.compress(x, T, 0, keep / V, k, u, out=out)
+        ctx.counters(clear=True)
+        for n in range(1, 4):
+            graph.replay()
+            assert ctx.counters()[0] == n * rows
+            assert (out[2] == keep).all() and (out[0][:, 0, :keep] == torch.arange(keep, dtype=i32, device="cuda")).all()
+        assert ctx.status()[0] == 0
+        del graph
+    finally:
+        ctx.close()
