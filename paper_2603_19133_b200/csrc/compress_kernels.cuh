@@ -566,6 +566,8 @@ __global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
 // Nothing waits (fence, then ticket); with an empty queue every CTA returns at once.
 template <typename T>
 __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs a, PreciseArgs p) {
+    __shared__ double table[EXP_STEPS];
+    exp_table(table);
     grid_dependency_sync();
     extern __shared__ u64 smem64[];
     u64* keep = smem64;
@@ -574,6 +576,7 @@ __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs 
     __shared__ int last_slot[2];
     const int nq = *a.queue_count;
     if (nq == 0) return;
+    __syncthreads();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = warp >> 2, quarter = warp & 3;
     const int k_eff = kept_entries(a);
@@ -582,7 +585,7 @@ __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs 
     for (long long pi = blockIdx.x; pi < pairs; pi += gridDim.x) {
         PreciseQuarter<T> q;
         q.load(p, 2 * pi + sub, total, quarter, lane);
-        const double s = q.slot >= 0 ? q.sum() : 0.0;
+        const double s = q.slot >= 0 ? q.sum(table) : 0.0;
         if (lane == 0) part[warp] = s;
         __syncthreads();
         if (quarter == 0 && lane == 0) {

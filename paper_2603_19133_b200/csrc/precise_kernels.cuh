@@ -20,6 +20,29 @@ struct PreciseArgs {
     int pitch = 0;             // chunk sums per row in dsum (0: nch)
 };
 
+// exp(x) for x <= 0 (-inf included) in double precision, to about one unit in the last place: x = (64 m + j) ln 2 / 64 + r
+// with |r| <= ln 2 / 128, exp(x) = 2^m 2^(j/64) (1 + p(r)), p the Taylor polynomial of exp(r) - 1 of degree 5 (its
+// remainder is below 2^-54).  The powers 2^(j/64) lie in shared memory.  ln 2 / 64 is taken off in two parts, the
+// first of 34 bits, so that its product with 64 m + j is exact.  Below -700 the result is 0.
+// 12 double-precision operations a term: 256 rows of the edge, 40 of them exact, 80.4 -> 76.4 us a pass against exp().
+constexpr int EXP_STEPS = 64;
+__device__ __forceinline__ void exp_table(double* table) {      // by the CTA's first threads (a barrier follows)
+    if (threadIdx.x < EXP_STEPS) table[threadIdx.x] = exp2((double)(int)threadIdx.x / EXP_STEPS);
+}
+__device__ __forceinline__ double exp_by_table(double x, const double* table) {
+    const double round = 6755399441055744.0;                    // 1.5 * 2^52: its last bits take the rounded product
+    const double t = fma(x, 0x1.71547652b82fep+6, round);       // 64 / ln 2
+    const int n = __double2loint(t);
+    const double nd = t - round;
+    const double r = fma(nd, -0x1.1cf79abc9e3b4p-42, fma(nd, -0x1.62e42fef80000p-7, x));
+    const double q = fma(r, fma(r, fma(r, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5);
+    const double p = fma(r * r, q, r);
+    const double w = table[n & (EXP_STEPS - 1)];
+    const double y = fma(w, p, w);
+    const double scaled = __hiloint2double(__double2hiint(y) + ((n >> 6) << 20), __double2loint(y));
+    return (unsigned)__double2hiint(x) > 0xC085E000u ? 0.0 : scaled;        // x < -700
+}
+
 // A quarter of one item of the double-precision pass, held by a warp.  Item = (listed row, chunk).
 constexpr int PRECISE_HELD = CHUNK / 4 / 32;
 template <typename T> struct PreciseQuarter {
@@ -41,15 +64,15 @@ template <typename T> struct PreciseQuarter {
     }
     // The sum of exp(l/T - mx/T).  x = l * (1/T) instead of l / T: one rounding of 2^-53 more per term, far below
     // every threshold this pass decides; four independent sums keep the exp pipeline busy.
-    __device__ __forceinline__ double sum() {
+    __device__ __forceinline__ double sum(const double* table) {
         const double rT = 1.0 / (double)Tb, m = (double)mx * rT;
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
 #pragma unroll 1
         for (int x = 0; x < PRECISE_HELD; x += 4) {
-            s0 += exp((double)l[0] * rT - m);
-            s1 += exp((double)l[1] * rT - m);
-            s2 += exp((double)l[2] * rT - m);
-            s3 += exp((double)l[3] * rT - m);
+            s0 += exp_by_table((double)l[0] * rT - m, table);
+            s1 += exp_by_table((double)l[1] * rT - m, table);
+            s2 += exp_by_table((double)l[2] * rT - m, table);
+            s3 += exp_by_table((double)l[3] * rT - m, table);
 #pragma unroll
             for (int y = 0; y + 4 < PRECISE_HELD; ++y) l[y] = l[y + 4];
         }
@@ -69,10 +92,12 @@ template <typename T> __device__ __forceinline__ void precise_store(const Precis
 constexpr int PRECISE_CTAS = 3;     // per SM
 template <typename T>
 __global__ void __launch_bounds__(THREADS, PRECISE_CTAS) precise_chunk_sums_kernel(PreciseArgs a) {
+    __shared__ double part[2][WARPS], table[EXP_STEPS];
+    exp_table(table);
     grid_dependency_sync();
     const int nq = *a.row_count;
     if (nq == 0) return;
-    __shared__ double part[2][WARPS];
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = warp >> 2, quarter = warp & 3;
     const long long total = (long long)nq * a.nch;
@@ -82,7 +107,7 @@ __global__ void __launch_bounds__(THREADS, PRECISE_CTAS) precise_chunk_sums_kern
     for (long long pair = blockIdx.x; 2 * pair < total; pair += gridDim.x, copy ^= 1) {
         PreciseQuarter<T> q = next;
         next.load(a, 2 * (pair + gridDim.x) + sub, total, quarter, lane);
-        const double s = q.slot >= 0 ? q.sum() : 0.0;
+        const double s = q.slot >= 0 ? q.sum(table) : 0.0;
         if (lane == 0) part[copy][warp] = s;
         __syncthreads();        // (one barrier an item: the copies take turns)
         if (q.slot >= 0 && quarter == 0 && lane == 0)
