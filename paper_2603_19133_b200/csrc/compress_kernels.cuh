@@ -30,15 +30,14 @@ struct CompressArgs {
     float* row_max;            // [B*G]
     double* dsum;              // [B*G, nch]
     int* queue;
-    int* queue_count;          // zero on entry (cleared by the previous call)
-    int* queue_count_next;     // cleared by this call for the next one
+    int* queue_count;          // zero between calls: compress_precise_kernel, which reads it last, clears it
+    unsigned* queue_readers;   // CTAs of that kernel that are done with the queue (zero between calls)
     int* tickets;              // per queue slot: chunk sums completed in the double-precision pass
     unsigned* status;
     unsigned long long* slow_rows;
     // rows the staged kernel hands to the direct kernel (candidate buffer overflow)
     int* redo_rows;            // [B*G]
-    int* redo_count;           // zero on entry of the staged kernel
-    int* redo_count_next;      // cleared for the next call
+    int* redo_count;           // cleared by the filter kernel of the same call
     int use_redo_list;         // direct kernel: 1 = process redo_rows[0 .. *redo_count) only
     unsigned long long* redo_total;   // cumulative number of rows handed over (reported by picospec_counters)
     // Top-K of selected rows (picospec_target_topk): output row r reads logits row
@@ -548,12 +547,6 @@ __global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
     grid_dependency_sync();
     extern __shared__ u64 smem64[];
     __shared__ CompressShared sh;
-    // a call that goes through this kernel alone clears both of the next call's counters, as the
-    // staged filter kernel does (the redo-list launch of a staged call must not: the filter did)
-    if (blockIdx.x == 0 && threadIdx.x == 0 && !a.use_redo_list) {
-        *a.queue_count_next = 0;
-        *a.redo_count_next = 0;
-    }
     const int nwork = a.use_redo_list ? *a.redo_count : a.B * a.G, k_eff = kept_entries(a);
     for (int wi = blockIdx.x; wi < nwork; wi += gridDim.x)
         compress_row<T, ALIGNED, STATS>(a, a.use_redo_list ? a.redo_rows[wi] : wi, k_eff, smem64, smem64 + CAND_CAP, sh);
@@ -563,7 +556,9 @@ __global__ void __launch_bounds__(THREADS, 2) compress_kernel(CompressArgs a) {
 // sums of the queued rows (four warps per chunk, two chunks per CTA at a time, the whole grid sharing
 // the work) and, by the CTA that completes a row's last chunk, the cut of that row -- the sorted
 // candidates are read back from q_idx, the exact normaliser is the sum of the row's chunk sums.
-// Nothing waits (fence, then ticket); with an empty queue every CTA returns at once.
+// Nothing waits (fence, then ticket); with an empty queue every CTA returns at once.  A queue that was not empty
+// is empty again when the kernel ends, so that a call relies on no other call of the host's order: a captured
+// call runs once, often or never, between whichever others.
 template <typename T>
 __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs a, PreciseArgs p) {
     __shared__ double table[EXP_STEPS];
@@ -623,6 +618,8 @@ __global__ void __launch_bounds__(THREADS) compress_precise_kernel(CompressArgs 
         }
         __syncthreads();
     }
+    // (every thread of this CTA has read the count, before the first barrier; the last CTA's turn wraps to zero)
+    if (tid == 0 && atomicInc(a.queue_readers, gridDim.x - 1) == gridDim.x - 1) *a.queue_count = 0;
 }
 
 }  // namespace picospec

@@ -681,11 +681,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
     if (tid < WARPS) cta.wcnt[tid] = 0;
     for (int i = tid; i < 2 * CS_HIST_WORDS; i += STREAM_THREADS) hists[i] = 0u;
     grid_dependency_sync();
-    if (tid == 0 && blockIdx.x == 0) {
-        // its own counters, so that a captured call can be replayed alone, and those of a next call by the direct kernel
-        *a.queue_count = *a.queue_count_next = 0;
-        *a.redo_count = *a.redo_count_next = 0;
-    }
+    if (tid == 0 && blockIdx.x == 0) *a.redo_count = 0;
     __syncthreads();
 
     if (warp == WARPS) {

@@ -27,7 +27,6 @@ struct picospec_ctx {
     int num_sms;
     unsigned long long wait_limit_ns;   // first limit of the staged kernels' waits
     int last_cuda_error;
-    unsigned long long compress_calls;
     int filter_ctas[2][2][2][2];        // resident CTAs per SM of the filter kernel's variants (0: not asked yet)
     // optional per-kernel timing (picospec_profile_*): rings of event pairs per kernel kind
     int prof_level;
@@ -41,7 +40,7 @@ struct picospec_ctx {
     float* row_max;
     int* queue;
     unsigned long long* need_rows;
-    int* counters;  // [0] verify queue, [1],[2] compress queue (alternating), [3],[4] compress redo list (alternating)
+    int* counters;  // [0] verify queue, [1] compress queue, [2] its readers, [3] compress redo list, [5] rowq
     int* redo_rows; // rows the staged compress kernel hands to the direct kernel
     unsigned long long* surv_keys;  // staged compress: survivors per row
     CsRowMeta* surv_meta;
@@ -257,12 +256,6 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
             else launch_compress_direct<T, false>(r, grid, stats, s);
         }
     } else {
-        // a captured call may be replayed alone, with no call between that clears its queue
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusActive) {
-            const cudaError_t em = cudaMemsetAsync(a.queue_count, 0, sizeof(int), s);
-            if (em != cudaSuccess) return em;
-        }
         ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_STREAM, 1, s);
         if (aligned) launch_compress_direct<T, true>(a, grid, stats, s);
         else launch_compress_direct<T, false>(a, grid, stats, s);
@@ -340,21 +333,18 @@ cudaError_t launch_verify(picospec_ctx* ctx, const VerifyArgs& a, cudaStream_t s
     return cudaGetLastError();
 }
 
-// workspace pointers and the alternating counters of one compress-type call
+// workspace pointers of a compress-type call
 void fill_compress_workspace(picospec_ctx* ctx, CompressArgs& a) {
     a.row_max = ctx->row_max; a.dsum = ctx->dsum; a.queue = ctx->queue;
-    const int cur = 1 + (int)(ctx->compress_calls & 1ull);
-    a.queue_count = ctx->counters + cur;
-    a.queue_count_next = ctx->counters + (3 - cur);
+    a.queue_count = ctx->counters + 1;
+    a.queue_readers = reinterpret_cast<unsigned*>(ctx->counters + 2);
     a.tickets = ctx->tickets;
     a.redo_rows = ctx->redo_rows;
-    a.redo_count = ctx->counters + 2 + cur;           // [3] / [4]
-    a.redo_count_next = ctx->counters + 2 + (3 - cur);
+    a.redo_count = ctx->counters + 3;
     a.use_redo_list = 0;
     a.redo_total = ctx->slow_rows + 1;
     a.surv_keys = ctx->surv_keys;
     a.surv_meta = ctx->surv_meta;
-    ctx->compress_calls++;
     a.status = ctx->status; a.slow_rows = ctx->slow_rows;
 }
 

@@ -184,3 +184,56 @@ def test_a_captured_call_is_replayed_alone(rows, V):
         del graph
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("V", [4096, 16384])
+@pytest.mark.parametrize("order", ["eager capture eager", "eager replay eager", "replay replay eager replay"])
+def test_captured_calls_between_others(order, V):
+    # every row takes the double-precision cut, so each call leaves a full queue; the last call has fewer rows and
+    # another vocabulary, for which a row number or a ticket left behind would lie outside its logits
+    import paper_2603_19133_b200 as ps
+    rows, k, keep, i32 = 24, 64, 40, torch.int32
+
+    def inputs(n, v):
+        out = (torch.empty((n, 1, k), dtype=i32, device="cuda"), torch.empty((n, 1, k), device="cuda"),
+               torch.empty((n, 1), dtype=i32, device="cuda"), torch.empty((n, 1), dtype=i32, device="cuda"))
+        return torch.zeros((n, 1, v), dtype=torch.bfloat16, device="cuda"), torch.ones((n,), device="cuda"), torch.rand((n, 1), device="cuda"), out
+
+    def call(x, T, u, out):
+        ctx.compress(x, T, 0, keep / x.shape[2], k, u, out=out)
+
+    def check(x, T, u, out):
+        assert (out[2] == keep).all() and (out[0][:, 0, :keep] == torch.arange(keep, dtype=i32, device="cuda")).all()
+        for t in out[:3]:
+            t.fill_(-7)
+
+    ctx = ps.Context(rows, 1, V, k)
+    try:
+        full, small = inputs(rows, V), inputs(5, V * 5 // 8)      # (keep / V is exact in both)
+        call(*full)
+        check(*full)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            call(*full)
+        ctx.counters(clear=True)
+        done = 0
+        for step in order.split()[1:]:
+            if step == "capture":
+                continue
+            if step == "replay":
+                graph.replay()
+                done += rows
+                assert ctx.counters()[0] == done
+                check(*full)
+            else:
+                call(*small)
+                done += 5
+                assert ctx.counters()[0] == done
+                check(*small)
+        call(*small)
+        assert ctx.counters()[0] == done + 5
+        check(*small)
+        assert ctx.status()[0] == 0
+        del graph
+    finally:
+        ctx.close()
