@@ -43,8 +43,11 @@ namespace picospec {
 // bound by instruction issue, so resident warps count for more than tiles in flight: two stages
 // measure the same as three, three CTAs 15 % faster than two).  Rows with k <= 512 need few live
 // candidates: a small candidate buffer; larger k takes the big buffer.  32-bit rows have 32 KB tiles:
-// two CTAs per SM in both shapes.
-constexpr int CS_CAP_SMALL = 2048, CS_CAP_LARGE = 3072;    // candidate keys held in shared memory
+// two CTAs per SM in both shapes.  With spread tiles a region that is full empties itself into the scratch area, and
+// the big buffer gives a quarter of its keys to a second histogram.  Without (k > 512: rows of at most two tiles) it
+// keeps them, a row whose regions overflow being lost to the direct kernel: with 3072 keys all of 60 rows of 16384 entries
+// (k = 1024, a third of them below index 1024) went there, with 4096 none.
+constexpr int CS_CAP_SMALL = 2048, CS_CAP_LARGE = 4096, CS_CAP_LARGE_SPREAD = 3072;    // candidate keys held in shared memory
 constexpr int CS_K_SMALL = 512;                            // largest k served by the small shape
 constexpr int CS_BINS = 4096;        // histogram bins above the first tile's bound; the last one is open-ended
 constexpr int CS_DEAD = 117 << 7;    // 16-bit magnitude codes below 2^-10: one bin on each side of zero
@@ -96,16 +99,21 @@ struct CsCta {
     int2 arg[WARPS];    // per warp: what crowded_chunk takes besides its arguments (chunk's offset, its first index)
 };
 // bf16: 2 stages x 16 KB, 66 KB SMALL, 74 KB LARGE (3 CTAs / SM).  fp32: 2 stages x 32 KB, 98 / 106 KB (2 CTAs / SM).
-template <typename T, bool SMALL> struct CsGeom {
-    static constexpr int CAP = SMALL ? CS_CAP_SMALL : CS_CAP_LARGE;
+template <typename T, bool SMALL, bool SPREAD> struct CsGeom {
+    static constexpr int CAP = SMALL ? CS_CAP_SMALL : SPREAD ? CS_CAP_LARGE_SPREAD : CS_CAP_LARGE;
     static constexpr int REGION = CAP / WARPS;             // each worker warp appends to its own region
+    static constexpr int TIES = SMALL ? 128 : 256;         // of one code in a chunk (crowded_chunk): hopeless
+    static constexpr int HISTS = SMALL || SPREAD ? 2 : 1;  // copies of the histogram
     static constexpr int STAGES = 2;
     static constexpr int CTAS = sizeof(T) == 2 ? 3 : 2;
     static constexpr int TILE_BYTES = TILE_CHUNKS * CHUNK * (int)sizeof(T);
     static constexpr int STAGE_BYTES = STAGES * TILE_BYTES;
     static constexpr int HIST_OFF = STAGE_BYTES + CAP * 8;
-    static constexpr int SHARED_OFF = HIST_OFF + 2 * CS_HIST_WORDS * 4;    // CsShared[2], CsCta
+    static constexpr int SHARED_OFF = HIST_OFF + HISTS * CS_HIST_WORDS * 4;    // CsShared[2], CsCta
     static constexpr int SMEM_BYTES = SHARED_OFF + 2 * (int)sizeof(CsShared) + (int)sizeof(CsCta);
+    __device__ static __forceinline__ unsigned* hist(unsigned char* dyn, int copy) {
+        return reinterpret_cast<unsigned*>(dyn + HIST_OFF) + (HISTS == 2 ? copy * CS_HIST_WORDS : 0);
+    }
 };
 
 __device__ __forceinline__ void cs_reset(CsShared& cs) {
@@ -325,7 +333,7 @@ __device__ __forceinline__ int compact_region(u64* region, int n, unsigned thr_k
 template <typename Geom> __device__ __noinline__ void refresh_bound(int copy, int rank, int k) {
     extern __shared__ __align__(1024) unsigned char dyn[];
     CsShared& cs = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF)[copy];
-    refresh_threshold(reinterpret_cast<const unsigned*>(dyn + Geom::HIST_OFF) + copy * CS_HIST_WORDS, cs, rank, k, threadIdx.x & 31);
+    refresh_threshold(Geom::hist(dyn, copy), cs, rank, k, threadIdx.x & 31);
 }
 // First tile of a piece: the bound is the NTH smallest of the warps' own (one warp, every warp with the same
 // result; out of line).  Returns the largest orderable logit of the tile (STATS).
@@ -397,7 +405,7 @@ __device__ __noinline__ int crowded_chunk(unsigned mask, int n, int copy) {
     CsCta* cta = reinterpret_cast<CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
     const unsigned char* chunk = dyn + cta->arg[warp].x;
     const int vchunk = cta->arg[warp].y;
-    unsigned* hist = reinterpret_cast<unsigned*>(dyn + Geom::HIST_OFF) + copy * CS_HIST_WORDS;
+    unsigned* hist = Geom::hist(dyn, copy);
     u64* region = reinterpret_cast<u64*>(dyn + Geom::STAGE_BYTES) + warp * REGION;
     u64* to = region;
     int* wcnt = &cta->wcnt[warp];
@@ -413,14 +421,14 @@ __device__ __noinline__ int crowded_chunk(unsigned mask, int n, int copy) {
         __syncwarp();
     } else {
         // Values that share the bound's own 16-bit code cannot be told apart by any bound: if, behind the first
-        // tile, they alone fill half a region, or if another warp has given up, so does this one.
+        // tile, a chunk holds TIES of them, or if another warp has given up, so does this one.
         const unsigned code = *(volatile unsigned*)&cs->thr_key >> 16;
         int same = 0;
         for (unsigned m = mask; m; m &= m - 1u)
             same += staged_key<T>(chunk, bit_offset(__ffs(m) - 1, lane, (const T*)nullptr)) >> 16 == code ? 1 : 0;
         __syncwarp();
         same = __reduce_add_sync(0xffffffffu, same);
-        if ((same > REGION / 2 && __any_sync(0xffffffffu, *(volatile int*)&cs->seen > WARPS)) ||
+        if ((same > Geom::TIES && __any_sync(0xffffffffu, *(volatile int*)&cs->seen > WARPS)) ||
             __any_sync(0xffffffffu, *(volatile int*)&cs->overflow))
             return -1;
         if (lane == 0) *(volatile unsigned*)&cs->certain = 1u;
@@ -644,22 +652,22 @@ __device__ __forceinline__ unsigned first_tile_key_lanes(float lane_max, int nee
 
 // SPREAD: bound_spreads for the call's rows
 template <typename T, bool STATS, bool SMALL, bool SPREAD>
-__global__ void __launch_bounds__(STREAM_THREADS, CsGeom<T, SMALL>::CTAS)
+__global__ void __launch_bounds__(STREAM_THREADS, CsGeom<T, SMALL, SPREAD>::CTAS)
 compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned long long wait_limit_ns) {
     extern __shared__ __align__(1024) unsigned char dyn[];
-    typedef CsGeom<T, SMALL> Geom;
+    typedef CsGeom<T, SMALL, SPREAD> Geom;
     constexpr int STAGES = Geom::STAGES;
     constexpr int TILE_BYTES = Geom::TILE_BYTES;
     constexpr int CS_CAND_CAP = Geom::CAP, CS_REGION = Geom::REGION;
     unsigned char* stage_mem = dyn;
     u64* cand = reinterpret_cast<u64*>(dyn + Geom::STAGE_BYTES);
-    unsigned* hists = reinterpret_cast<unsigned*>(cand + CS_CAND_CAP);         // bins, then super-bins; two copies
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES];
     // Two copies of the per-piece state and of the histogram, used in turn, so that a piece has one barrier, that
     // of its first tile: behind it every warp is done with the piece before, whose record is written and whose copies
     // are cleared there.  (With three barriers a piece, a last exact bound and one histogram the kernel took 70.8 us for
     // 4096 rows of 32000 entries at k = 8, 29.5 for 256 of 128256 at k = 10, 11.4 for 40 of 128256 at k = 64; now 67.8,
-    // 27.6 and 10.6, and the finish behind it 6.6 instead of 10.3 at k = 8.  Long rows: no difference.)
+    // 27.6 and 10.6, and the finish behind it 6.6 instead of 10.3 at k = 8.  Long rows: no difference.)  A shape with one
+    // histogram has a second barrier there, behind its clearing.
     CsShared* css = reinterpret_cast<CsShared*>(dyn + Geom::SHARED_OFF);
     CsCta& cta = *reinterpret_cast<CsCta*>(dyn + Geom::SHARED_OFF + 2 * sizeof(CsShared));
 
@@ -679,7 +687,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
         cta.surv_keys = a.surv_keys;
     }
     if (tid < WARPS) cta.wcnt[tid] = 0;
-    for (int i = tid; i < 2 * CS_HIST_WORDS; i += STREAM_THREADS) hists[i] = 0u;
+    for (int i = tid; i < Geom::HISTS * CS_HIST_WORDS; i += STREAM_THREADS) Geom::hist(dyn, 0)[i] = 0u;
     grid_dependency_sync();
     if (tid == 0 && blockIdx.x == 0) *a.redo_count = 0;
     __syncthreads();
@@ -749,7 +757,7 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
     for (int k = 0; plan_piece(plan, blockIdx.x, k, pc); ++k) {
         if (pc.tile0 >= pc.tile1) continue;
         CsShared& cs = css[parity];
-        unsigned* hist = hists + parity * CS_HIST_WORDS;
+        unsigned* hist = Geom::hist(dyn, parity);
         parity ^= 1;
         const int row = pc.row;
         const float Tb = a.temperature[row / a.G];
@@ -814,7 +822,8 @@ compress_filter_kernel(CompressArgs a, FilterPlan plan, FilterBound fb, unsigned
                     cs.flags = !in_range ? CSF_RANGE : !valid ? CSF_TEMPERATURE : 0;
                 }
                 if (i)
-                    for (int x = tid; x < CS_HIST_WORDS; x += THREADS) hists[parity * CS_HIST_WORDS + x] = 0u;
+                    for (int x = tid; x < CS_HIST_WORDS; x += THREADS) Geom::hist(dyn, parity)[x] = 0u;
+                if (Geom::HISTS == 1) workers_sync();
                 const unsigned first_top = first_bound<Geom, SPREAD ? 3 : 1>(parity ^ 1, pc.area);
                 if (STATS) ref_off = __fmul_rn(from_orderable(first_top), c32);
                 if (valid && __any_sync(0xffffffffu, *(volatile unsigned*)&cs.thr_key < 0x00800000u)) {

@@ -108,7 +108,7 @@ template <typename T> void set_compress_attrs() {
 }
 
 template <typename T, bool SMALL, bool SPREAD> cudaError_t set_filter_attrs() {
-    constexpr int bytes = CsGeom<T, SMALL>::SMEM_BYTES;
+    constexpr int bytes = CsGeom<T, SMALL, SPREAD>::SMEM_BYTES;
     cudaError_t e = cudaFuncSetAttribute(compress_filter_kernel<T, true, SMALL, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(compress_filter_kernel<T, false, SMALL, SPREAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -213,7 +213,8 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         void (*kern)(CompressArgs, FilterPlan, FilterBound, unsigned long long) =
             small ? (stats ? filter_kernel<T, true, true>(fb) : filter_kernel<T, false, true>(fb))
                   : (stats ? filter_kernel<T, true, false>(fb) : filter_kernel<T, false, false>(fb));
-        const int smem = small ? CsGeom<T, true>::SMEM_BYTES : CsGeom<T, false>::SMEM_BYTES;
+        const int smem = fb.spread ? (small ? CsGeom<T, true, true>::SMEM_BYTES : CsGeom<T, false, true>::SMEM_BYTES)
+                                   : (small ? CsGeom<T, true, false>::SMEM_BYTES : CsGeom<T, false, false>::SMEM_BYTES);
         // resident CTAs per SM for this kernel's registers and shared memory (asking costs a microsecond: once)
         int& per_sm = ctx->filter_ctas[sizeof(T) == 2][small][stats][fb.spread];
         if (per_sm == 0) {

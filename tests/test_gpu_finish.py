@@ -237,3 +237,17 @@ def test_captured_calls_between_others(order, V):
         del graph
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V,k,share", [(16384, 1024, 1 / 3), (12000, 800, 1 / 2), (12000, 1024, 1 / 4)])
+def test_crowded_place_in_rows_of_two_tiles(V, k, share, dtype):
+    # more than 512 wanted of a row that has no more than two tiles, a share of them among the ids below 1024: a warp's
+    # region holds its chunk's part of them, so that no row is read again
+    rows, m = 60, int(k * share)
+    g = torch.Generator(device="cuda").manual_seed(V + k)
+    x = 1.5 * torch.randn((rows, V), generator=g, device="cuda") - 1.1 * torch.log(torch.floor(torch.rand((rows, V), generator=g, device="cuda") * V) + 1.0)
+    at = torch.rand((rows, 1024), generator=g, device="cuda").argsort(dim=1)[:, :m]
+    kth = torch.topk(x, k - m + 1, dim=1).values[:, -1:]
+    x.scatter_(1, at, kth + 0.02 + 0.9 * (x.amax(dim=1, keepdim=True) - kth) * torch.rand((rows, m), generator=g, device="cuda"))
+    _check_compress(x[:, None].to(torch.bfloat16 if dtype == "bf16" else torch.float32), k, 1.0, 0.9, g)
