@@ -936,8 +936,8 @@ struct CsFinishShared {
 // bin of the k-th into its bin's stretch, then place each by its rank among the keys of its own stretch
 // (all pairs: a few keys).  Bound by latency for few rows (meta, survivors, six
 // short phases: about 9 K cycles) and by issue for many.  It replaces a trim and a bitonic network over
-// the survivors, which was 32 of 51 K cycles of a row with k = 1024: 172 -> 72 us for 4096 rows with
-// k = 1024, 22 -> 15.5 us for 1536 rows with k = 256, 41 -> 9.1 us for 4096 rows with k = 8 (a warp
+// the survivors, which was 32 of 51 K cycles of a row with k = 1024: 172 -> 78 us for 4096 rows with
+// k = 1024, 22 -> 15.5 us for 1536 rows with k = 256, 41 -> 6.6 us for 4096 rows with k = 8 (a warp
 // each), 16.4 -> 7.0 us for 40 rows in eight pieces with k = 64 (the pieces' records are read by one
 // lane each instead of one after the other).
 // With one bin per code, bf16 logits around 30 / 100 (k = 1024) took 95 / 267 us for 1536 rows; now 37 / 37, and

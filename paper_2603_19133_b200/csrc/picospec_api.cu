@@ -238,9 +238,9 @@ cudaError_t launch_compress(picospec_ctx* ctx, const CompressArgs& a, bool align
         const bool few = rows <= 2 * ctx->num_sms;      // (compress_finish_few_kernel)
         {
             ProfScope ps(ctx, PICOSPEC_PROF_COMPRESS_FINISH, 2, s);
-            // A warp per row while the row that has most survivors has few of them: a row dealt in 8 pieces
+            // A warp per row while k is at most a warp's (of a whole row; of a row in pieces the sum of their ranks): a row dealt in 8 pieces
             // at k = 64 (560 survivors) took 15.9 us of a call by warps, 7.0 by CTAs; 4096 whole rows at
-            // k = 8 take 9.1 us by warps and took 41 with a CTA and a sort network each.
+            // k = 8 take 6.6 us by warps and took 41 with a CTA and a sort network each.
             const int survivors = plan.rem > 0 ? plan.split * bound_rank(k_eff, 1.0f / (float)plan.split) : k_eff;
             if (few) launch_compress_finish_few<T>(a, plan, aligned, stats, s);
             else if (survivors <= FinishGeom<32>::KCAP) launch_compress_finish<T, 32>(a, plan, stats, s);

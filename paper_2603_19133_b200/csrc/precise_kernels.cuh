@@ -87,8 +87,8 @@ template <typename T> __device__ __forceinline__ void precise_store(const Precis
 // A CTA takes two chunks at a time, four warps per chunk (a quarter of the chunk each, so that a handful of rows
 // still spreads over the whole GPU); the four partial sums of a chunk are added in a fixed order.  Where a CTA
 // takes several, the next one's logits are on the way while the exponentials of the one at hand are taken, so that
-// three CTAs per SM do what took six (40 rows of 128256 entries: 17 us either way, bound by the chain of one
-// item).  Few rows are bound by the launch: see precise_grid.
+// three CTAs per SM do what took six (40 rows of 128256 entries: 17 us either way, 12 since the exponential goes by table,
+// of which its operations are 3.3 at the nominal rate).  Few rows are bound by the launch: see precise_grid.
 constexpr int PRECISE_CTAS = 3;     // per SM
 template <typename T>
 __global__ void __launch_bounds__(THREADS, PRECISE_CTAS) precise_chunk_sums_kernel(PreciseArgs a) {
